@@ -8,13 +8,11 @@
 // Sec. III-D one value factorisation for all heads), here once per cache row
 // for all of a sequence's queries, as two dense GEMM chains:
 //
-//  1. recon_kernel: for every 128-row tile of every sequence and every KV
-//     head h, K^_h = RoPE(C_g B_g[:, slot(h)]) at the rows' positions and
-//     V^_h = C_v B_v[:, h d : (h+1) d] (tcgen05.mma M = 128 rows, N = 128,
-//     K = r_g or r_v in TMA-staged pieces, fp32 in TMEM), written as bf16 to
-//     the workspace [n_rows][Hkv][d] (keys) and [n_rows][Hkv][d] (values);
-//     the values, where the cache rows are mostly in use, instead as one GEMM
-//     V^ = C_v B_v over all rows on the pair kernel of append_tc.cu;
+//  1. recon_kernel: for every KV head h, K^_h = RoPE(C_g B_g[:, slot(h)]) at the
+//     rows' positions and V^_h = C_v B_v[:, h d : (h+1) d] of every sequence's
+//     rows (tcgen05 pair MMAs), written as bf16 to the workspace [n_rows][Hkv][d]
+//     (keys) and [n_rows][Hkv][d] (values); the new tokens' queries, rotated
+//     and scaled, go to `out`;
 //  2. attn_kernel: causal flash attention over them, one CTA per 128 query
 //     rows of one KV head (the qpg query heads of a KV head packed into the
 //     rows: row r = query index r / qpg, head r % qpg), S = Q^ K^T and
@@ -33,200 +31,435 @@
 
 namespace dck {
 
-// C[M x N] = A[M x K] B[K x N], bf16 row-major, fp32 accumulation, on the
-// persistent CTA pairs of the long latent append (append_tc.cu).
-cudaError_t launch_gemm_pair(const void* A, int64_t M, int K, const void* Bm, int N, void* C, int* err,
-                             cudaStream_t s);
-
 namespace {
 
 using namespace sm100;
 using namespace tc;
 
 constexpr int kPD = 128;               // head dim of the tensor-core prefill
-constexpr int kRThreads = 192;         // recon: warp 0 TMA, warp 1 MMA/TMEM, warps 2-5 epilogue
-constexpr int kRStages = 4;
-constexpr int kRASlot = 16384;         // latent piece [128 rows][<= 64] bf16
-constexpr int kRBSlot = 16384;         // factor piece [<= 64 ranks][128 cols] as two 64-column atoms
 constexpr int kMaxGroupsP = 16;
-constexpr float kTwoPiP = 6.28318530717958647692f;
-constexpr float kInvTwoPiP = 0.15915494309189533577f;
+
+// ---------------------------------------------------------------------------
+// RoPE angles in turns
+// ---------------------------------------------------------------------------
+
+// Frequency w_i / (2 pi) as a 64-bit binary fraction: position t turns pair i
+// by the fraction t * f (mod 2^64), exactly, so an angle needs two integer
+// multiplies and no fp64, and its reduction mod 2 pi is the wrap-around.
+struct RopeFreqs {
+  uint2 f[kPD / 2];  // {low, high} words
+};
+
+// sin and cos of 2 pi u / 2^32.  The nearest quarter turn is taken off exactly
+// in integers; the remainder, within +-pi/4, goes through the Taylor series of
+// sine (to x^9) and cosine (to x^10), whose truncation errors there (1.8e-9
+// and 1.2e-10) are below fp32 rounding.
+__device__ __forceinline__ void turn_sincos(uint32_t u, float& sn, float& cs) {
+  const uint32_t q = (u + 0x20000000u) >> 30;
+  const float x = (float)(int32_t)(u - (q << 30)) * 1.4629180792671596e-9f;  // 2 pi / 2^32
+  const float x2 = x * x;
+  float s = fmaf(x2, 2.7557319e-6f, -1.9841270e-4f);
+  s = fmaf(x2, s, 8.3333333e-3f);
+  s = fmaf(x2, s, -1.6666667e-1f);
+  s = fmaf(x * x2, s, x);
+  float c = fmaf(x2, -2.7557319e-7f, 2.4801587e-5f);
+  c = fmaf(x2, c, -1.3888889e-3f);
+  c = fmaf(x2, c, 4.1666667e-2f);
+  c = fmaf(x2, c, -0.5f);
+  c = fmaf(x2, c, 1.f);
+  const float a = (q & 1) ? c : s, b = (q & 1) ? s : c;
+  sn = __uint_as_float(__float_as_uint(a) ^ ((q & 2) << 30));
+  cs = __uint_as_float(__float_as_uint(b) ^ (((q + 1) & 2) << 30));
+}
+__device__ __forceinline__ void rope_sincos(uint2 f, uint32_t pos, float& sn, float& cs) {
+  turn_sincos(__umulhi(pos, f.x) + pos * f.y, sn, cs);
+}
 
 // ---------------------------------------------------------------------------
 // 1. reconstruction
+//
+// Keys and values of every sequence as dense GEMMs over its latent rows on
+// persistent CTA pairs (tcgen05 pair MMAs, M = 256 rows): a tile is 256 rows of
+// one sequence x the columns of one or two heads (w = 256 or 128), K = the
+// group's rank or r_v in 64-wide stages, each CTA holding its 128 latent rows
+// and half of the factor columns; two 256-column TMEM accumulators, so that the
+// epilogue of one tile overlaps the next tile's MMAs.  Key tiles are rotated in
+// the epilogue (a thread holds one row, both halves of every frequency pair).
+// Pair p takes tiles p, p + P, ... of the list (values of every row tile, then
+// keys: the costliest tiles first).  Four more warps of each CTA rotate and
+// scale the queries into `out`, from where the attention kernel loads them by
+// TMA before it overwrites them with the results: the tensor-bound GEMM hides
+// that pass over q.
+//
+// One CTA per (row tile, head), as before, read a latent tile once per head and
+// formed 64 sines and cosines per row and head (and the attention kernel 64 per
+// query row).  Whole prefill calls, before and after: 32-head MHA prompt 2 x 4096
+// 1193 -> 738 us, GQA prompt 8192 1228 -> 1041 us, four 300-512 token chunks in a
+// pooled GQA cache 436 -> 268 us, eight MHA prompts of 44-214 tokens 139 -> 75 us.
 // ---------------------------------------------------------------------------
 
+constexpr int kRThreads = 320;   // warp 0 TMA, warp 1 MMA/TMEM, warps 2-5 epilogue, warps 6-9 queries
+constexpr int kRStages = 6;
+constexpr int kRBK = 64;
+constexpr int kRABytes = kTile * kRBK * 2;   // 16 KB: this CTA's 128 latent rows x 64 of K
+constexpr int kRBBytes = kRBK * 128 * 2;     // 16 KB: up to 128 factor columns x 64 of K (64-column boxes)
+constexpr int kRStageBytes = kRABytes + kRBBytes;
+constexpr int kRRows = 2 * kTile;            // rows of a pair tile
+constexpr int kMaxColTiles = 160;            // key: <= 64 + 16, value: <= 64
+
 struct RMaps {
-  CUtensorMap kc64, kc32, kc16;  // key latents: box {w, 128 rows}, 128/64/32B swizzle
-  CUtensorMap vc64, vc32, vc16;  // value latents
-  CUtensorMap bv;                // B_v [r_v][Hkv d]: box {64 cols, 16 rows}, 128B swizzle
-  CUtensorMap bk[kMaxGroupsP];   // B_g [r_g][n_g d]: box {64 cols, 16 rows}, 128B swizzle
+  CUtensorMap ka[kMaxGroupsP];  // key latents of group g: [n_rows][r_g], box {64, 128 rows}, 128B swizzle
+  CUtensorMap kb[kMaxGroupsP];  // B_g [r_g][n_g d]: box {64 columns, 64 ranks}, 128B swizzle
+  CUtensorMap va, vb;           // value latents, B_v [r_v][Hkv d]
+};
+
+// Column tile of a row tile: factor columns [n0, n0 + w) of group g's B_g (g >= 0)
+// or of B_v (g = -1), reduction length k, output heads h0 (and h1 when w = 256).
+struct RCol {
+  int16_t g, n0, w, h0, h1;
+  int32_t k;
 };
 
 struct RArgs {
   const int64_t* seq_start;
   const int32_t* seq_len;
+  const int32_t* q_len;
   int64_t n_rows;
-  int B, Hkv, G, Rk, rv, max_len;
-  int grp_roff[kMaxGroupsP], grp_rank[kMaxGroupsP];
-  int head_group[128], head_slot[128];
-  double om[kPD / 2];
-  __nv_bfloat16* kw;  // [n_rows][Hkv][d]
-  __nv_bfloat16* vw;  // [n_rows][Hkv][d]
+  int B, Hq, Hkv, qmax, max_len;
+  int n_val, n_key;               // value and key column tiles of this launch (either may be 0)
+  RCol col[kMaxColTiles];         // value tiles, then key tiles
+  RopeFreqs rf;
+  float qscale;                   // log2(e) / sqrt(d)
+  const __nv_bfloat16* q;         // null: this launch does not rotate the queries
+  __nv_bfloat16* qr;              // rotated, scaled queries (the out buffer)
+  __nv_bfloat16* kw;              // [n_rows][Hkv][d]
+  __nv_bfloat16* vw;              // [n_rows][Hkv][d]
   int* err;
 };
 
-struct RSmem {
-  uint8_t a[kRStages][kRASlot];
-  uint8_t b[kRStages][kRBSlot];
-  float beta[kPD / 2], om32[kPD / 2];  // RoPE: (t0 w_i) mod 2 pi of the tile's first row, and w_i
-  uint64_t full[kRStages], empty[kRStages], acc;
-  uint32_t tmem_base;
-  int abort_flag;
-};
+// Cache rows of sequence b whose keys and values the attention kernel will read
+// (0 for a sequence without new tokens or one that kernel rejects).
+__device__ __forceinline__ int prefill_len(const int32_t* seq_len, const int64_t* seq_start, const int32_t* q_len,
+                                           int b, int64_t n_rows, int qmax, int max_len) {
+  const int L = valid_len(seq_len, seq_start, b, n_rows);
+  const int Q = q_len[b];
+  return Q <= 0 || Q > L || Q > qmax || L > max_len ? 0 : L;
+}
 
-__device__ __forceinline__ uint32_t swz_w(int w) { return w == 64 ? kSw128 : (w == 32 ? kSw64 : kSw32); }
-__device__ __forceinline__ int piece_w(int left) { return left >= 64 ? 64 : (left >= 32 ? 32 : 16); }
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float2 unpack2(uint32_t v) {
+  return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+}
 
-// grid (row tiles of the longest sequence, B, 2 Hkv): blockIdx.z < Hkv -> keys of head z, else values of head z - Hkv
 __global__ void __launch_bounds__(kRThreads, 1)
     recon_kernel(const __grid_constant__ RMaps maps, const __grid_constant__ RArgs ra) {
   extern __shared__ uint8_t smem_raw[];
-  RSmem& sm = *reinterpret_cast<RSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRStages * kRStageBytes);
+  uint64_t* empty = full + kRStages;
+  uint64_t* acc_full = empty + kRStages;
+  uint64_t* acc_empty = acc_full + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  int* scan = reinterpret_cast<int*>(smem);            // [2][kRThreads], before the first copy into the ring
+  int* rpre = reinterpret_cast<int*>(tmem_slot + 2);   // [B + 1] row tiles before sequence b
+  int* qpre = rpre + ra.B + 1;                         // [B + 1] queries before sequence b
+
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  volatile int* abort_flag = &sm.abort_flag;
-  const int b = blockIdx.y;
-  const bool is_v = (int)blockIdx.z >= ra.Hkv;
-  const int h = is_v ? blockIdx.z - ra.Hkv : blockIdx.z;
-  const int L = valid_len(ra.seq_len, ra.seq_start, b, ra.n_rows);
-  const int t0 = blockIdx.x * kTile;  // first position of the tile
-  // whole CTA, before any barrier or TMEM is set up; a sequence longer than the
-  // launch's bound is left to the attention kernel, which reports it
-  if (t0 >= L || L > ra.max_len) return;
-  const int64_t row0 = ra.seq_start[b] + t0;
-  const int g = ra.head_group[h];
-  const int K = is_v ? ra.rv : ra.grp_rank[g];
-  const int kcol0 = is_v ? 0 : ra.grp_roff[g];                 // first latent column
-  const int bcol0 = is_v ? h * kPD : ra.head_slot[h] * kPD;    // first factor column
-  const CUtensorMap* bmap = is_v ? &maps.bv : &maps.bk[g];
+  const int hr = (int)cluster_ctarank();  // this CTA's half of every pair tile
+  const bool leader = hr == 0;            // the even CTA issues the pair MMAs
+  const int P = gridDim.x / 2, pair = blockIdx.x >> 1;
   if (tid == 0) {
     for (int s = 0; s < kRStages; ++s) {
-      mbar_init(&sm.full[s], 1);
-      mbar_init(&sm.empty[s], 1);
+      mbar_init(&full[s], 1);   // even CTA: its producer's expect_tx; both CTAs' copies complete on it
+      mbar_init(&empty[s], 1);  // the pair MMAs' commit, in both CTAs
     }
-    mbar_init(&sm.acc, 1);
-    sm.abort_flag = 0;
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], 8);  // even CTA: the four epilogue warps of both CTAs
+    }
+    *abort_flag = 0;
     fence_mbar_init();
   }
-  // RoPE angle of row t0 + r and pair i: (t0 w_i reduced mod 2 pi in fp64, once
-  // per tile) + r w_i in fp32; the fp64 work stays off the per-row path
-  if (!is_v && tid < kPD / 2) {
-    const double ang = (double)t0 * ra.om[tid];
-    sm.beta[tid] = (float)(ang - 6.283185307179586 * floor(ang * 0.15915494309189535));
-    sm.om32[tid] = (float)ra.om[tid];
-  }
   if (warp == 1) {
-    tmem_alloc(&sm.tmem_base, 128);
-    tmem_relinquish();
+    tmem_alloc_pair(tmem_slot, 512);
+    tmem_relinquish_pair();
+  }
+  // exclusive prefixes of row tiles and of queries over the sequences
+  {
+    const int per = (ra.B + kRThreads - 1) / kRThreads, b0 = tid * per;
+    int nr = 0, nq = 0;
+    for (int b = b0; b < b0 + per && b < ra.B; ++b) {
+      const int L = prefill_len(ra.seq_len, ra.seq_start, ra.q_len, b, ra.n_rows, ra.qmax, ra.max_len);
+      nr += (L + kRRows - 1) / kRRows;
+      nq += L ? ra.q_len[b] : 0;
+    }
+    scan[tid] = nr;
+    scan[kRThreads + tid] = nq;
+    __syncthreads();
+    for (int off = 1; off < kRThreads; off <<= 1) {
+      const int v = tid >= off ? scan[tid - off] : 0, w = tid >= off ? scan[kRThreads + tid - off] : 0;
+      __syncthreads();
+      scan[tid] += v;
+      scan[kRThreads + tid] += w;
+      __syncthreads();
+    }
+    int r = scan[tid] - nr, q = scan[kRThreads + tid] - nq;
+    for (int b = b0; b < b0 + per && b < ra.B; ++b) {
+      const int L = prefill_len(ra.seq_len, ra.seq_start, ra.q_len, b, ra.n_rows, ra.qmax, ra.max_len);
+      rpre[b] = r;
+      qpre[b] = q;
+      r += (L + kRRows - 1) / kRRows;
+      q += L ? ra.q_len[b] : 0;
+    }
+    if (tid == 0) {
+      rpre[ra.B] = scan[kRThreads - 1];
+      qpre[ra.B] = scan[2 * kRThreads - 1];
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();  // both CTAs' barriers initialised and TMEM allocated (and the prefixes written)
   tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
+  const uint32_t tmem = *tmem_slot;
+  auto lead = [](const void* q) { return mapa_shared(smem_u32(q), 0); };
+  auto stop_peer = [&]() { st_cluster_u32(mapa_shared(smem_u32((const void*)abort_flag), (uint32_t)(hr ^ 1)), 1u); };
+
+  const int64_t n_rt = rpre[ra.B];
+  const int64_t n_vt = n_rt * ra.n_val, n_tiles = n_vt + n_rt * ra.n_key;
+  // tile t: column tile, row tile of the flattened list
+  auto tile_at = [&](int64_t t, int& rt) -> const RCol& {
+    const bool v = t < n_vt;
+    const int n = v ? ra.n_val : ra.n_key;
+    const int64_t u = v ? t : t - n_vt;
+    rt = (int)(u / n);
+    return ra.col[(v ? 0 : ra.n_val) + (int)(u - (int64_t)rt * n)];
+  };
+
   if (warp == 0) {
+    // ---- TMA producer (both CTAs): this CTA's latent rows and its half of the factor columns
     if (lane == 0) {
-      const uint64_t pol = policy_evict_first();
-      int n = 0;
-      for (int k0 = 0; k0 < K; ++n) {
-        const int w = piece_w(K - k0), s = n % kRStages;
-        if (n >= kRStages && !mbar_wait(&sm.empty[s], ((n / kRStages) - 1) & 1, abort_flag)) break;
-        // latent piece [128 rows][w] + factor rows [w][128 columns] (two 64-column atoms, 16-row boxes)
-        mbar_expect_tx(&sm.full[s], kTile * w * 2 + w * kPD * 2);
-        const CUtensorMap* am = is_v ? (w == 64 ? &maps.vc64 : (w == 32 ? &maps.vc32 : &maps.vc16))
-                                     : (w == 64 ? &maps.kc64 : (w == 32 ? &maps.kc32 : &maps.kc16));
-        tma_load_2d_hint(sm.a[s], am, &sm.full[s], kcol0 + k0, (int32_t)row0, pol);
-        for (int half = 0; half < 2; ++half)
-          for (int r = 0; r < w; r += 16)
-            tma_load_2d(sm.b[s] + half * (w * 128) + r * 128, bmap, &sm.full[s], bcol0 + 64 * half, k0 + r);
-        k0 += w;
+      const uint64_t pol = policy_evict_last();
+      int64_t it = 0;
+      bool ok = true;
+      for (int64_t t = pair; t < n_tiles && ok; t += P) {
+        int rt;
+        const RCol& c = tile_at(t, rt);
+        const int b = seq_of_tile(rpre, ra.B, rt);
+        const int32_t y = (int32_t)(ra.seq_start[b] + (int64_t)(rt - rpre[b]) * kRRows + hr * kTile);
+        const CUtensorMap* am = c.g >= 0 ? &maps.ka[c.g] : &maps.va;
+        const CUtensorMap* bm = c.g >= 0 ? &maps.kb[c.g] : &maps.vb;
+        const int half = c.w / 2, nbx = half / 64;
+        for (int k0 = 0; k0 < c.k; k0 += kRBK, ++it) {
+          const int s = (int)(it % kRStages);
+          if (it >= kRStages && !(ok = mbar_wait(&empty[s], (uint32_t)(((it / kRStages) - 1) & 1), abort_flag))) break;
+          uint8_t* as = smem + s * kRStageBytes;
+          uint8_t* bs = as + kRABytes;
+          if (leader) mbar_expect_tx(&full[s], 2u * (uint32_t)(kRABytes + nbx * kRBK * 64 * 2));
+          tma_load_2d_pair(as, am, lead(&full[s]), k0, y, pol);
+          for (int bx = 0; bx < nbx; ++bx)
+            tma_load_2d_pair(bs + bx * (kRBK * 64 * 2), bm, lead(&full[s]), c.n0 + hr * half + 64 * bx, k0, pol);
+        }
       }
+      if (!ok) stop_peer();
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(128, kPD, false, true);
-      int n = 0;
+    // ---- pair MMAs (even CTA, one thread) -------------------------------------
+    if (leader && lane == 0) {
+      int64_t it = 0;
       bool ok = true;
-      for (int k0 = 0; k0 < K && ok; ++n) {
-        const int w = piece_w(K - k0), s = n % kRStages;
-        if (!(ok = mbar_wait(&sm.full[s], (n / kRStages) & 1, abort_flag))) break;
+      int lt = 0;  // tiles of this pair so far
+      for (int64_t t = pair; t < n_tiles && ok; t += P, ++lt) {
+        int rt;
+        const RCol& c = tile_at(t, rt);
+        const int buf = lt & 1;
+        if (lt >= 2 && !(ok = mbar_wait(&acc_empty[buf], (uint32_t)(((lt >> 1) - 1) & 1), abort_flag))) break;
         tc_fence_after();
-        const uint32_t ab = smem_u32(sm.a[s]), bb = smem_u32(sm.b[s]);
-        for (int k = 0; k < w / 16; ++k)
-          umma_f16(tmem, sdesc(ab + k * 32, 16, 16 * w, swz_w(w)), sdesc(bb + k * 2048, 128 * w, 1024, kSw128), idesc,
-                   (k0 > 0 || k > 0) ? 1u : 0u);
-        umma_commit(&sm.empty[s]);
-        k0 += w;
+        const uint32_t idesc = idesc_bf16(kRRows, c.w, false, true);
+        const uint32_t d = tmem + buf * 256;
+        for (int k0 = 0; k0 < c.k; k0 += kRBK, ++it) {
+          const int s = (int)(it % kRStages);
+          if (!(ok = mbar_wait(&full[s], (uint32_t)((it / kRStages) & 1), abort_flag))) break;
+          tc_fence_after();
+          const uint32_t xa = smem_u32(smem + s * kRStageBytes);
+          const uint32_t ba = xa + kRABytes;
+          const int nk = min(kRBK, c.k - k0) / 16;
+          for (int k = 0; k < nk; ++k)
+            umma_f16_pair(d, sdesc(xa + k * 32, 16, 1024, kSw128), sdesc(ba + k * 2048, kRBK * 64 * 2, 1024, kSw128),
+                          idesc, (k0 > 0 || k > 0) ? 1u : 0u);
+          umma_commit_pair(&empty[s]);  // the stage's slots in both CTAs, once these MMAs are done
+        }
+        if (ok) umma_commit_pair(&acc_full[buf]);
       }
-      umma_commit(&sm.acc);
+      if (!ok) stop_peer();
     }
-  } else {
-    // epilogue: thread = row of the tile (TMEM lane); RoPE for keys; bf16 to the workspace
-    const int quad = warp & 3, r = quad * 32 + lane;
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(&sm.acc, 0, abort_flag));
-    const int pos = t0 + r;
-    if (ok) {
+    __syncwarp();
+  } else if (warp < 6) {
+    // ---- epilogue (warps 2-5, both CTAs): this CTA's 128 rows of each tile -----
+    const int quad = warp & 3;
+    const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+    int lt = 0;
+    bool ok = true;
+    for (int64_t t = pair; t < n_tiles && ok; t += P, ++lt) {
+      int rt;
+      const RCol& c = tile_at(t, rt);
+      const int b = seq_of_tile(rpre, ra.B, rt);
+      const int pos = (rt - rpre[b]) * kRRows + hr * kTile + quad * 32 + lane;
+      const bool in = pos < ra.seq_len[b];
+      const int64_t row = ra.seq_start[b] + pos;
+      const bool key = c.g >= 0;
+      const int nh = c.w / kPD, buf = lt & 1;
+      __nv_bfloat16* dst = (key ? ra.kw : ra.vw) + row * ra.Hkv * kPD;
+      ok = wwait(&acc_full[buf], (uint32_t)((lt >> 1) & 1), abort_flag);
+      if (!ok) break;
       tc_fence_after();
-      __nv_bfloat16* dst = (is_v ? ra.vw : ra.kw) + ((row0 + r) * ra.Hkv + h) * kPD;
-      // frequency pairs (i, i + 64): columns [cc, cc + 32) with [64 + cc, 64 + cc + 32)
+      const uint32_t acc = tmem + lane_base + buf * 256;
+      // frequency pairs (i, i + 64): columns [cc, cc + 16) with [64 + cc, 64 + cc + 16)
+#pragma unroll 1
+      for (int cc = 0; cc < kPD / 2; cc += 16) {
+        float sn[16], cs[16];
+        if (key) {
 #pragma unroll
-      for (int cc = 0; cc < kPD / 2; cc += 32) {
-        float x[32], y[32];
-        tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + cc, x);
-        tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + kPD / 2 + cc, y);
-        tmem_wait_ld();
-        if (!is_v) {
+          for (int i = 0; i < 16; ++i) rope_sincos(ra.rf.f[cc + i], (uint32_t)pos, sn[i], cs[i]);
+        }
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            // angle (t0 w_i mod 2 pi) + r w_i, reduced to [-pi, pi] in fp32
-            float ph = fmaf((float)r, sm.om32[cc + i], sm.beta[cc + i]);
-            ph = fmaf(-kTwoPiP, rintf(ph * kInvTwoPiP), ph);
-            float sn, cs;
-            sincosf(ph, &sn, &cs);
-            const float xr = x[i] * cs - y[i] * sn, yr = x[i] * sn + y[i] * cs;
-            x[i] = xr;
-            y[i] = yr;
+        for (int hh = 0; hh < 2; ++hh) {
+          if (hh == nh) break;
+          float x[16], y[16];
+          tmem_ld16(acc + hh * kPD + cc, x);
+          tmem_ld16(acc + hh * kPD + kPD / 2 + cc, y);
+          tmem_wait_ld();
+          if (key) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const float xr = x[i] * cs[i] - y[i] * sn[i];
+              y[i] = x[i] * sn[i] + y[i] * cs[i];
+              x[i] = xr;
+            }
+          }
+          if (in) {
+            __nv_bfloat16* o = dst + (hh ? c.h1 : c.h0) * kPD + cc;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              reinterpret_cast<uint4*>(o)[q] =
+                  make_uint4(pack2(x[8 * q], x[8 * q + 1]), pack2(x[8 * q + 2], x[8 * q + 3]),
+                             pack2(x[8 * q + 4], x[8 * q + 5]), pack2(x[8 * q + 6], x[8 * q + 7]));
+              reinterpret_cast<uint4*>(o + kPD / 2)[q] =
+                  make_uint4(pack2(y[8 * q], y[8 * q + 1]), pack2(y[8 * q + 2], y[8 * q + 3]),
+                             pack2(y[8 * q + 4], y[8 * q + 5]), pack2(y[8 * q + 6], y[8 * q + 7]));
+            }
           }
         }
-        if (pos < L)
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (leader) mbar_arrive(&acc_empty[buf]);
+        else mbar_arrive_cluster(lead(&acc_empty[buf]));
+      }
+    }
+    if (!ok && lane == 0) stop_peer();
+  } else if (ra.q) {
+    // ---- queries (warps 6-9): one warp per (sequence, new token); lane = (one of
+    // four heads at a time, frequency pairs [8 c, 8 c + 8)) ----------------------
+    const int nw = 4 * gridDim.x, nq = qpre[ra.B];
+    const int c8 = lane & 7, hs = lane >> 3;
+    for (int u = 4 * blockIdx.x + warp - 6; u < nq; u += nw) {
+      const int b = seq_of_tile(qpre, ra.B, u), qi = u - qpre[b];
+      const uint32_t pos = (uint32_t)(ra.seq_len[b] - ra.q_len[b] + qi);
+      float sn[8], cs[8];
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            uint4 ox, oy;
-            __nv_bfloat162* px = reinterpret_cast<__nv_bfloat162*>(&ox);
-            __nv_bfloat162* py = reinterpret_cast<__nv_bfloat162*>(&oy);
+      for (int i = 0; i < 8; ++i) {
+        rope_sincos(ra.rf.f[8 * c8 + i], pos, sn[i], cs[i]);
+        sn[i] *= ra.qscale;
+        cs[i] *= ra.qscale;
+      }
+      const int64_t off = ((int64_t)b * ra.qmax + qi) * ra.Hq * kPD + 8 * c8;
+#pragma unroll 4
+      for (int h = hs; h < ra.Hq; h += 4) {
+        const __nv_bfloat16* src = ra.q + off + h * kPD;
+        const uint4 xv = *reinterpret_cast<const uint4*>(src), yv = *reinterpret_cast<const uint4*>(src + kPD / 2);
+        const uint32_t xs[4] = {xv.x, xv.y, xv.z, xv.w}, ys[4] = {yv.x, yv.y, yv.z, yv.w};
+        uint32_t xo[4], yo[4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              px[t] = __floats2bfloat162_rn(x[8 * c + 2 * t], x[8 * c + 2 * t + 1]);
-              py[t] = __floats2bfloat162_rn(y[8 * c + 2 * t], y[8 * c + 2 * t + 1]);
-            }
-            *reinterpret_cast<uint4*>(dst + cc + 8 * c) = ox;
-            *reinterpret_cast<uint4*>(dst + kPD / 2 + cc + 8 * c) = oy;
-          }
+        for (int i = 0; i < 4; ++i) {
+          const float2 x = unpack2(xs[i]), y = unpack2(ys[i]);
+          xo[i] = pack2(x.x * cs[2 * i] - y.x * sn[2 * i], x.y * cs[2 * i + 1] - y.y * sn[2 * i + 1]);
+          yo[i] = pack2(x.x * sn[2 * i] + y.x * cs[2 * i], x.y * sn[2 * i + 1] + y.y * cs[2 * i + 1]);
+        }
+        __nv_bfloat16* dst = ra.qr + off + h * kPD;
+        *reinterpret_cast<uint4*>(dst) = make_uint4(xo[0], xo[1], xo[2], xo[3]);
+        *reinterpret_cast<uint4*>(dst + kPD / 2) = make_uint4(yo[0], yo[1], yo[2], yo[3]);
       }
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (sm.abort_flag) {
+  if (*abort_flag) {
+    // let copies and MMAs already in flight land before the memory is released
     const long long c0 = clock64();
     while (clock64() - c0 < 4000000ll) {
     }
     if (tid == 0) atomicOr(ra.err, kErrTimeout);
   }
-  __syncthreads();
+  cluster_sync();  // the peer no longer reads this CTA's operands or arrives on its barriers
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, 128);
+    tmem_dealloc_pair(tmem, 512);
   }
+}
+
+size_t recon_smem(int B) {
+  return 1024 + (size_t)kRStages * kRStageBytes + 256 + 2 * sizeof(int) * ((size_t)B + 1);
+}
+
+// CTA pairs of the reconstruction kernel that fit the device at once.
+int recon_pairs_of_device() {
+  static int cache[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (cache[dev]) return cache[dev];
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  const size_t smem = recon_smem(kMaxBatch);
+  if (cudaFuncSetAttribute(recon_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * (sms / 2));
+  cfg.blockDim = dim3(kRThreads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, recon_kernel, &cfg) != cudaSuccess || n <= 0) {
+    cudaGetLastError();
+    return 0;
+  }
+  cache[dev] = std::min(n, sms / 2);
+  return cache[dev];
+}
+
+cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * pairs);
+  cfg.blockDim = dim3(kRThreads);
+  cfg.dynamicSmemBytes = recon_smem(ra.B);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, recon_kernel, rm, ra);
 }
 
 // ---------------------------------------------------------------------------
@@ -236,22 +469,19 @@ __global__ void __launch_bounds__(kRThreads, 1)
 constexpr int kAThreadsP = 192;  // warp 0 TMA, warp 1 MMA/TMEM, warps 2-5 softmax (thread = query row)
 constexpr int kAtom = 128 * 128;  // one 64-column swizzle atom of 128 rows (16 KB)
 constexpr float kThr = 8.f;       // lazy reference max: probabilities stay <= 2^8
-constexpr float kLog2eP = 1.4426950408889634f;
 
 struct AMapsP {
   CUtensorMap kw, vw;  // [n_rows][Hkv d] bf16: box {64, 128 rows}, 128B swizzle
 };
 
 struct AArgsP {
-  const __nv_bfloat16* q;  // [B, Qmax, Hq, d] before RoPE
   const int32_t* q_len;    // [B]
   int qmax, max_len;
   const int64_t* seq_start;
   const int32_t* seq_len;
   int64_t n_rows;
   int B, Hq, Hkv, qpg;
-  double om[kPD / 2];
-  __nv_bfloat16* out;      // [B, Qmax, Hq, d]
+  __nv_bfloat16* out;      // [B, Qmax, Hq, d]: rotated queries in, results out
   int* err;
 };
 
@@ -261,7 +491,6 @@ struct ASmemP {
   uint8_t v[2][2][kAtom];   // V^ ring [stage][d atom][128 keys][128 B] (TMA)
   uint8_t p[2][kAtom];      // P [key atom][128 rows][128 B], K-major, 128B-swizzled
   uint64_t kv_full[2], kv_empty[2], s_full[2], s_free[2], p_ready, o_ready, q_ready;
-  float qbeta[kPD / 2], om32[kPD / 2];  // RoPE: (p0 w_i) mod 2 pi of the tile's first query, and w_i
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -313,13 +542,6 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
     mbar_init(&sm.q_ready, 4);
     sm.abort_flag = 0;
     fence_mbar_init();
-  }
-  // query RoPE angles: (p0 w_i reduced mod 2 pi in fp64, once per tile) + (row
-  // offset) w_i in fp32, p0 the position of the tile's first query
-  if (tid < kPD / 2) {
-    const double ang = (double)(L - Q + i0) * aa.om[tid];
-    sm.qbeta[tid] = (float)(ang - 6.283185307179586 * floor(ang * 0.15915494309189535));
-    sm.om32[tid] = (float)aa.om[tid];
   }
   if (warp == 1) {
     tmem_alloc(&sm.tmem_base, 512);
@@ -379,39 +601,12 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
     const int qi = i0 + r / qpg, j = h * qpg + r % qpg;
     const bool valid = qi < Q;
     const int pos = L - Q + (valid ? qi : 0);
-    // Q^ row: RoPE at pos, times log2(e)/sqrt(d) (scores in log2 units), bf16
+    // Q^ row (rotated and scaled by the reconstruction launch)
     {
-      const __nv_bfloat16* qr = aa.q + (((int64_t)b * aa.qmax + (valid ? qi : 0)) * aa.Hq + j) * kPD;
-      const float sc = kLog2eP * rsqrtf((float)kPD);
+      const uint4* qr = reinterpret_cast<const uint4*>(aa.out + (((int64_t)b * aa.qmax + (valid ? qi : 0)) * aa.Hq + j) * kPD);
 #pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {  // pairs [8 cc, 8 cc + 8): chunks cc (x-halves) and 8 + cc (y-halves)
-        const uint4 xr = *reinterpret_cast<const uint4*>(qr + 8 * cc);
-        const uint4 yr = *reinterpret_cast<const uint4*>(qr + kPD / 2 + 8 * cc);
-        const __nv_bfloat16* xh = reinterpret_cast<const __nv_bfloat16*>(&xr);
-        const __nv_bfloat16* yh = reinterpret_cast<const __nv_bfloat16*>(&yr);
-        uint4 ox, oy;
-        __nv_bfloat162* px = reinterpret_cast<__nv_bfloat162*>(&ox);
-        __nv_bfloat162* py = reinterpret_cast<__nv_bfloat162*>(&oy);
-#pragma unroll
-        for (int t = 0; t < 8; t += 2) {
-          float rx[2], ry[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int pi = 8 * cc + t + u;
-            float ph = fmaf((float)(valid ? qi - i0 : 0), sm.om32[pi], sm.qbeta[pi]);
-            ph = fmaf(-kTwoPiP, rintf(ph * kInvTwoPiP), ph);
-            float sn, cs;
-            sincosf(ph, &sn, &cs);
-            const float x = valid ? __bfloat162float(xh[t + u]) : 0.f, y = valid ? __bfloat162float(yh[t + u]) : 0.f;
-            rx[u] = (x * cs - y * sn) * sc;
-            ry[u] = (x * sn + y * cs) * sc;
-          }
-          px[t / 2] = __floats2bfloat162_rn(rx[0], rx[1]);
-          py[t / 2] = __floats2bfloat162_rn(ry[0], ry[1]);
-        }
-        *reinterpret_cast<uint4*>(&sm.q[0][0] + swz_chunk(r, cc)) = ox;
-        *reinterpret_cast<uint4*>(&sm.q[0][0] + swz_chunk(r, 8 + cc)) = oy;
-      }
+      for (int cc = 0; cc < 16; ++cc)
+        *reinterpret_cast<uint4*>(&sm.q[0][0] + swz_chunk(r, cc)) = valid ? qr[cc] : make_uint4(0, 0, 0, 0);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.q_ready);
@@ -541,7 +736,8 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
 
 }  // namespace
 
-static_assert(sizeof(RSmem) + 1024 <= 232448, "shared memory of the reconstruction kernel");
+static_assert(1024 + kRStages * kRStageBytes + 256 + 8 * (kMaxBatch + 1) <= 232448,
+              "shared memory of the reconstruction kernel");
 static_assert(sizeof(ASmemP) + 1024 <= 232448, "shared memory of the prefill attention kernel");
 
 // ---------------------------------------------------------------------------
@@ -571,20 +767,15 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   const uint64_t rows = (uint64_t)std::max<int64_t>(1, n_rows);
   RMaps rm;
   std::memset(&rm, 0, sizeof(rm));
-  bool ok = true;
-  const int widths[3] = {64, 32, 16};
-  const CUtensorMapSwizzle sws[3] = {CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_SWIZZLE_32B};
-  CUtensorMap* km[3] = {&rm.kc64, &rm.kc32, &rm.kc16};
-  CUtensorMap* vm[3] = {&rm.vc64, &rm.vc32, &rm.vc16};
-  for (int i = 0; i < 3 && ok; ++i) {
-    ok = make_tmap_2d_bf16(km[i], kc, lt.Rk, rows, (uint64_t)lt.Rk * 2, widths[i], kTile, sws[i]) &&
-         make_tmap_2d_bf16(vm[i], vc, lt.rv, rows, (uint64_t)lt.rv * 2, widths[i], kTile, sws[i]);
-  }
-  ok = ok && make_tmap_2d_bf16(&rm.bv, Bv, (uint64_t)lt.Hkv * kPD, lt.rv, (uint64_t)lt.Hkv * kPD * 2, 64, 16,
-                               CU_TENSOR_MAP_SWIZZLE_128B);
+  bool ok = make_tmap_2d_bf16(&rm.va, vc, lt.rv, rows, (uint64_t)lt.rv * 2, kRBK, kTile, CU_TENSOR_MAP_SWIZZLE_128B) &&
+            make_tmap_2d_bf16(&rm.vb, Bv, (uint64_t)lt.Hkv * kPD, lt.rv, (uint64_t)lt.Hkv * kPD * 2, 64, kRBK,
+                              CU_TENSOR_MAP_SWIZZLE_128B);
+  // a group's own columns and ranks only: a 64-wide stage past them loads zeros
   for (int g = 0; g < lt.G && ok; ++g)
-    ok = make_tmap_2d_bf16(&rm.bk[g], static_cast<const __nv_bfloat16*>(Bk) + lt.grp_boff[g],
-                           (uint64_t)lt.grp_nh[g] * kPD, lt.grp_rank[g], (uint64_t)lt.grp_nh[g] * kPD * 2, 64, 16,
+    ok = make_tmap_2d_bf16(&rm.ka[g], static_cast<const __nv_bfloat16*>(kc) + lt.grp_roff[g], lt.grp_rank[g], rows,
+                           (uint64_t)lt.Rk * 2, kRBK, kTile, CU_TENSOR_MAP_SWIZZLE_128B) &&
+         make_tmap_2d_bf16(&rm.kb[g], static_cast<const __nv_bfloat16*>(Bk) + lt.grp_boff[g],
+                           (uint64_t)lt.grp_nh[g] * kPD, lt.grp_rank[g], (uint64_t)lt.grp_nh[g] * kPD * 2, 64, kRBK,
                            CU_TENSOR_MAP_SWIZZLE_128B);
   AMapsP am;
   ok = ok && make_tmap_2d_bf16(&am.kw, kw, (uint64_t)lt.Hkv * kPD, rows, (uint64_t)lt.Hkv * kPD * 2, 64, kTile,
@@ -596,55 +787,60 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   std::memset(&ra, 0, sizeof(ra));
   ra.seq_start = seq_start;
   ra.seq_len = seq_len;
+  ra.q_len = q_len;
   ra.n_rows = n_rows;
-  ra.max_len = max_len;
   ra.B = B;
+  ra.Hq = lt.Hq;
   ra.Hkv = lt.Hkv;
-  ra.G = lt.G;
-  ra.Rk = lt.Rk;
-  ra.rv = lt.rv;
-  for (int g = 0; g < lt.G; ++g) {
-    ra.grp_roff[g] = lt.grp_roff[g];
-    ra.grp_rank[g] = lt.grp_rank[g];
+  ra.qmax = qmax;
+  ra.max_len = max_len;
+  RCol val[kMaxColTiles], key[kMaxColTiles];
+  int n_val = 0, n_key = 0;
+  for (int h = 0; h < lt.Hkv; h += 2) {
+    const int nh = std::min(2, lt.Hkv - h);
+    val[n_val++] = RCol{-1, (int16_t)(h * kPD), (int16_t)(nh * kPD), (int16_t)h, (int16_t)(h + 1), lt.rv};
   }
-  for (int hh = 0; hh < lt.Hkv; ++hh) {
-    ra.head_group[hh] = lt.head_group[hh];
-    ra.head_slot[hh] = lt.head_slot[hh];
+  int head_at[kMaxGroupsP][kMaxKvHeads];
+  for (int h = 0; h < lt.Hkv; ++h) head_at[lt.head_group[h]][lt.head_slot[h]] = h;
+  for (int g = 0; g < lt.G; ++g)
+    for (int sl = 0; sl < lt.grp_nh[g]; sl += 2) {
+      const int nh = std::min(2, lt.grp_nh[g] - sl);
+      key[n_key++] = RCol{(int16_t)g, (int16_t)(sl * kPD), (int16_t)(nh * kPD), (int16_t)head_at[g][sl],
+                          (int16_t)(nh == 2 ? head_at[g][sl + 1] : 0), lt.grp_rank[g]};
+    }
+  for (int i = 0; i < kPD / 2; ++i) {
+    const double turns = std::exp2(-2.0 * i / kPD * std::log2((double)theta)) * 0.15915494309189533577;
+    const double fr = turns - std::floor(turns);  // a whole number of turns per position is none
+    const uint64_t f = (uint64_t)std::ldexp(fr, 64);
+    ra.rf.f[i] = make_uint2((uint32_t)f, (uint32_t)(f >> 32));
   }
-  for (int i = 0; i < kPD / 2; ++i) ra.om[i] = std::exp2(-2.0 * i / kPD * std::log2((double)theta));
+  ra.qscale = 1.4426950408889634f / std::sqrt((float)kPD);
   ra.kw = kw;
   ra.vw = vw;
+  ra.qr = static_cast<__nv_bfloat16*>(out);
   ra.err = err;
   cudaError_t e = hook_begin(hook, s);
   if (e != cudaSuccess) return e;
-  const size_t rsmem = sizeof(RSmem) + 1024, asmem = sizeof(ASmemP) + 1024;
-  e = cudaFuncSetAttribute(recon_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
-  if (e != cudaSuccess) return e;
+  const size_t asmem = sizeof(ASmemP) + 1024;
+  const int pairs = recon_pairs_of_device();
+  if (pairs <= 0) return cudaErrorInvalidConfiguration;
   e = cudaFuncSetAttribute(prefill_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)asmem);
   if (e != cudaSuccess) return e;
-  // Values: V^ = C_v B_v is one dense GEMM over the cache rows (no position
-  // enters it), run on the persistent CTA pairs of the long latent append,
-  // where the per-head reconstruction CTAs would each stream the whole latent
-  // tile for one head; taken when the rows in use can be most of the cache
-  // (every row is computed).  Keys (RoPE at each row's position, the head
-  // groups' factors) stay with the reconstruction kernel.
-  bool v_gemm = n_rows <= 2 * (int64_t)B * max_len && n_rows < (int64_t(1) << 31) - 256;
-  if (v_gemm) {
-    e = launch_gemm_pair(vc, n_rows, lt.rv, Bv, lt.Hkv * kPD, vw, err, s);
-    if (e == cudaErrorNotSupported) {
-      cudaGetLastError();
-      v_gemm = false;
-    } else if (e != cudaSuccess) {
-      return e;
-    } else if ((e = hook_launched(hook, s)) != cudaSuccess) {
-      return e;
-    }
+  // Where the caches hold little but these sequences' rows: the values (tensor
+  // bound, with the pass over q beside them), then the keys; in a pooled cache
+  // one launch for both.
+  const int n_launch = n_rows <= 2 * (int64_t)B * max_len ? 2 : 1;
+  for (int l = 0; l < n_launch; ++l) {
+    ra.n_val = l == 0 ? n_val : 0;
+    ra.n_key = l == n_launch - 1 ? n_key : 0;
+    ra.q = l == 0 ? static_cast<const __nv_bfloat16*>(q) : nullptr;
+    std::copy(val, val + ra.n_val, ra.col);
+    std::copy(key, key + ra.n_key, ra.col + ra.n_val);
+    if ((e = launch_recon(rm, ra, pairs, s)) != cudaSuccess) return e;
+    if ((e = hook_launched(hook, s)) != cudaSuccess) return e;
   }
-  recon_kernel<<<dim3((max_len + kTile - 1) / kTile, B, (v_gemm ? 1 : 2) * lt.Hkv), kRThreads, rsmem, s>>>(rm, ra);
-  if ((e = hook_launched(hook, s)) != cudaSuccess) return e;
   AArgsP aa;
   std::memset(&aa, 0, sizeof(aa));
-  aa.q = static_cast<const __nv_bfloat16*>(q);
   aa.q_len = q_len;
   aa.qmax = qmax;
   aa.max_len = max_len;
@@ -655,7 +851,6 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   aa.Hq = lt.Hq;
   aa.Hkv = lt.Hkv;
   aa.qpg = lt.qpg;
-  std::memcpy(aa.om, ra.om, sizeof(aa.om));
   aa.out = static_cast<__nv_bfloat16*>(out);
   aa.err = err;
   const int qtiles = (qmax * lt.qpg + 127) / 128;
