@@ -13,8 +13,8 @@
 //     rows (tcgen05 pair MMAs), written as bf16 to the workspace [n_rows][Hkv][d]
 //     (keys) and [n_rows][Hkv][d] (values); the new tokens' queries, rotated
 //     and scaled, go to `out`;
-//  2. attn_kernel: causal flash attention over them, one CTA per 128 query
-//     rows of one KV head (the qpg query heads of a KV head packed into the
+//  2. prefill_attn_kernel: causal flash attention over them, 128 query rows of
+//     one KV head per tile (the qpg query heads of a KV head packed into the
 //     rows: row r = query index r / qpg, head r % qpg), S = Q^ K^T and
 //     O += P V^ on the tensor cores (M = 128 rows, N = 128, K = 128 / 128
 //     keys), online softmax in log2 units with a lazy reference max (O in
@@ -464,14 +464,39 @@ cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, cudaStream
 
 // ---------------------------------------------------------------------------
 // 2. causal flash attention over the reconstructed keys and values
+//
+// Persistent CTAs, one per SM, over a list of items (longest first).  An item is
+// two query tiles of 128 rows of one KV head (tile 1 the 128 / qpg positions
+// after tile 0's; it may be missing), so that each K^ / V^ tile read from L2
+// serves 256 rows (64 KB per 2048 cycles of MMA; a tile per CTA took 64 KB per
+// 1024, the ~64 B/clk an SM takes in).  Per key tile the MMA thread issues
+//   O0 += P0 V(j), S0 = Q0 K(j+1)^T, O1 += P1 V(j), S1 = Q1 K(j+1)^T
+// so one tile's softmax runs under the other's MMAs.  P overwrites its scores in
+// TMEM (the softmax has them in registers) and is the A operand of O += P V from
+// there: shared memory holds two query tiles and five K^/V^ slots.  MMAs of one
+// thread run in order, so S(j+1) may be issued right after the P V(j) that reads
+// the same columns, and S(j+1) complete implies P V(j) complete (the softmax
+// may then rescale O).  A softmax thread owns a row: no shuffles.  Four warps
+// of their own write finished tiles out, while the next item's scores and
+// probabilities are formed.
+// TMEM: S0/P0 at column 0, S1/P1 at 128, O0 at 256, O1 at 384.
+//
+// A CTA per 128-row query tile, its softmax on four warps in series with its
+// MMAs and P through shared memory, took 960 us on a 32-head MHA prompt of
+// 2 x 4096 (275 GFLOP) and 1163 us on a GQA prompt of 8192 (550 GFLOP); this
+// kernel 267 and 426 us (339 and 556 with its MMAs issued from a one-lane branch).
 // ---------------------------------------------------------------------------
 
-constexpr int kAThreadsP = 192;  // warp 0 TMA, warp 1 MMA/TMEM, warps 2-5 softmax (thread = query row)
+constexpr int kAThreadsP = 512;   // warp 0 TMA, warp 1 MMA/TMEM, warps 4-7 / 8-11 softmax of tile 0 / 1, 12-15 output
 constexpr int kAtom = 128 * 128;  // one 64-column swizzle atom of 128 rows (16 KB)
+constexpr int kKvSlots = 5;       // ring of K^ and V^ tiles (32 KB): K(0), V(0), K(1), V(1), ...
 constexpr float kThr = 8.f;       // lazy reference max: probabilities stay <= 2^8
+// registers: 512 threads x 128 at launch = 2 x 128 x 176 (softmax) + 2 x 128 x 80
+constexpr int kRegsSoftmax = 176, kRegsOther = 80;
 
 struct AMapsP {
   CUtensorMap kw, vw;  // [n_rows][Hkv d] bf16: box {64, 128 rows}, 128B swizzle
+  CUtensorMap q;       // out as [B Qmax][Hq][d]: box {64, qpg, 128 / qpg}: 128 rows (position, head of the KV head)
 };
 
 struct AArgsP {
@@ -481,65 +506,103 @@ struct AArgsP {
   const int32_t* seq_len;
   int64_t n_rows;
   int B, Hq, Hkv, qpg;
+  int ntp;                 // items (query tile pairs) of q_max queries
+  int group;               // (sequence, KV head) streams whose items are interleaved
   __nv_bfloat16* out;      // [B, Qmax, Hq, d]: rotated queries in, results out
   int* err;
 };
 
 struct ASmemP {
-  uint8_t q[2][kAtom];      // Q^ [d atom][128 rows][128 B], K-major, 128B-swizzled
-  uint8_t k[2][2][kAtom];   // K^ ring [stage][d atom][128 keys][128 B] (TMA)
-  uint8_t v[2][2][kAtom];   // V^ ring [stage][d atom][128 keys][128 B] (TMA)
-  uint8_t p[2][kAtom];      // P [key atom][128 rows][128 B], K-major, 128B-swizzled
-  uint64_t kv_full[2], kv_empty[2], s_full[2], s_free[2], p_ready, o_ready, q_ready;
+  uint8_t q[2][2][kAtom];          // Q^ [query tile][d atom][128 rows][128 B], K-major, 128B-swizzled
+  uint8_t kv[kKvSlots][2][kAtom];  // K^ / V^ [slot][d atom][128 keys][128 B]
+  float linv[2][128];              // [query tile][row] 1 / softmax denominator
+  uint64_t kv_full[kKvSlots], kv_empty[kKvSlots], q_full, q_empty;
+  uint64_t s_full[2], p_full[2][2], l_full[2], o_full[2], o_free[2];  // [query tile] (P: [half of its keys])
   uint32_t tmem_base;
   int abort_flag;
 };
 
-// 16-byte chunk c (0..15 over 128 columns of two atoms) of row r in a K-major
-// 128B-swizzled [2 atoms][128 rows][128 B] tile.
-__device__ __forceinline__ uint32_t swz_chunk(int r, int c) {
-  return (uint32_t)((c >> 3) * kAtom + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+// One item: tiles 0 and 1 start at query indices i0 and i0 + 128 / qpg and
+// attend to n[0] and n[1] key tiles (0: no such tile).
+struct PItem {
+  int b, h, i0, Q, L;
+  int n[2];
+  bool bad;  // the sequence is rejected
+  __device__ int nk() const { return max(n[0], n[1]); }
+};
+
+// Walks the items of CTA blockIdx.x: rounds of gridDim.x items, every other one
+// backwards.  The list takes `group` (sequence, KV head) streams at a time (their
+// keys and values stay in L2 together), their last query tiles, which attend to
+// the most keys, first.
+struct PWalk {
+  int round = 0;
+  __device__ bool next(const AArgsP& aa, PItem& it) {
+    const int64_t streams = (int64_t)aa.B * aa.Hkv, total = streams * aa.ntp;
+    const int G = gridDim.x, c = blockIdx.x;
+    while (true) {
+      const int64_t idx = (int64_t)round * G + ((round & 1) ? G - 1 - c : c);
+      if (idx >= total) return false;
+      ++round;
+      const int64_t per = (int64_t)aa.group * aa.ntp;
+      const int64_t g = idx / per, first = g * aa.group;
+      const int gsz = (int)min((int64_t)aa.group, streams - first);
+      const int64_t rem = idx - g * per;
+      const int t = (int)(rem / gsz);
+      const int64_t st = first + (rem - (int64_t)t * gsz);
+      it.b = (int)(st / aa.Hkv);
+      it.h = (int)(st - (int64_t)it.b * aa.Hkv);
+      const int pp = 128 / aa.qpg;
+      it.i0 = (aa.ntp - 1 - t) * 2 * pp;
+      it.Q = aa.q_len[it.b];
+      if (it.Q == 0) continue;  // no new tokens: nothing to write
+      const int64_t L = aa.seq_len[it.b], row0 = aa.seq_start[it.b];
+      it.L = (int)L;
+      it.bad = it.Q < 0 || it.Q > L || it.Q > aa.qmax || L > aa.max_len || row0 < 0 || row0 + L > aa.n_rows;
+      it.n[0] = it.n[1] = 0;
+      if (it.bad) return true;
+      if (it.i0 >= it.Q) continue;
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const int i = it.i0 + a * pp;
+        if (i < it.Q) it.n[a] = (it.L - it.Q + min(it.Q, i + pp) - 1) / kTile + 1;
+      }
+      return true;
+    }
+  }
+};
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n"
+      " mov.b64 {%0, %1}, z;\n}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
 }
 
-// grid (query tiles of 128 rows, B, Hkv)
 __global__ void __launch_bounds__(kAThreadsP, 1)
     prefill_attn_kernel(const __grid_constant__ AMapsP maps, const __grid_constant__ AArgsP aa) {
   extern __shared__ uint8_t smem_raw[];
   ASmemP& sm = *reinterpret_cast<ASmemP*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* abort_flag = &sm.abort_flag;
-  const int b = blockIdx.y, h = blockIdx.z, qpg = aa.qpg;
-  const int64_t Lraw = aa.seq_len[b], st = aa.seq_start[b];
-  const int Q = aa.q_len[b];
-  const int PP = 128 / qpg;                             // query positions per tile
-  const int i0 = (gridDim.x - 1 - blockIdx.x) * PP;    // first query index (longest tiles first)
-  if (Q == 0) return;                                   // no new tokens: nothing to write
-  if (Q < 0 || Q > Lraw || Q > aa.qmax || Lraw > aa.max_len || st < 0 || st + Lraw > aa.n_rows) {
-    // an invalid sequence: recorded, and its output rows of this tile are zero
-    if (tid == 0 && blockIdx.x == 0 && h == 0) atomicOr(aa.err, kErrBadSeq);
-    for (int e = tid; e < 128 * (kPD / 8); e += blockDim.x) {
-      const int r = e / (kPD / 8), qi = i0 + r / qpg;
-      if (qi < aa.qmax)
-        *reinterpret_cast<uint4*>(aa.out + (((int64_t)b * aa.qmax + qi) * aa.Hq + h * qpg + r % qpg) * kPD +
-                                  8 * (e % (kPD / 8))) = make_uint4(0, 0, 0, 0);
-    }
-    return;
-  }
-  if (i0 >= Q) return;
-  const int L = (int)Lraw;
-  const int64_t row0 = aa.seq_start[b];
-  const int pmax = L - Q + min(Q - 1, i0 + PP - 1);  // last position of the tile's queries
-  const int nkt = pmax / kTile + 1;                   // key tiles it attends to
+  const int qpg = aa.qpg, pp = 128 / qpg;
   if (tid == 0) {
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kKvSlots; ++i) {
       mbar_init(&sm.kv_full[i], 1);
       mbar_init(&sm.kv_empty[i], 1);
-      mbar_init(&sm.s_full[i], 1);
-      mbar_init(&sm.s_free[i], 4);
     }
-    mbar_init(&sm.p_ready, 4);
-    mbar_init(&sm.o_ready, 1);
-    mbar_init(&sm.q_ready, 4);
+    mbar_init(&sm.q_full, 1);
+    mbar_init(&sm.q_empty, 1);
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&sm.s_full[a], 1);
+      mbar_init(&sm.p_full[a][0], 4);
+      mbar_init(&sm.p_full[a][1], 4);
+      mbar_init(&sm.l_full[a], 4);
+      mbar_init(&sm.o_full[a], 1);
+      mbar_init(&sm.o_free[a], 4);
+    }
     sm.abort_flag = 0;
     fence_mbar_init();
   }
@@ -550,172 +613,287 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;  // S buffers at columns 0 and 128, O at 256
-  if (warp == 0) {
-    if (lane == 0) {
-      const uint64_t pol = policy_evict_last();  // a KV tile is read by several query tiles
-      for (int kt = 0; kt < nkt; ++kt) {
-        const int sl = kt & 1;
-        if (kt >= 2 && !mbar_wait(&sm.kv_empty[sl], ((kt - 2) >> 1) & 1, abort_flag)) break;
-        mbar_expect_tx(&sm.kv_full[sl], 4 * kAtom);
-        const int32_t y = (int32_t)(row0 + (int64_t)kTile * kt);
-        for (int a = 0; a < 2; ++a) {
-          tma_load_2d_hint(sm.k[sl][a], &maps.kw, &sm.kv_full[sl], h * kPD + 64 * a, y, pol);
-          tma_load_2d_hint(sm.v[sl][a], &maps.vw, &sm.kv_full[sl], h * kPD + 64 * a, y, pol);
+  const uint32_t tmem = sm.tmem_base;
+  PWalk walk;
+  PItem it;
+
+  if (warp < 4) {
+    reg_dec<kRegsOther>();
+    if (warp == 0) {
+      if (lane == 0) {
+        const uint64_t pol = policy_evict_last();  // a K^ / V^ tile is read by several items
+        int cnt = 0, items = 0;
+        bool ok = true;
+        while (ok && walk.next(aa, it)) {
+          const int nk = it.nk();
+          if (nk == 0) continue;
+          const int64_t row0 = aa.seq_start[it.b];
+          auto load_kv = [&](const CUtensorMap* m, int kt) -> bool {
+            const int sl = cnt % kKvSlots;
+            if (cnt >= kKvSlots && !mbar_wait(&sm.kv_empty[sl], ((cnt / kKvSlots) - 1) & 1, abort_flag)) return false;
+            mbar_expect_tx(&sm.kv_full[sl], 2 * kAtom);
+            const int32_t y = (int32_t)(row0 + (int64_t)kTile * kt);
+            for (int at = 0; at < 2; ++at)
+              tma_load_2d_hint(sm.kv[sl][at], m, &sm.kv_full[sl], it.h * kPD + 64 * at, y, pol);
+            ++cnt;
+            return true;
+          };
+          if (!(ok = load_kv(&maps.kw, 0))) break;
+          // the previous item's scores are all formed: its queries can go
+          if (items >= 1 && !(ok = mbar_wait(&sm.q_empty, (items - 1) & 1, abort_flag))) break;
+          mbar_expect_tx(&sm.q_full, (it.n[1] ? 4 : 2) * kAtom);
+          for (int a = 0; a < (it.n[1] ? 2 : 1); ++a)
+            for (int at = 0; at < 2; ++at)
+              tma_load_3d(sm.q[a][at], &maps.q, &sm.q_full, 64 * at, it.h * qpg, it.b * aa.qmax + it.i0 + a * pp);
+          ++items;
+          for (int kt = 0; kt < nk && ok; ++kt) {
+            if (kt > 0) ok = load_kv(&maps.kw, kt);
+            ok = ok && load_kv(&maps.vw, kt);
+          }
+        }
+      }
+    } else if (warp == 1) {
+      // the whole warp runs the schedule and one elected lane issues (see elect_one)
+      const bool el = elect_one();
+      const uint32_t id_s = idesc_bf16(128, 128, false, false);  // S = Q K^T: both K-major
+      const uint32_t id_o = idesc_bf16(128, 128, false, true);   // O += P V: V MN-major
+      const uint64_t dq = sdesc(smem_u32(sm.q[0][0]), 16, 1024, kSw128);
+      const uint64_t dk = sdesc(smem_u32(sm.kv[0][0]), 16, 1024, kSw128);
+      const uint64_t dv = sdesc(smem_u32(sm.kv[0][0]), kAtom, 1024, kSw128);
+      int slot = 0;                     // ring slot of the next K^/V^ tile and its phase
+      uint32_t sphase = 0;
+      uint32_t items = 0;
+      uint32_t pph[2] = {0, 0};         // P tiles so far
+      uint32_t oph[2] = {0, 0};         // finished output tiles so far
+      bool ok = true;
+      // waits for the ring's next tile; its slot
+      auto kv_next = [&](int& sl) {
+        sl = slot;
+        const bool r = wwait(&sm.kv_full[slot], sphase, abort_flag);
+        if (++slot == kKvSlots) {
+          slot = 0;
+          sphase ^= 1;
+        }
+        return r;
+      };
+      while (ok && walk.next(aa, it)) {
+        const int nk = it.nk();
+        if (nk == 0) continue;
+        const int n0 = it.n[0], n1 = it.n[1];
+        // S_a = Q_a K^T
+        auto scores = [&](int a, int sl) {
+          const uint64_t qb = dq + (uint64_t)(a * (2 * kAtom >> 4)), kb = dk + (uint64_t)(sl * (2 * kAtom >> 4));
+          if (el) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const uint64_t o = ((k >> 2) * kAtom + (k & 3) * 32) >> 4;
+              umma_f16(tmem + 128 * a, qb + o, kb + o, id_s, k > 0 ? 1u : 0u);
+            }
+            umma_commit(&sm.s_full[a]);
+          }
+        };
+        int ks, vs, kn = 0;
+        if (!(ok = wwait(&sm.q_full, items & 1, abort_flag))) break;
+        ++items;
+        if (!(ok = kv_next(ks))) break;
+        tc_fence_after();
+        if (n0) scores(0, ks);
+        if (n1) scores(1, ks);
+        if (el) {
+          umma_commit(&sm.kv_empty[ks]);
+          if (nk == 1) umma_commit(&sm.q_empty);
+        }
+        for (int kt = 0; kt < nk && ok; ++kt) {
+          const bool more = kt + 1 < nk;
+          bool have_k = false;
+          if (!(ok = kv_next(vs))) break;
+          const uint64_t vb = dv + (uint64_t)(vs * (2 * kAtom >> 4));
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            const int n = a ? n1 : n0;
+            if (kt < n) {
+              if (kt == 0 && oph[a] >= 1 && !(ok = wwait(&sm.o_free[a], (oph[a] - 1) & 1, abort_flag))) break;
+#pragma unroll
+              for (int hf = 0; hf < 2; ++hf) {
+                if (!(ok = wwait(&sm.p_full[a][hf], pph[a] & 1, abort_flag))) break;
+                tc_fence_after();
+                if (el) {
+#pragma unroll
+                  for (int k = 4 * hf; k < 4 * hf + 4; ++k)
+                    umma_f16_ts(tmem + 256 + 128 * a, tmem + 128 * a + 8 * k, vb + (uint64_t)(k * 2048 >> 4), id_o,
+                                (kt > 0 || k > 0) ? 1u : 0u);
+                }
+              }
+              if (!ok) break;
+              ++pph[a];
+              if (kt + 1 == n) {
+                if (el) umma_commit(&sm.o_full[a]);
+                ++oph[a];
+              }
+            }
+            if (kt + 1 < n) {
+              if (!have_k && !(ok = kv_next(kn))) break;
+              have_k = true;
+              tc_fence_after();
+              scores(a, kn);
+            }
+          }
+          if (!ok) break;
+          if (el) {
+            umma_commit(&sm.kv_empty[vs]);
+            if (more) umma_commit(&sm.kv_empty[kn]);
+            if (kt + 2 == nk) umma_commit(&sm.q_empty);  // every score of the item has been issued
+          }
         }
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t id_s = idesc_bf16(128, 128, false, false);   // S = Q K^T: both K-major
-      const uint32_t id_o = idesc_bf16(128, 128, false, true);    // O += P V: V MN-major
-      bool ok = mbar_wait(&sm.q_ready, 0, abort_flag);
-      auto pv = [&](int j) -> bool {  // O += P_j V_j
-        if (!mbar_wait(&sm.p_ready, j & 1, abort_flag)) return false;
-        tc_fence_after();
-        const int sl = j & 1;
-        for (int k = 0; k < 8; ++k)
-          umma_f16(tmem + 256, sdesc(smem_u32(sm.p[k >> 2]) + (k & 3) * 32, 16, 1024, kSw128),
-                   sdesc(smem_u32(sm.v[sl][0]) + k * 2048, kAtom, 1024, kSw128), id_o, (j > 0 || k > 0) ? 1u : 0u);
-        umma_commit(&sm.kv_empty[sl]);
-        umma_commit(&sm.o_ready);
-        return true;
-      };
-      for (int kt = 0; kt < nkt && ok; ++kt) {
-        const int sl = kt & 1;
-        if (!(ok = mbar_wait(&sm.kv_full[sl], (kt >> 1) & 1, abort_flag))) break;
-        if (kt >= 2 && !(ok = mbar_wait(&sm.s_free[sl], ((kt - 2) >> 1) & 1, abort_flag))) break;
-        tc_fence_after();
-        for (int k = 0; k < 8; ++k)
-          umma_f16(tmem + 128 * sl, sdesc(smem_u32(sm.q[k >> 2]) + (k & 3) * 32, 16, 1024, kSw128),
-                   sdesc(smem_u32(sm.k[sl][k >> 2]) + (k & 3) * 32, 16, 1024, kSw128), id_s, k > 0 ? 1u : 0u);
-        umma_commit(&sm.s_full[sl]);
-        if (kt >= 1 && !(ok = pv(kt - 1))) break;
+  } else if (warp < 12) {
+    // ---- softmax of query tile a: thread = row r ---------------------------------
+    reg_inc<kRegsSoftmax>();
+    const int a = (warp - 4) >> 2, quad = warp & 3, r = quad * 32 + lane;
+    const uint32_t lb = (uint32_t)(quad * 32) << 16;
+    const uint32_t sb = tmem + lb + 128 * a, ob = tmem + lb + 256 + 128 * a;
+    int base = 0;
+    uint32_t sph = 0, oph = 0;
+    bool ok = true;
+    while (ok && walk.next(aa, it)) {
+      const int nk = it.nk(), n = it.n[a];
+      if (n == 0) {
+        base += 2 * nk;
+        continue;
       }
-      if (ok) pv(nkt - 1);
+      const int qi = it.i0 + a * pp + r / qpg;
+      const bool valid = qi < it.Q;
+      const int pos = it.L - it.Q + qi;
+      float m = -INFINITY;
+      float2 l = make_float2(0.f, 0.f);
+      for (int kt = 0; kt < n; ++kt) {
+        if (!(ok = wwait(&sm.s_full[a], sph & 1, abort_flag))) break;
+        ++sph;
+        tc_fence_after();
+        float sv[128];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tmem_ld32(sb + 32 * c, *reinterpret_cast<float(*)[32]>(&sv[32 * c]));
+        tmem_wait_ld();
+        const int kbase = kTile * kt;
+        const int vis = valid ? pos - kbase + 1 : 0;  // visible keys of this tile: [0, vis)
+        if (!__all_sync(0xffffffffu, vis >= kTile)) {
+#pragma unroll
+          for (int i = 0; i < 128; ++i) sv[i] = i < vis ? sv[i] : -INFINITY;
+        }
+        float mx[4] = {sv[0], sv[1], sv[2], sv[3]};
+#pragma unroll
+        for (int i = 4; i < 128; i += 8)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) mx[u] = fmaxf(mx[u], i + 4 + u < 128 ? fmaxf(sv[i + u], sv[i + 4 + u]) : sv[i + u]);
+        const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        // a new reference max for this row when the tile's max passes the old one by
+        // kThr; O and l are rescaled where a reference existed.  The TMEM loads and
+        // stores are warp-collective, so the whole warp runs them when any row
+        // rescales (factor 1 for the other rows).
+        const bool upd = mt != -INFINITY && (m == -INFINITY || mt > m + kThr);
+        const bool resc = upd && m != -INFINITY;
+        if (__any_sync(0xffffffffu, resc)) {
+          const float al = resc ? exp2f(m - mt) : 1.f;
+#pragma unroll 1
+          for (int c = 0; c < 8; ++c) {
+            float v[16];
+            tmem_ld16(ob + 16 * c, v);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] *= al;
+            tmem_st16(ob + 16 * c, v);
+          }
+          l.x *= al;
+          l.y *= al;
+        }
+        if (upd) m = mt;
+        // keys past the sequence in its last tile: exact zeros in V^ (P is zero there),
+        // written once by the first query tile that uses them
+        if (kbase + kTile > it.L && a == (kt < it.n[0] ? 0 : 1)) {
+          const int c = base + 2 * kt + 1;
+          if (!(ok = wwait(&sm.kv_full[c % kKvSlots], (c / kKvSlots) & 1, abort_flag))) break;
+          if (kbase + r >= it.L)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              reinterpret_cast<uint4*>(sm.kv[c % kKvSlots][0] + r * 128)[q] = make_uint4(0, 0, 0, 0);
+              reinterpret_cast<uint4*>(sm.kv[c % kKvSlots][1] + r * 128)[q] = make_uint4(0, 0, 0, 0);
+            }
+          fence_proxy_async_smem();
+        }
+        // P = 2^(s - m) (bf16, the row sum over the rounded values); no visible key yet: all zero
+        const float mu = m == -INFINITY ? 0.f : m;
+        const float2 nm = make_float2(-mu, -mu);
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          uint32_t pk[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float2 d = add2(make_float2(sv[64 * hf + 2 * i], sv[64 * hf + 2 * i + 1]), nm);
+            pk[i] = pack2(ex2_approx(d.x), ex2_approx(d.y));
+            l = add2(l, unpack2(pk[i]));
+          }
+          tmem_st32(sb + 32 * hf, pk);
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.p_full[a][hf]);
+        }
+      }
+      if (!ok) break;
+      base += 2 * nk;
+      // the previous item's 1 / l has been read
+      if (oph >= 1 && !(ok = wwait(&sm.o_free[a], (oph - 1) & 1, abort_flag))) break;
+      ++oph;
+      const float lt = l.x + l.y;
+      sm.linv[a][r] = lt > 0.f ? 1.f / lt : 0.f;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.l_full[a]);
     }
   } else {
-    // ---- softmax and output: thread = query row r ----------------------------
+    // ---- output: thread = row r of each tile --------------------------------------
+    reg_dec<kRegsOther>();
     const int quad = warp & 3, r = quad * 32 + lane;
     const uint32_t lb = (uint32_t)(quad * 32) << 16;
-    const int qi = i0 + r / qpg, j = h * qpg + r % qpg;
-    const bool valid = qi < Q;
-    const int pos = L - Q + (valid ? qi : 0);
-    // Q^ row (rotated and scaled by the reconstruction launch)
-    {
-      const uint4* qr = reinterpret_cast<const uint4*>(aa.out + (((int64_t)b * aa.qmax + (valid ? qi : 0)) * aa.Hq + j) * kPD);
-#pragma unroll
-      for (int cc = 0; cc < 16; ++cc)
-        *reinterpret_cast<uint4*>(&sm.q[0][0] + swz_chunk(r, cc)) = valid ? qr[cc] : make_uint4(0, 0, 0, 0);
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.q_ready);
-    }
-    float m = -INFINITY, l = 0.f;
+    uint32_t oph[2] = {0, 0};
     bool ok = true;
-    for (int kt = 0; kt < nkt && ok; ++kt) {
-      const int sl = kt & 1;
-      if (!(ok = wwait(&sm.s_full[sl], (kt >> 1) & 1, abort_flag))) break;
-      tc_fence_after();
-      const uint32_t sb = tmem + lb + 128 * sl;
-      const int kbase = kTile * kt;
-      const int vis = valid ? min(pos - kbase + 1, kTile) : 0;  // visible keys of this tile: [0, vis)
-      // the row's 128 scores in one TMEM round trip, then the tile's max over visible keys
-      float sv[4][32];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) tmem_ld32(sb + 32 * c, sv[c]);
-      tmem_wait_ld();
-      float mt = -INFINITY;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (32 * c + i < vis) mt = fmaxf(mt, sv[c][i]);
-      // the S buffer has been read
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.s_free[sl]);
-      // a new reference max for this row when the tile's max passes the old one by kThr;
-      // O and l are rescaled where a reference existed.  The TMEM loads and stores are
-      // warp-collective, so the whole warp runs them when any row rescales (factor 1
-      // for the other rows).
-      const bool upd = mt != -INFINITY && (m == -INFINITY || mt > m + kThr);
-      const bool resc = upd && m != -INFINITY;
-      const float al = resc ? exp2f(m - mt) : 1.f;
-      // PV of the previous tile must be done before P is overwritten and before O is rescaled
-      if (kt >= 1 && !(ok = wwait(&sm.o_ready, (kt - 1) & 1, abort_flag))) break;
-      tc_fence_after();
-      if (__any_sync(0xffffffffu, resc)) {
-#pragma unroll
+    while (ok && walk.next(aa, it)) {
+      if (it.bad) {
+        // an invalid sequence: recorded, and its output rows of this item are zero
+        if (tid == 12 * 32 && it.i0 == 0 && it.h == 0) atomicOr(aa.err, kErrBadSeq);
+        for (int e = tid - 12 * 32; e < 256 * (kPD / 8); e += 128) {
+          const int rr = e / (kPD / 8), qi = it.i0 + rr / qpg;
+          if (qi < aa.qmax)
+            *reinterpret_cast<uint4*>(aa.out + (((int64_t)it.b * aa.qmax + qi) * aa.Hq + it.h * qpg + rr % qpg) * kPD +
+                                      8 * (e % (kPD / 8))) = make_uint4(0, 0, 0, 0);
+        }
+        continue;
+      }
+#pragma unroll 1
+      for (int a = 0; a < 2 && ok; ++a) {
+        if (it.n[a] == 0) continue;
+        if (!(ok = wwait(&sm.o_full[a], oph[a] & 1, abort_flag))) break;
+        if (!(ok = wwait(&sm.l_full[a], oph[a] & 1, abort_flag))) break;
+        ++oph[a];
+        tc_fence_after();
+        const int qi = it.i0 + a * pp + r / qpg;
+        const float inv = sm.linv[a][r];
+        __nv_bfloat16* orow = aa.out + (((int64_t)it.b * aa.qmax + qi) * aa.Hq + it.h * qpg + r % qpg) * kPD;
+#pragma unroll 1
         for (int c = 0; c < 4; ++c) {
           float v[32];
-          tmem_ld32(tmem + lb + 256 + 32 * c, v);
+          tmem_ld32(tmem + lb + 256 + 128 * a + 32 * c, v);
           tmem_wait_ld();
-          float w16[16];
+          if (qi < it.Q)
 #pragma unroll
-          for (int i = 0; i < 16; ++i) w16[i] = v[i] * al;
-          tmem_st16(tmem + lb + 256 + 32 * c, w16);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) w16[i] = v[16 + i] * al;
-          tmem_st16(tmem + lb + 256 + 32 * c + 16, w16);
+            for (int q = 0; q < 4; ++q)
+              *reinterpret_cast<uint4*>(orow + 32 * c + 8 * q) =
+                  make_uint4(pack2(v[8 * q] * inv, v[8 * q + 1] * inv), pack2(v[8 * q + 2] * inv, v[8 * q + 3] * inv),
+                             pack2(v[8 * q + 4] * inv, v[8 * q + 5] * inv), pack2(v[8 * q + 6] * inv, v[8 * q + 7] * inv));
         }
-        tmem_wait_st();
-      }
-      l *= al;
-      if (upd) m = mt;
-      // P = 2^(s - m) over visible keys (bf16, the row sum over the rounded values)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float* v = sv[c];
-#pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          uint4 o;
-          __nv_bfloat162* po = reinterpret_cast<__nv_bfloat162*>(&o);
-#pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int k0 = 32 * c + 8 * cc + 2 * t;
-            const float p0 = k0 < vis ? ex2_approx(v[8 * cc + 2 * t] - m) : 0.f;
-            const float p1 = k0 + 1 < vis ? ex2_approx(v[8 * cc + 2 * t + 1] - m) : 0.f;
-            po[t] = __floats2bfloat162_rn(p0, p1);
-            const float2 pr = __bfloat1622float2(po[t]);
-            l += pr.x + pr.y;
-          }
-          *reinterpret_cast<uint4*>(&sm.p[0][0] + swz_chunk(r, 4 * c + cc)) = o;
-        }
-      }
-      // keys past the sequence in its last tile: exact zeros in V^ (P is zero there)
-      if (kbase + r >= L) {
-        uint4* z0 = reinterpret_cast<uint4*>(sm.v[sl][0] + r * 128);
-        uint4* z1 = reinterpret_cast<uint4*>(sm.v[sl][1] + r * 128);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          z0[c] = make_uint4(0, 0, 0, 0);
-          z1[c] = make_uint4(0, 0, 0, 0);
-        }
-      }
-      fence_proxy_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.p_ready);
-    }
-    if (ok) ok = wwait(&sm.o_ready, (nkt - 1) & 1, abort_flag);
-    if (ok) {
-      tc_fence_after();
-      const float inv = l > 0.f ? 1.f / l : 0.f;
-      __nv_bfloat16* orow = aa.out + (((int64_t)b * aa.qmax + qi) * aa.Hq + j) * kPD;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float v[32];
-        tmem_ld32(tmem + lb + 256 + 32 * c, v);
-        tmem_wait_ld();
-        if (valid)
-#pragma unroll
-          for (int cc = 0; cc < 4; ++cc) {
-            uint4 o;
-            __nv_bfloat162* po = reinterpret_cast<__nv_bfloat162*>(&o);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) po[t] = __floats2bfloat162_rn(v[8 * cc + 2 * t] * inv, v[8 * cc + 2 * t + 1] * inv);
-            *reinterpret_cast<uint4*>(orow + 32 * c + 8 * cc) = o;
-          }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.o_free[a]);
       }
     }
   }
@@ -781,7 +959,9 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   ok = ok && make_tmap_2d_bf16(&am.kw, kw, (uint64_t)lt.Hkv * kPD, rows, (uint64_t)lt.Hkv * kPD * 2, 64, kTile,
                                CU_TENSOR_MAP_SWIZZLE_128B) &&
        make_tmap_2d_bf16(&am.vw, vw, (uint64_t)lt.Hkv * kPD, rows, (uint64_t)lt.Hkv * kPD * 2, 64, kTile,
-                         CU_TENSOR_MAP_SWIZZLE_128B);
+                         CU_TENSOR_MAP_SWIZZLE_128B) &&
+       make_tmap_3d_bf16(&am.q, out, kPD, lt.Hq, (uint64_t)B * qmax, kPD * 2, (uint64_t)lt.Hq * kPD * 2, 64, lt.qpg,
+                         128 / lt.qpg, CU_TENSOR_MAP_SWIZZLE_128B);
   if (!ok) return cudaErrorInvalidValue;
   RArgs ra;
   std::memset(&ra, 0, sizeof(ra));
@@ -853,8 +1033,16 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   aa.qpg = lt.qpg;
   aa.out = static_cast<__nv_bfloat16*>(out);
   aa.err = err;
-  const int qtiles = (qmax * lt.qpg + 127) / 128;
-  prefill_attn_kernel<<<dim3(qtiles, B, lt.Hkv), kAThreadsP, asmem, s>>>(am, aa);
+  const int pp2 = 2 * (128 / lt.qpg);
+  aa.ntp = (qmax + pp2 - 1) / pp2;
+  // streams whose keys and values (at most) share L2: about half of it
+  const int64_t streams = (int64_t)B * lt.Hkv;
+  aa.group = (int)std::max<int64_t>(1, std::min<int64_t>(streams, (int64_t(64) << 20) / ((int64_t)max_len * kPD * 4)));
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const int64_t items = streams * aa.ntp;
+  prefill_attn_kernel<<<(int)std::min<int64_t>(items, sms), kAThreadsP, asmem, s>>>(am, aa);
   return hook_launched(hook, s);
 }
 
