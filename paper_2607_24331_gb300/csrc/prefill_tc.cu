@@ -469,7 +469,7 @@ cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, cudaStream
 // two query tiles of 128 rows of one KV head (tile 1 the 128 / qpg positions
 // after tile 0's; it may be missing), so that each K^ / V^ tile read from L2
 // serves 256 rows (64 KB per 2048 cycles of MMA; a tile per CTA took 64 KB per
-// 1024, the ~64 B/clk an SM takes in).  Per key tile the MMA thread issues
+// 1024, the ~64 B/clk an SM takes in).  Per key tile the MMA warp issues
 //   O0 += P0 V(j), S0 = Q0 K(j+1)^T, O1 += P1 V(j), S1 = Q1 K(j+1)^T
 // so one tile's softmax runs under the other's MMAs.  P overwrites its scores in
 // TMEM (the softmax has them in registers) and is the A operand of O += P V from
@@ -487,8 +487,11 @@ cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, cudaStream
 // kernel 267 and 426 us (339 and 556 with its MMAs issued from a one-lane branch).
 // ---------------------------------------------------------------------------
 
-constexpr int kAThreadsP = 512;   // warp 0 TMA, warp 1 MMA/TMEM, warps 4-7 / 8-11 softmax of tile 0 / 1, 12-15 output
+// warp 0 TMA, warp 1 MMA/TMEM, warp 2 schedule, warps 4-7 and 8-11 softmax of tile 0 and 1, warps 12-15 output
+constexpr int kAThreadsP = 512;
 constexpr int kAtom = 128 * 128;  // one 64-column swizzle atom of 128 rows (16 KB)
+constexpr int kItems = 4;         // items in flight between the scheduler warp and the others
+constexpr int kItemReaders = 14;  // producer, MMA warp, eight softmax warps, four output warps
 constexpr int kKvSlots = 5;       // ring of K^ and V^ tiles (32 KB): K(0), V(0), K(1), V(1), ...
 constexpr float kThr = 8.f;       // lazy reference max: probabilities stay <= 2^8
 // registers: 512 threads x 128 at launch = 2 x 128 x 176 (softmax) + 2 x 128 x 80
@@ -512,23 +515,26 @@ struct AArgsP {
   int* err;
 };
 
-struct ASmemP {
-  uint8_t q[2][2][kAtom];          // Q^ [query tile][d atom][128 rows][128 B], K-major, 128B-swizzled
-  uint8_t kv[kKvSlots][2][kAtom];  // K^ / V^ [slot][d atom][128 keys][128 B]
-  float linv[2][128];              // [query tile][row] 1 / softmax denominator
-  uint64_t kv_full[kKvSlots], kv_empty[kKvSlots], q_full, q_empty;
-  uint64_t s_full[2], p_full[2][2], l_full[2], o_full[2], o_free[2];  // [query tile] (P: [half of its keys])
-  uint32_t tmem_base;
-  int abort_flag;
-};
-
 // One item: tiles 0 and 1 start at query indices i0 and i0 + 128 / qpg and
 // attend to n[0] and n[1] key tiles (0: no such tile).
 struct PItem {
   int b, h, i0, Q, L;
   int n[2];
-  bool bad;  // the sequence is rejected
+  int bad;  // the sequence is rejected
+  int64_t row0;
   __device__ int nk() const { return max(n[0], n[1]); }
+};
+
+struct ASmemP {
+  uint8_t q[2][2][kAtom];          // Q^ [query tile][d atom][128 rows][128 B], K-major, 128B-swizzled
+  uint8_t kv[kKvSlots][2][kAtom];  // K^ / V^ [slot][d atom][128 keys][128 B]
+  float linv[2][128];              // [query tile][row] 1 / softmax denominator
+  PItem item[kItems];              // items handed to the warps, in order; b < 0 ends the list
+  uint64_t i_full[kItems], i_empty[kItems];
+  uint64_t kv_full[kKvSlots], kv_empty[kKvSlots], q_full, q_empty;
+  uint64_t s_full[2], p_full[2][2], l_full[2], o_full[2], o_free[2];  // [query tile] (P: [half of its keys])
+  uint32_t tmem_base;
+  int abort_flag;
 };
 
 // Walks the items of CTA blockIdx.x: rounds of gridDim.x items, every other one
@@ -556,9 +562,10 @@ struct PWalk {
       it.i0 = (aa.ntp - 1 - t) * 2 * pp;
       it.Q = aa.q_len[it.b];
       if (it.Q == 0) continue;  // no new tokens: nothing to write
-      const int64_t L = aa.seq_len[it.b], row0 = aa.seq_start[it.b];
+      const int64_t L = aa.seq_len[it.b];
+      it.row0 = aa.seq_start[it.b];
       it.L = (int)L;
-      it.bad = it.Q < 0 || it.Q > L || it.Q > aa.qmax || L > aa.max_len || row0 < 0 || row0 + L > aa.n_rows;
+      it.bad = it.Q < 0 || it.Q > L || it.Q > aa.qmax || L > aa.max_len || it.row0 < 0 || it.row0 + L > aa.n_rows;
       it.n[0] = it.n[1] = 0;
       if (it.bad) return true;
       if (it.i0 >= it.Q) continue;
@@ -569,6 +576,20 @@ struct PWalk {
       }
       return true;
     }
+  }
+};
+
+// A warp's copy of its CTA's item list (written by the scheduler warp).
+struct PItems {
+  int n = 0;
+  __device__ bool next(ASmemP& sm, PItem& it, int lane, volatile int* abort_flag) {
+    const int i = n % kItems;
+    if (!wwait(&sm.i_full[i], (n / kItems) & 1, abort_flag)) return false;
+    it = sm.item[i];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sm.i_empty[i]);
+    ++n;
+    return it.b >= 0;
   }
 };
 
@@ -593,6 +614,10 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
       mbar_init(&sm.kv_full[i], 1);
       mbar_init(&sm.kv_empty[i], 1);
     }
+    for (int i = 0; i < kItems; ++i) {
+      mbar_init(&sm.i_full[i], 1);
+      mbar_init(&sm.i_empty[i], kItemReaders);
+    }
     mbar_init(&sm.q_full, 1);
     mbar_init(&sm.q_empty, 1);
     for (int a = 0; a < 2; ++a) {
@@ -614,57 +639,62 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
-  PWalk walk;
+  PItems list;
   PItem it;
 
   if (warp < 4) {
     reg_dec<kRegsOther>();
     if (warp == 0) {
-      if (lane == 0) {
-        const uint64_t pol = policy_evict_last();  // a K^ / V^ tile is read by several items
-        int cnt = 0, items = 0;
-        bool ok = true;
-        while (ok && walk.next(aa, it)) {
-          const int nk = it.nk();
-          if (nk == 0) continue;
-          const int64_t row0 = aa.seq_start[it.b];
-          auto load_kv = [&](const CUtensorMap* m, int kt) -> bool {
-            const int sl = cnt % kKvSlots;
-            if (cnt >= kKvSlots && !mbar_wait(&sm.kv_empty[sl], ((cnt / kKvSlots) - 1) & 1, abort_flag)) return false;
-            mbar_expect_tx(&sm.kv_full[sl], 2 * kAtom);
-            const int32_t y = (int32_t)(row0 + (int64_t)kTile * kt);
-            for (int at = 0; at < 2; ++at)
-              tma_load_2d_hint(sm.kv[sl][at], m, &sm.kv_full[sl], it.h * kPD + 64 * at, y, pol);
-            ++cnt;
-            return true;
-          };
-          if (!(ok = load_kv(&maps.kw, 0))) break;
-          // the previous item's scores are all formed: its queries can go
-          if (items >= 1 && !(ok = mbar_wait(&sm.q_empty, (items - 1) & 1, abort_flag))) break;
-          mbar_expect_tx(&sm.q_full, (it.n[1] ? 4 : 2) * kAtom);
-          for (int a = 0; a < (it.n[1] ? 2 : 1); ++a)
-            for (int at = 0; at < 2; ++at)
-              tma_load_3d(sm.q[a][at], &maps.q, &sm.q_full, 64 * at, it.h * qpg, it.b * aa.qmax + it.i0 + a * pp);
-          ++items;
-          for (int kt = 0; kt < nk && ok; ++kt) {
-            if (kt > 0) ok = load_kv(&maps.kw, kt);
-            ok = ok && load_kv(&maps.vw, kt);
+      const uint64_t pol = policy_evict_last();  // a K^ / V^ tile is read by several items
+      int slot = 0;
+      uint32_t sphase = 1, items = 0;  // a fresh barrier passes a wait for the phase before its first
+      bool ok = true;
+      while (ok && list.next(sm, it, lane, abort_flag)) {
+        const int nk = it.nk();
+        if (nk == 0) continue;
+        auto load_kv = [&](const CUtensorMap* m, int kt) -> bool {
+          if (!wwait(&sm.kv_empty[slot], sphase, abort_flag)) return false;
+          if (lane == 0) mbar_expect_tx(&sm.kv_full[slot], 2 * kAtom);
+          __syncwarp();
+          const int32_t y = (int32_t)(it.row0 + (int64_t)kTile * kt);
+          if (lane < 2) tma_load_2d_hint(sm.kv[slot][lane], m, &sm.kv_full[slot], it.h * kPD + 64 * lane, y, pol);
+          if (++slot == kKvSlots) {
+            slot = 0;
+            sphase ^= 1;
           }
+          return true;
+        };
+        if (!(ok = load_kv(&maps.kw, 0))) break;
+        // the previous item's scores are all formed: its queries can go
+        if (items >= 1 && !(ok = wwait(&sm.q_empty, (items - 1) & 1, abort_flag))) break;
+        const int nq = it.n[1] ? 4 : 2;
+        if (lane == 0) mbar_expect_tx(&sm.q_full, nq * kAtom);
+        __syncwarp();
+        if (lane < nq)
+          tma_load_3d(sm.q[lane >> 1][lane & 1], &maps.q, &sm.q_full, 64 * (lane & 1), it.h * qpg,
+                      it.b * aa.qmax + it.i0 + (lane >> 1) * pp);
+        ++items;
+        for (int kt = 0; kt < nk && ok; ++kt) {
+          if (kt > 0) ok = load_kv(&maps.kw, kt);
+          ok = ok && load_kv(&maps.vw, kt);
         }
       }
     } else if (warp == 1) {
-      // the whole warp runs the schedule and one elected lane issues (see elect_one)
+      // ---- MMAs: the whole warp runs the schedule and one elected lane issues (see
+      // elect_one).  One warp for both query tiles: with a warp for each, their MMAs
+      // interleaved one by one, both tiles' scores were ready at the same time and
+      // the tensor pipe idled under both softmaxes (GQA prompt 8192: 490 us against
+      // 426). ----------------------------------------------------------------------
       const bool el = elect_one();
       const uint32_t id_s = idesc_bf16(128, 128, false, false);  // S = Q K^T: both K-major
       const uint32_t id_o = idesc_bf16(128, 128, false, true);   // O += P V: V MN-major
       const uint64_t dq = sdesc(smem_u32(sm.q[0][0]), 16, 1024, kSw128);
       const uint64_t dk = sdesc(smem_u32(sm.kv[0][0]), 16, 1024, kSw128);
       const uint64_t dv = sdesc(smem_u32(sm.kv[0][0]), kAtom, 1024, kSw128);
-      int slot = 0;                     // ring slot of the next K^/V^ tile and its phase
-      uint32_t sphase = 0;
-      uint32_t items = 0;
-      uint32_t pph[2] = {0, 0};         // P tiles so far
-      uint32_t oph[2] = {0, 0};         // finished output tiles so far
+      int slot = 0;  // ring slot of the next K^/V^ tile and its phase
+      uint32_t sphase = 0, items = 0;
+      uint32_t pph[2] = {0, 0};  // P tiles so far
+      uint32_t oph[2] = {0, 0};  // finished output tiles so far
       bool ok = true;
       // waits for the ring's next tile; its slot
       auto kv_next = [&](int& sl) {
@@ -676,7 +706,7 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
         }
         return r;
       };
-      while (ok && walk.next(aa, it)) {
+      while (ok && list.next(sm, it, lane, abort_flag)) {
         const int nk = it.nk();
         if (nk == 0) continue;
         const int n0 = it.n[0], n1 = it.n[1];
@@ -746,6 +776,20 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
           }
         }
       }
+    } else if (warp == 2) {
+      // ---- schedule: the item list, a few items ahead ---------------------------
+      PWalk walk;
+      bool more = true;
+      for (int n = 0; more; ++n) {
+        const int i = n % kItems;
+        if (n >= kItems && !wwait(&sm.i_empty[i], ((n / kItems) - 1) & 1, abort_flag)) break;
+        more = walk.next(aa, it);
+        if (!more) it.b = -1;
+        if (lane == 0) {
+          sm.item[i] = it;
+          mbar_arrive(&sm.i_full[i]);
+        }
+      }
     }
   } else if (warp < 12) {
     // ---- softmax of query tile a: thread = row r ---------------------------------
@@ -756,7 +800,7 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
     int base = 0;
     uint32_t sph = 0, oph = 0;
     bool ok = true;
-    while (ok && walk.next(aa, it)) {
+    while (ok && list.next(sm, it, lane, abort_flag)) {
       const int nk = it.nk(), n = it.n[a];
       if (n == 0) {
         base += 2 * nk;
@@ -857,7 +901,7 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
     const uint32_t lb = (uint32_t)(quad * 32) << 16;
     uint32_t oph[2] = {0, 0};
     bool ok = true;
-    while (ok && walk.next(aa, it)) {
+    while (ok && list.next(sm, it, lane, abort_flag)) {
       if (it.bad) {
         // an invalid sequence: recorded, and its output rows of this item are zero
         if (tid == 12 * 32 && it.i0 == 0 && it.h == 0) atomicOr(aa.err, kErrBadSeq);
