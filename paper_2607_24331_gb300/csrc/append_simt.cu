@@ -1,7 +1,9 @@
 // CUDA-core latent append: key and value latents of new tokens,
 //   kcache[rows[i]] = x_i A_k,  vcache[rows[i]] = x_i A_v     (Sec. III-A z = x L)
-// with fp32 accumulation; a plain 64x64-tiled GEMM.  Used for fp32 layers and
-// as the general kernel; bf16 layers take the tensor-core kernel.
+// with fp32 accumulation.  Used for fp32 layers and as the general kernel; bf16
+// layers take the tensor-core kernel.  A few tokens (a decode step's) are a
+// matrix-vector product that wants every factor byte in flight at once; many
+// are a plain 64x64-tiled GEMM.
 #include "common.cuh"
 
 namespace dck {
@@ -62,20 +64,102 @@ __global__ void __launch_bounds__(256) append_simt_kernel(const T* __restrict__ 
   }
 }
 
+// Few tokens: block (8 output columns, 8 tokens).  Bound by latency (the fp32
+// layer's factors are 0.6 MB): the 128 row lanes of a block each take every
+// 128th row of D, four rows' loads in flight together, and the sums of the
+// lanes meet in shuffles and shared memory once.
+constexpr int kVCols = 8, kVTok = 8;
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 v = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xFFFF0000u));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) append_few_kernel(const T* __restrict__ x, int n_tok, int D,
+                                                         const T* __restrict__ Ak, const T* __restrict__ Av, int Rk,
+                                                         int rv, const int64_t* __restrict__ rows, T* kc, T* vc,
+                                                         int64_t n_rows, int* err) {
+  __shared__ float red[8][kVTok][kVCols];
+  pdl_launch_dependents();
+  const int c0 = blockIdx.x * kVCols;  // R_k and r_v are multiples of 16: a block has columns of one factor
+  const bool is_k = c0 < Rk;
+  const int N = is_k ? Rk : rv, col = is_k ? c0 : c0 - Rk;
+  const int m0 = blockIdx.y * kVTok, nm = min(kVTok, n_tok - m0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kl = threadIdx.x >> 1;     // row lane
+  const T* __restrict__ A = (is_k ? Ak : Av) + col + 4 * (threadIdx.x & 1);
+  const T* __restrict__ xm = x + (int64_t)m0 * D;
+  float acc[kVTok][4] = {};
+  for (int k0 = kl; k0 < D; k0 += 4 * 128) {
+    float4 w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      w[q] = k0 + 128 * q < D ? load4(A + (int64_t)(k0 + 128 * q) * N) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < kVTok; ++m) {
+      if (m >= nm) break;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float xv = k0 + 128 * q < D ? to_f32(xm[(int64_t)m * D + k0 + 128 * q]) : 0.f;
+        acc[m][0] = fmaf(xv, w[q].x, acc[m][0]);
+        acc[m][1] = fmaf(xv, w[q].y, acc[m][1]);
+        acc[m][2] = fmaf(xv, w[q].z, acc[m][2]);
+        acc[m][3] = fmaf(xv, w[q].w, acc[m][3]);
+      }
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < kVTok; ++m) {
+    if (m >= nm) break;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+      for (int o = 16; o > 1; o >>= 1) acc[m][j] += __shfl_xor_sync(0xffffffffu, acc[m][j], o);
+      if (lane < 2) red[warp][m][4 * lane + j] = acc[m][j];
+    }
+  }
+  __syncthreads();
+  const int m = threadIdx.x / kVCols, c = threadIdx.x % kVCols;
+  if (m >= nm) return;
+  float v = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) v += red[w][m][c];
+  const int64_t row = rows[m0 + m];
+  if (row < 0 || row >= n_rows) {
+    atomicOr(err, kErrBadRow);
+    return;
+  }
+  (is_k ? kc : vc)[row * N + col + c] = from_f32<T>(v);
+}
+
+// The tile kernel's time is set by its D / 16 steps in series; the other's grows with
+// every eight tokens, for which the factors are read again from L2.  fp32 layer,
+// D = 512, tile kernel / this one: 16 tokens 103 / 16 us, 64 130 / 19, 256 119 / 41,
+// 512 115 / 72, 1024 119 / 129.
+constexpr int kFewTokens = 512;
+
+template <typename T>
+cudaError_t launch_t(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
+                     const int64_t* rows, void* kc, void* vc, int64_t n_rows, int* err, cudaStream_t s) {
+  if (n_tok <= kFewTokens)
+    append_few_kernel<T><<<dim3((Rk + rv) / kVCols, (n_tok + kVTok - 1) / kVTok), 256, 0, s>>>(
+        (const T*)x, n_tok, D, (const T*)A_k, (const T*)A_v, Rk, rv, rows, (T*)kc, (T*)vc, n_rows, err);
+  else
+    append_simt_kernel<T><<<dim3((Rk + rv + kBN - 1) / kBN, (n_tok + kBM - 1) / kBM), 256, 0, s>>>(
+        (const T*)x, n_tok, D, (const T*)A_k, (const T*)A_v, Rk, rv, rows, (T*)kc, (T*)vc, n_rows, err);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_append_simt(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
                                const int64_t* rows, void* kc, void* vc, int64_t n_rows, int dtype, int* err,
                                cudaStream_t s) {
-  dim3 grid((Rk + rv + kBN - 1) / kBN, (n_tok + kBM - 1) / kBM);
-  if (dtype == DCK_F32)
-    append_simt_kernel<float><<<grid, 256, 0, s>>>((const float*)x, n_tok, D, (const float*)A_k, (const float*)A_v,
-                                                   Rk, rv, rows, (float*)kc, (float*)vc, n_rows, err);
-  else
-    append_simt_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(
-        (const __nv_bfloat16*)x, n_tok, D, (const __nv_bfloat16*)A_k, (const __nv_bfloat16*)A_v, Rk, rv, rows,
-        (__nv_bfloat16*)kc, (__nv_bfloat16*)vc, n_rows, err);
-  return cudaGetLastError();
+  return dtype == DCK_F32
+             ? launch_t<float>(x, n_tok, D, A_k, A_v, Rk, rv, rows, kc, vc, n_rows, err, s)
+             : launch_t<__nv_bfloat16>(x, n_tok, D, A_k, A_v, Rk, rv, rows, kc, vc, n_rows, err, s);
 }
 
 }  // namespace dck

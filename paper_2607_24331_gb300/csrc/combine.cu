@@ -3,7 +3,7 @@
 // Every work item wrote, for each sequence b it touched and each query head j,
 // the un-normalised latent accumulator u = sum_t 2^(s_t - m) v_t, its reference
 // max m (log2 units) and l = sum_t 2^(s_t - m).  CUDA-core path: item c covers
-// a contiguous range of 128-token tiles and writes slot c + b.  Tensor-core
+// a contiguous range of 32-token tiles and writes slot c + b.  Tensor-core
 // path (the pair-tile plan of tc_common.cuh): each half of CTA pair p writes
 // slot 2 (p + b) + half, and each half of an extra pair tile e its own slot;
 // a slot whose half holds no token of b is not read.  For sequence b this
@@ -129,11 +129,11 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
     cp_async_commit();
   }
 
-  // tiles: pair tiles (tensor-core path) or 128-token tiles; items: CTA pairs or CTAs
+  // tiles: pair tiles (tensor-core path) or kSimtTile-token tiles; items: CTA pairs or CTAs
   const bool pairs = a.split_extra != 0;
   const int n_it = pairs ? a.n_items / 2 : a.n_items;
   // tiles per sequence (every thread a share), then an exclusive prefix by warp 0
-  const int tile = pairs ? 2 * kTile : kTile;
+  const int tile = pairs ? 2 * kTile : kSimtTile;
   for (int b = threadIdx.x; b < B; b += kThreads)
     prefix[b + 1] = (valid_len(a.seq_len, a.seq_start, b, a.n_rows) + tile - 1) / tile;
   __syncthreads();

@@ -16,6 +16,7 @@ constexpr int kMaxRankV = 2048;
 constexpr int kMaxBatch = 4096;
 constexpr int kMaxPrefillLen = 1 << 24;  // bound on a prefill call's q_max and max_seq_len
 constexpr int kTile = 128;        // tokens per work tile (one UMMA M block)
+constexpr int kSimtTile = 32;     // tokens per work tile of the CUDA-core path
 
 // Device error word values (bit flags).
 constexpr int kErrBadSeq = 1;     // a sequence's rows fall outside the cache
@@ -33,10 +34,11 @@ struct LayerTable {
   int64_t grp_boff[kMaxGroups];     // element offset of B_g in the packed B_k
 };
 
-// Work decomposition of a decode call: every sequence is cut into 128-token
-// tiles; the flattened tile list is split into n_items contiguous ranges
-// (item c: tiles [floor(c*NT/n), floor((c+1)*NT/n))).  Item c writes one
-// partial per sequence b it touches, in slot c + b.
+// Work decomposition of a decode call on the CUDA-core path: every sequence is
+// cut into kSimtTile-token tiles; the flattened tile list is split into n_items
+// contiguous ranges (item c: tiles [floor(c*NT/n), floor((c+1)*NT/n))).  Item c
+// writes one partial per sequence b it touches, in slot c + b.  (Tensor-core
+// path: the pair-tile plan of tc_common.cuh.)
 struct DecodeArgs {
   const void* q;
   const void* kc;
@@ -75,7 +77,9 @@ inline cudaError_t hook_end(LaunchHook* h, cudaStream_t s);       // after the c
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Host launchers (each defined in its own translation unit).
-cudaError_t launch_decode_simt(const LayerTable& lt, const DecodeArgs& a, int dtype, cudaStream_t s);
+int simt_items(const LayerTable& lt, int dtype, int B, int64_t n_rows, int sms);
+cudaError_t launch_decode_simt(const LayerTable& lt, const DecodeArgs& a, int dtype, bool after_append,
+                               cudaStream_t s);
 cudaError_t launch_combine(const LayerTable& lt, const DecodeArgs& a, int dtype, cudaStream_t s);
 cudaError_t launch_append_simt(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk,
                                int rv, const int64_t* rows, void* kc, void* vc, int64_t n_rows, int dtype,
@@ -106,47 +110,47 @@ template <>
 __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // Number of `tile`-token tiles of every sequence, as an exclusive prefix in
-// shared memory prefix[0..B].  Sequences whose rows fall outside the cache
-// count as empty and raise kErrBadSeq.  Must be called by the whole block.
-// Returns the total tile count NT.
+// shared memory prefix[0..B] (scratch: one int per warp).  Sequences whose rows
+// fall outside the cache count as empty and raise kErrBadSeq.  Must be called
+// by the whole block (full warps).  Returns the total tile count NT.
 __device__ __forceinline__ int build_tile_prefix(const int32_t* __restrict__ seq_len,
                                                  const int64_t* __restrict__ seq_start, int B,
                                                  int64_t n_rows, int* prefix, int* scratch, int* err,
-                                                 bool report, int tile = kTile) {
-  const int nt = blockDim.x;
-  const int per = (B + nt - 1) / nt;
-  const int b0 = threadIdx.x * per;
-  int local = 0;
-  for (int b = b0; b < b0 + per && b < B; ++b) {
-    int64_t L = seq_len[b];
-    int64_t st = seq_start[b];
-    if (L < 0 || st < 0 || st + L > n_rows) {
-      if (report) atomicOr(err, kErrBadSeq);
-      L = 0;
+                                                 bool report, int tile) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  int base = 0;
+  for (int c0 = 0; c0 < B; c0 += blockDim.x) {  // a sequence per thread
+    const int b = c0 + (int)threadIdx.x;
+    int n = 0;
+    if (b < B) {
+      int64_t L = seq_len[b];
+      const int64_t st = seq_start[b];
+      if (L < 0 || st < 0 || st + L > n_rows) {
+        if (report) atomicOr(err, kErrBadSeq);
+        L = 0;
+      }
+      n = (int)((L + tile - 1) / tile);
     }
-    local += (int)((L + tile - 1) / tile);
-  }
-  scratch[threadIdx.x] = local;
-  __syncthreads();
-  // Hillis-Steele inclusive scan over the per-thread sums
-  for (int off = 1; off < nt; off <<= 1) {
-    int v = threadIdx.x >= off ? scratch[threadIdx.x - off] : 0;
+    int v = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += y;
+    }
+    if (lane == 31) scratch[warp] = v;
     __syncthreads();
-    scratch[threadIdx.x] += v;
+    int before = base, all = base;
+    for (int w = 0; w < nw; ++w) {
+      if (w < warp) before += scratch[w];
+      all += scratch[w];
+    }
+    if (b < B) prefix[b] = before + v - n;
+    base = all;
     __syncthreads();
   }
-  int run = threadIdx.x ? scratch[threadIdx.x - 1] : 0;
-  for (int b = b0; b < b0 + per && b < B; ++b) {
-    prefix[b] = run;
-    int64_t L = seq_len[b];
-    int64_t st = seq_start[b];
-    if (L < 0 || st < 0 || st + L > n_rows) L = 0;
-    run += (int)((L + tile - 1) / tile);
-  }
-  int total = scratch[nt - 1];
-  if (threadIdx.x == 0) prefix[B] = total;
+  if (threadIdx.x == 0) prefix[B] = base;
   __syncthreads();
-  return total;
+  return base;
 }
 
 // Length of sequence b as used by the kernels (0 when its rows are invalid).

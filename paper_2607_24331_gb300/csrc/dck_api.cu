@@ -125,7 +125,7 @@ LayerTable make_table(const dck_layer_desc* d) {
   return lt;
 }
 
-// Partial slots: CUDA-core path, c + b for work item c (one per SM) and
+// Partial slots: CUDA-core path, c + b for work item c (at most one per SM) and
 // sequence b it touched; tensor-core path, two per (CTA pair, sequence) and two
 // per extra pair tile (tc::pair_slot_count, at most SMs / 2 pairs).  The
 // workspace holds the larger count, so one size query serves both paths.
@@ -257,11 +257,12 @@ dck_status dck_prefill_attention(const dck_layer_desc* desc, const void* q, cons
 namespace {
 // The decode call, optionally with the decode step's latent append fused into
 // its first launch (app != nullptr: the caller has checked that the fused
-// append applies).
+// append applies).  after_append: the stream's last kernel is this library's
+// latent append, put there by the same call.
 dck_status decode_call(const dck_layer_desc* desc, const void* q, const void* kcache, const void* vcache,
                        int64_t n_rows, const void* B_k, const void* B_v, const int64_t* d_seq_start,
                        const int32_t* d_seq_len, int32_t batch, float rope_theta, void* out, void* workspace,
-                       size_t ws_bytes, const TcStepAppend* app, void* stream) {
+                       size_t ws_bytes, const TcStepAppend* app, bool after_append, void* stream) {
   t_last_launches = 0;
   const dck_status st =
       decode_precheck(desc, q, kcache, vcache, n_rows, B_k, B_v, d_seq_start, d_seq_len, batch, rope_theta, out);
@@ -305,9 +306,10 @@ dck_status decode_call(const dck_layer_desc* desc, const void* q, const void* kc
   hook.n_ev = t_n_events;
   a.hook = &hook;
   a.split_extra = use_tc ? 1 : 0;
-  if (use_tc) a.n_items = 2 * pairs;  // the tensor-core kernels run on the pairs' SMs
+  // the tensor-core kernels run on the pairs' SMs
+  a.n_items = use_tc ? 2 * pairs : simt_items(lt, desc->dtype, batch, n_rows, sms);
   if (use_tc) e = launch_decode_tc(lt, a, app, s);
-  else e = launch_decode_simt(lt, a, desc->dtype, s);
+  else e = launch_decode_simt(lt, a, desc->dtype, after_append, s);
   if (e != cudaSuccess) return DCK_ERR_CUDA;
   e = launch_combine(lt, a, desc->dtype, s);
   if (e == cudaSuccess) e = hook_end(&hook, s);
@@ -334,7 +336,7 @@ dck_status dck_decode_attention(const dck_layer_desc* desc, const void* q, const
                                 const int32_t* d_seq_len, int32_t batch, float rope_theta, void* out,
                                 void* workspace, size_t ws_bytes, void* stream) {
   return decode_call(desc, q, kcache, vcache, n_rows, B_k, B_v, d_seq_start, d_seq_len, batch, rope_theta, out,
-                     workspace, ws_bytes, nullptr, stream);
+                     workspace, ws_bytes, nullptr, false, stream);
 }
 
 size_t dck_decode_step_workspace_size(const dck_layer_desc* desc, int32_t batch, int64_t n_rows) {
@@ -363,7 +365,7 @@ dck_status dck_decode_step(const dck_layer_desc* desc, const void* x, const void
     app.rows = d_rows;
     app.D = desc->hidden;
     return decode_call(desc, q, kcache, vcache, n_rows, B_k, B_v, d_seq_start, d_seq_len, batch, rope_theta, out,
-                       workspace, ws_bytes, &app, stream);
+                       workspace, ws_bytes, &app, false, stream);
   }
   // separate append, then the decode call (the append's scratch after the decode workspace)
   const size_t dw = align_up(dck_decode_workspace_size(desc, batch, n_rows), 256);
@@ -372,8 +374,8 @@ dck_status dck_decode_step(const dck_layer_desc* desc, const void* x, const void
                                    static_cast<char*>(workspace) + dw, ws_bytes - dw, stream);
   if (r != DCK_OK) return r;
   const int appended = t_last_launches;
-  r = dck_decode_attention(desc, q, kcache, vcache, n_rows, B_k, B_v, d_seq_start, d_seq_len, batch, rope_theta,
-                           out, workspace, dw, stream);
+  r = decode_call(desc, q, kcache, vcache, n_rows, B_k, B_v, d_seq_start, d_seq_len, batch, rope_theta, out,
+                  workspace, dw, nullptr, true, stream);
   t_last_launches += appended;
   return r;
 }

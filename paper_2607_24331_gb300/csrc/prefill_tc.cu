@@ -26,6 +26,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "rope.cuh"
 #include "tc_common.cuh"
 #include "tmap.h"
 
@@ -38,42 +39,6 @@ using namespace tc;
 
 constexpr int kPD = 128;               // head dim of the tensor-core prefill
 constexpr int kMaxGroupsP = 16;
-
-// ---------------------------------------------------------------------------
-// RoPE angles in turns
-// ---------------------------------------------------------------------------
-
-// Frequency w_i / (2 pi) as a 64-bit binary fraction: position t turns pair i
-// by the fraction t * f (mod 2^64), exactly, so an angle needs two integer
-// multiplies and no fp64, and its reduction mod 2 pi is the wrap-around.
-struct RopeFreqs {
-  uint2 f[kPD / 2];  // {low, high} words
-};
-
-// sin and cos of 2 pi u / 2^32.  The nearest quarter turn is taken off exactly
-// in integers; the remainder, within +-pi/4, goes through the Taylor series of
-// sine (to x^9) and cosine (to x^10), whose truncation errors there (1.8e-9
-// and 1.2e-10) are below fp32 rounding.
-__device__ __forceinline__ void turn_sincos(uint32_t u, float& sn, float& cs) {
-  const uint32_t q = (u + 0x20000000u) >> 30;
-  const float x = (float)(int32_t)(u - (q << 30)) * 1.4629180792671596e-9f;  // 2 pi / 2^32
-  const float x2 = x * x;
-  float s = fmaf(x2, 2.7557319e-6f, -1.9841270e-4f);
-  s = fmaf(x2, s, 8.3333333e-3f);
-  s = fmaf(x2, s, -1.6666667e-1f);
-  s = fmaf(x * x2, s, x);
-  float c = fmaf(x2, -2.7557319e-7f, 2.4801587e-5f);
-  c = fmaf(x2, c, -1.3888889e-3f);
-  c = fmaf(x2, c, 4.1666667e-2f);
-  c = fmaf(x2, c, -0.5f);
-  c = fmaf(x2, c, 1.f);
-  const float a = (q & 1) ? c : s, b = (q & 1) ? s : c;
-  sn = __uint_as_float(__float_as_uint(a) ^ ((q & 2) << 30));
-  cs = __uint_as_float(__float_as_uint(b) ^ (((q + 1) & 2) << 30));
-}
-__device__ __forceinline__ void rope_sincos(uint2 f, uint32_t pos, float& sn, float& cs) {
-  turn_sincos(__umulhi(pos, f.x) + pos * f.y, sn, cs);
-}
 
 // ---------------------------------------------------------------------------
 // 1. reconstruction
@@ -1032,12 +997,7 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
       key[n_key++] = RCol{(int16_t)g, (int16_t)(sl * kPD), (int16_t)(nh * kPD), (int16_t)head_at[g][sl],
                           (int16_t)(nh == 2 ? head_at[g][sl + 1] : 0), lt.grp_rank[g]};
     }
-  for (int i = 0; i < kPD / 2; ++i) {
-    const double turns = std::exp2(-2.0 * i / kPD * std::log2((double)theta)) * 0.15915494309189533577;
-    const double fr = turns - std::floor(turns);  // a whole number of turns per position is none
-    const uint64_t f = (uint64_t)std::ldexp(fr, 64);
-    ra.rf.f[i] = make_uint2((uint32_t)f, (uint32_t)(f >> 32));
-  }
+  ra.rf = rope_freqs_of(theta, kPD);
   ra.qscale = 1.4426950408889634f / std::sqrt((float)kPD);
   ra.kw = kw;
   ra.vw = vw;

@@ -1,0 +1,79 @@
+"""The CUDA-core decode kernel and the few-token append at the edges of their
+tiles, against the fp64 oracle: sequences cut at 32 tokens, more sequences than
+a block has threads, both head dims, one and several query heads per KV head,
+the smallest and the largest group rank, value ranks past one column per
+thread, hidden widths that no lane count divides.
+
+Decode bound: max|o - o_ref| / ||o_ref||_inf <= 1e-5 (fp32) or 2e-2 (bf16
+outputs).  Append bound per element: u |c| + K 2^-23 sum_k |x_k a_k|.
+"""
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2607_24331_gb300 import dck, device
+from paper_2607_24331_gb300 import synth as S
+from gpu_util import assert_parity, gpu_decode, oracle_decode
+from test_step_gpu import _step
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(hq, groups, ranks, rv, d, dtype="f32", hidden=200):
+    hkv = sum(len(g) for g in groups)
+    return S.LayerSpec(hidden, hq, hkv, d, groups, ranks, rv, dtype, 1e4)
+
+
+LAYERS = {
+    "mha64": _layer(3, ((2,), (0, 1)), (16, 96), 160, 64),
+    "mha128": _layer(2, ((1,), (0,)), (256, 48), 272, 128),
+    "gqa4-64": _layer(8, ((1, 0),), (32,), 528, 64),
+    "gqa8-128": _layer(8, ((0,),), (256,), 48, 128),
+    "mha128-bf16": _layer(2, ((1, 0),), (112,), 288, 128, "bf16"),
+    "gqa2-64-bf16": _layer(4, ((1,), (0,)), (16, 48), 32, 64, "bf16"),
+}
+
+
+@pytest.mark.parametrize("name", list(LAYERS))
+@pytest.mark.parametrize("lens", [(1, 31, 32, 33, 0, 65, 500), (3000,)], ids=["edges", "long"])
+def test_decode_tiles(name, lens):
+    spec = LAYERS[name]
+    got, di = gpu_decode(spec, lens, seed=4, kernel=1)
+    live = [b for b, n in enumerate(lens) if n]  # the oracle takes no empty sequence: its output is zero
+    ref = oracle_decode(di, batch_ids=live)
+    assert_parity(got[live], ref[live], spec.dtype, f"{name} {lens}")
+    assert all((got[b] == 0).all() for b, n in enumerate(lens) if not n)
+
+
+def test_many_sequences():
+    spec = LAYERS["mha64"]
+    lens = tuple(1 + (7 * i) % 70 for i in range(300))
+    got, di = gpu_decode(spec, lens, seed=5, kernel=1)
+    assert_parity(got, oracle_decode(di), "f32", "300 sequences")
+
+
+@pytest.mark.parametrize("lens", [(1,), (33, 400, 64), tuple(range(1, 70))], ids=["one", "three", "many"])
+def test_step_fp32(lens):
+    _step(S.workload(0).layer, lens, seed=6)
+
+
+@pytest.mark.parametrize("hidden", [1, 127, 130, 512, 1100])
+@pytest.mark.parametrize("n_tok", [1, 8, 9, 512, 513])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_append_few(dtype, n_tok, hidden):
+    # (a bf16 layer whose rank sums the tensor-core append does not take goes the same way)
+    spec = _layer(2, ((1,), (0,)), (16, 32), 16, 64, dtype, hidden)
+    x, A_k, A_v = S.make_append_inputs(spec, n_tok, seed=hidden)
+    rows = np.random.default_rng(n_tok).choice(n_tok + 5, size=n_tok, replace=False)
+    buf = device.AppendBuffers(spec, n_tok, n_tok + 5).load_host(x, A_k, A_v, rows)
+    dck.check(buf.run(), "dck_latent_append")
+    torch.cuda.synchronize()
+    assert dck.dck_last_device_error() == dck.DCK_OK
+    u = 2.0 ** -8 if dtype == "bf16" else 2.0 ** -23
+    for got, ref, A in zip((buf.kcache, buf.vcache), oracle.latent_append(x, A_k, A_v), (A_k, A_v)):
+        got = got.float().cpu().numpy().astype(np.float64)
+        bound = u * np.abs(ref) + hidden * 2.0 ** -23 * (np.abs(x.astype(np.float64)) @ np.abs(A.astype(np.float64)))
+        assert (np.abs(got[rows] - ref) <= bound).all()
+        assert (got[np.setdiff1d(np.arange(n_tok + 5), rows)] == 0).all()
