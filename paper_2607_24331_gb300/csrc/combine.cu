@@ -286,16 +286,18 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll 4
     for (int k0 = 0; k0 < rr; k0 += 8) {
+      const bool hi = k0 + 8 <= rr;  // r_v slices of 4 mod 8 rows: the last step has rows k0 .. k0 + 3 only
       uint32_t af[4];
       af[0] = f32_to_tf32(su[(size_t)gid * ldu + k0 + tig]);
       af[1] = f32_to_tf32(su[(size_t)(gid + 8) * ldu + k0 + tig]);
-      af[2] = f32_to_tf32(su[(size_t)gid * ldu + k0 + tig + 4]);
-      af[3] = f32_to_tf32(su[(size_t)(gid + 8) * ldu + k0 + tig + 4]);
+      af[2] = hi ? f32_to_tf32(su[(size_t)gid * ldu + k0 + tig + 4]) : 0u;
+      af[3] = hi ? f32_to_tf32(su[(size_t)(gid + 8) * ldu + k0 + tig + 4]) : 0u;
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt) {
         const int col = 16 * warp + 8 * nt + gid;
         const uint32_t b0 = (uint32_t)__bfloat16_as_ushort(sbv[(size_t)(k0 + tig) * ldb<T, D>() + col]) << 16;
-        const uint32_t b1 = (uint32_t)__bfloat16_as_ushort(sbv[(size_t)(k0 + tig + 4) * ldb<T, D>() + col]) << 16;
+        const uint32_t b1 =
+            hi ? (uint32_t)__bfloat16_as_ushort(sbv[(size_t)(k0 + tig + 4) * ldb<T, D>() + col]) << 16 : 0u;
         mma_tf32(acc[nt], af, b0, b1);
       }
     }

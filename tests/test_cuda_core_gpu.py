@@ -31,7 +31,7 @@ LAYERS = {
     "mha128": _layer(2, ((1,), (0,)), (256, 48), 272, 128),
     "gqa4-64": _layer(8, ((1, 0),), (32,), 528, 64),
     "gqa8-128": _layer(8, ((0,),), (256,), 48, 128),
-    "mha128-bf16": _layer(2, ((1, 0),), (112,), 288, 128, "bf16"),
+    "mha128-bf16": _layer(2, ((1, 0),), (112,), 272, 128, "bf16"),
     "gqa2-64-bf16": _layer(4, ((1,), (0,)), (16, 48), 32, 64, "bf16"),
 }
 
