@@ -44,24 +44,30 @@
 // P) are written as the segment's split partial.  The absorption kernel
 // (absorb_tc.cu) forms U = C_v^T P from them.
 //
-// Warp roles (384 threads query-folded, 352 key mode), in both CTAs unless
-// noted.  Every TMA instruction costs its issuing thread a long round trip, so
-// loads are issued by two producer warps, each putting several copies (one per
-// lane) into one instruction; the copies of both CTAs complete on the even
-// CTA's barriers, which its MMA threads wait on:
+// Warp roles (640 threads), in both CTAs unless noted; the copies of both CTAs
+// complete on the even CTA's barriers, which its MMA warps wait on:
 //   warp 0     latent pieces of C_g (ring A)
-//   warp 10    factor items (ring W; query-folded mode: one ring per MMA thread)
-//   warp 1     TMEM owner; in the even CTA its lane 0 issues pair MMAs.  On this
-//              GPU every barrier test, commit or fence costs the issuing thread a
-//              dependent round trip of 100-500 cycles, so in query-folded mode
-//              lane 0 of the even CTA's warp 11 issues every other unit into the
-//              other accumulator and the two threads' bookkeeping overlaps the
-//              other's MMAs; the MMA commits arrive on both CTAs' barriers
-//   warps 2-9  epilogue: each TMEM lane quadrant (32 tokens) is served by two
-//              warps that split the 64 RoPE frequency pairs of a head; their
-//              partial scores go to one shared-memory array per frequency
-//              half, summed at the tile end.  Both CTAs' epilogues release an
+//   warp 2     factor items (ring W)
+//   warp 1     TMEM owner; in the even CTA it issues pair MMAs (in query-folded
+//              mode every other unit, warp 3 the others into the other
+//              accumulator, so that one warp's waits and commits overlap the
+//              other's MMAs); the MMA commits arrive on both CTAs' barriers
+//   warps 4-19 epilogue: each TMEM lane quadrant (32 tokens) is served by four
+//              warps, each with 16 of the 64 RoPE frequency pairs of every head;
+//              their partial scores go to one shared-memory array per frequency
+//              quarter, summed at the tile end.  Both CTAs' epilogues release an
 //              accumulator on the even CTA's barrier.
+// What bounds it: the chain of one accumulator (MMAs, commit, epilogue reads,
+// release; all of TMEM is two 256-column accumulators) and the epilogue's work
+// per unit, about 1.3 k cycles each against 1.1 k of MMAs on the 32-head MHA layer
+// (clock64 timelines).  With eight epilogue warps of 32 frequencies each, whose
+// loads, arithmetic and hand-offs ran in series, a unit took 2.2 k (query-folded)
+// and 3.0 k (key mode); key mode's keys went through shared memory to reach the
+// score MMA's operand layout, which the 16x256b TMEM load gives directly.  The
+// rings hand out single pieces and items: with whole units, a second unit of
+// three items did not fit and its load came after the first one's MMAs.
+// Whole calls, before / now: 32-head MHA 16 x 4096 169.5 / 147.6 us, 32 ragged
+// 367 / 321; GQA 8 x 32768 251 / 228, 2 x 131072 286 / 222.
 // Every wait is bounded (about 2 s); on expiry the CTA stops issuing work,
 // tells its peer to stop, records kErrTimeout, waits for work in flight and
 // still releases TMEM.
@@ -80,6 +86,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "rope.cuh"
 #include "tc_common.cuh"
 #include "tc_host.h"
 #include "tmap.h"
@@ -98,8 +105,11 @@ constexpr int kMaxPieces = 5;
 constexpr int kMaxHqTc = 32;
 constexpr int kMaxItems = 256;
 constexpr int kMaxUnits = 32;
-constexpr int kEpiThreads = 256;
-constexpr int kEpiWarps = kEpiThreads / 32;
+constexpr int kCtlWarps = 4;      // producers and MMA issuers
+constexpr int kEpiWarps = 16;
+constexpr int kEpiThreads = 32 * kEpiWarps;
+constexpr int kThreadsTc = 32 * kCtlWarps + kEpiThreads;
+constexpr int kFreqW = kD / 2 / 4;  // RoPE pairs of a frequency quarter
 // Latent tiles prefetched toward L2 ahead of their loads: two in query-folded
 // mode; none in key mode, whose TMA loads keep enough of the latent stream in
 // flight themselves and whose prefetches only competed with it (7B GQA layer,
@@ -109,23 +119,27 @@ __host__ __device__ constexpr int prefetch_ahead() { return kFold ? 2 : 0; }
 constexpr float kRescaleThr = 8.f;  // log2 units: probabilities stay <= 256
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kKCols = 256;    // TMEM columns of one key accumulator
-constexpr float kTwoPi = 6.28318530717958647692f;
-constexpr float kInvTwoPi = 0.15915494309189533577f;
+constexpr float kTurn32 = 1.4629180792671596e-9f;  // 2 pi / 2^32
 constexpr float kLog2e = 1.4426950408889634f;
+
+// Full barriers of the factor ring.  An MMA warp passes over the other's items
+// without waiting for them, so it may wait for an item whose slot still awaits an
+// earlier fill: with a barrier per slot it would take an older phase for that
+// item's.  With 16, the item 16 earlier is complete whenever a warp waits: its own
+// last item is at most 10 back (units of up to 5 items), and an item is loaded
+// only once the one NW <= 5 before it has been read.
+constexpr int kItemBars = 16;
 
 template <bool kFold>
 struct Ring {
   // latent-piece slots (16 KB each) and factor-item slots (half items, 16 KB
-  // each).  The latent ring holds the group in use while the next group's
-  // pieces arrive from HBM; key mode's B_g items are few and L2-resident, so
-  // five of its slots go to the latents (measured on the 7B GQA layer: 4/6
-  // latent/factor slots 233 us, 5/5 200 us, 6/4 204 us, 8/2 225 us)
+  // each): what the scores leave of shared memory.  The latent ring holds the
+  // group in use while the next group's pieces arrive from HBM.
   static constexpr int NA = 5;
-  static constexpr int NW = kFold ? 6 : 5;
-  // MMA-issuing threads: two in query-folded mode; key mode's units carry up
-  // to four items, which one thread streams better
+  static constexpr int NW = kFold ? 5 : 4;
+  // MMA-issuing warps: two in query-folded mode; key mode's units carry up
+  // to four items, which one warp streams better
   static constexpr int kMma = kFold ? 2 : 1;
-  static constexpr int kThreads = kFold ? 384 : 352;
 };
 
 // Latent-piece maps (box 64/32/16 ranks x 128 tokens, 128/64/32B swizzle) and
@@ -160,10 +174,10 @@ struct TcArgs {
   uint8_t* pglob;                // per-tile P images (workspace)
   float* mglob;                  // per-tile reference maxima (workspace)
   int64_t max_tiles;
-  double om[kD / 2];             // RoPE frequencies theta^(-2i/d), fp64
+  RopeFreqs rf;                  // RoPE frequencies theta^(-2i/d) in turns
   GroupSm grp[kMaxGroupsTc];
-  int16_t order[kMaxHqTc];       // KV head at each MMA position (group-major, slot order)
   int n_units;                   // units per tile
+  uint32_t uinfo[kMaxUnits];     // KV heads of each unit: first | second << 8 | count << 16
   int16_t uitem[kMaxUnits + 1];  // first factor item of each unit (and the item count)
   int8_t hunit[kMaxHqTc];        // unit of each query head
   uint32_t item[kMaxItems];      // factor item n: byte offset | (bytes / 4096) << 26
@@ -173,44 +187,28 @@ template <bool kFold>
 struct Smem {
   uint8_t a[Ring<kFold>::NA][kSlot];
   uint8_t w[Ring<kFold>::NW][kSlotW];
-  // scores [frequency half][query head][token]: each half's partial scores by
-  // plain stores, summed at the tile end
-  float x[2 * kMaxHqTc * 128];
+  // scores [frequency quarter][query head][token]: each quarter's partial
+  // scores by plain stores, summed at the tile end
+  float x[4 * kMaxHqTc * 128];
   // key mode: rotated queries * log2(e)/sqrt(d), bf16 [query head][d] (the
-  // B operand of the warps' score MMAs), and per epilogue warp a staging tile
-  // of its 32 tokens' rotated keys [token][32] bf16 (the A operand), 16-byte
-  // chunks swizzled by (token / 2) % 4
+  // B operand of the warps' score MMAs)
   __nv_bfloat16 qr[kFold ? 2 : kMaxHqTc * kD];
-  uint8_t kst[kFold ? 1 : kEpiWarps][kFold ? 16 : 32 * 64];
-  double om64[kD / 2];
-  float om32[kD / 2];
-  float beta[kD / 2];
-  float qcs[kFold ? 1 : kD / 2], qsn[kFold ? 1 : kD / 2];  // key mode: RoPE of the query position
-  // latent ring: one full/empty pair per group instance; factor rings: one
-  // pair per unit (batch of items) of each MMA thread (see SlotFifo)
-  uint64_t g_full[kFifoBars], g_empty[kFifoBars];
-  uint64_t u_full[kFifoBars], u_empty[kFifoBars];
-  uint64_t k_full[2], k_empty[2], epi_bar;
+  uint2 freq[kD / 2];
+  uint64_t a_full[Ring<kFold>::NA], a_empty[Ring<kFold>::NA];  // latent pieces
+  uint64_t w_full[kItemBars], w_empty[Ring<kFold>::NW];        // factor items (full: item % kItemBars; empty: slot)
+  uint64_t k_full[2], k_empty[2], epi_bar, x_free;
   GroupSm grp[kMaxGroupsTc];
-  int16_t order[kMaxHqTc];
-  int16_t uitem[kMaxUnits + 1];
+  uint32_t uinfo[kMaxUnits];
+  PairWalker walk[2];  // main and extra pair tiles of this pair
   int8_t hunit[kMaxHqTc];
   uint32_t tmem_base;
   int abort_flag;
 };
 
-__device__ __forceinline__ uint32_t swz_of(int w) { return w == 64 ? kSw128 : (w == 32 ? kSw64 : kSw32); }
-
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-  return (uint32_t)__bfloat16_as_ushort(h.x) | ((uint32_t)__bfloat16_as_ushort(h.y) << 16);
-}
-// Four 8x8 b16 matrices from shared memory; lane i gives the row address of row
-// i % 8 of matrix i / 8.
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
 }
 // d += a b for one 16 x 8 x 16 tile, bf16 inputs, fp32 accumulators.
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -230,11 +228,11 @@ __device__ __forceinline__ int im_map_of(uint32_t half_rows) {
 // ---------------------------------------------------------------------------
 
 template <bool kFold>
-__global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
+__global__ void __launch_bounds__(kThreadsTc, 1)
     decode_tc_kernel(const __grid_constant__ Maps maps, const LayerTable lt, const DecodeArgs a,
                      const __grid_constant__ TcArgs ta) {
   constexpr int kMma = Ring<kFold>::kMma, NW = Ring<kFold>::NW, kNA = Ring<kFold>::NA;
-  constexpr int kThreads = Ring<kFold>::kThreads;
+  constexpr int kThreads = kThreadsTc;
   extern __shared__ uint8_t smem_raw[];
   Smem<kFold>& sm =
       *reinterpret_cast<Smem<kFold>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -248,17 +246,18 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
 
   // ---- setup -------------------------------------------------------------
   if (tid == 0) {
-    for (int i = 0; i < kFifoBars; ++i) {
-      mbar_init(&sm.g_full[i], 1);      // even CTA: its producer's expect_tx; both CTAs' copies complete on it
-      mbar_init(&sm.g_empty[i], kMma);  // released by every MMA thread (arrivals reach both CTAs)
-      mbar_init(&sm.u_full[i], 1);
-      mbar_init(&sm.u_empty[i], 1);
+    for (int i = 0; i < kNA; ++i) {
+      mbar_init(&sm.a_full[i], 1);      // even CTA: its producer's expect_tx; both CTAs' copies complete on it
+      mbar_init(&sm.a_empty[i], kMma);  // released by every MMA warp (arrivals reach both CTAs)
     }
+    for (int i = 0; i < NW; ++i) mbar_init(&sm.w_empty[i], 1);
+    for (int i = 0; i < kItemBars; ++i) mbar_init(&sm.w_full[i], 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sm.k_full[i], 1);
       mbar_init(&sm.k_empty[i], 2 * kEpiWarps);  // even CTA: both CTAs' epilogue warps
     }
     mbar_init(&sm.epi_bar, kEpiWarps);
+    mbar_init(&sm.x_free, kEpiWarps);
     sm.abort_flag = 0;
     fence_mbar_init();
   }
@@ -267,13 +266,9 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
     tmem_relinquish_pair();
   }
   if (tid < lt.G) sm.grp[tid] = ta.grp[tid];
-  if (tid < lt.Hkv) sm.order[tid] = ta.order[tid];
-  if (tid <= ta.n_units) sm.uitem[tid] = ta.uitem[tid];
+  if (tid < ta.n_units) sm.uinfo[tid] = ta.uinfo[tid];
   if (tid < Hq) sm.hunit[tid] = ta.hunit[tid];
-  if (tid < kD / 2) {
-    sm.om64[tid] = ta.om[tid];
-    sm.om32[tid] = (float)ta.om[tid];
-  }
+  if (tid < kD / 2) sm.freq[tid] = ta.rf.f[tid];
   // Work of this pair: main pair tiles [X0, X1) (every unit), then units
   // [u_lo, u_hi) of the flattened (extra tile, unit) list, every extra tile a
   // segment of its own.
@@ -294,8 +289,14 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
   const int u_lo = fits ? (int)((int64_t)pair * xu / P) : 0;
   const int u_hi = fits ? (int)((int64_t)(pair + 1) * xu / P) : 0;
   const int xe0 = sp.NPm + (u_lo < u_hi ? u_lo / U : 0), xe1 = sp.NPm + (u_lo < u_hi ? (u_hi - 1) / U + 1 : 0);
-  const PairWalker walk_m = pair_walker_at(a, s256, s128, X0, X1, false);
-  const PairWalker walk_x = pair_walker_at(a, s256, s128, xe0, xe1, true);
+  {
+    const PairWalker wm = pair_walker_at(a, s256, s128, X0, X1, false);
+    const PairWalker wx = pair_walker_at(a, s256, s128, xe0, xe1, true);
+    if (tid == 0) {
+      sm.walk[0] = wm;
+      sm.walk[1] = wx;
+    }
+  }
   const bool has_work = X0 < X1 || xe0 < xe1;  // the same in both CTAs of the pair
   // units [ua, ub) of flattened pair tile X in phase ph (0: main, 1: extra)
   auto units_of = [&](int ph, int X, int& ua, int& ub) {
@@ -307,7 +308,6 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
       ub = min(u_hi - e * U, U);
     }
   };
-  for (int i = tid; i < (int)(sizeof(sm.x) / sizeof(float)); i += kThreads) sm.x[i] = 0.f;
   tc_fence_before();
   cluster_sync();  // both CTAs' barriers initialised and TMEM allocated
   tc_fence_after();
@@ -319,35 +319,6 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
   auto stop_peer = [&]() { st_cluster_u32(peer(&sm.abort_flag), 1u); };
   PSegment seg;
 
-  // Half items (this CTA's head, or its half of a lone head) of one unit into
-  // the factor ring, in batches of at most NW items: each batch is one
-  // instance of the ring (one full barrier, which the even CTA's lane 0 arms
-  // with the bytes of both CTAs' copies; one TMA copy per lane).  The units of
-  // both MMA threads share the ring, in unit order.
-  auto put_unit = [&](SlotFifo& f, int n, int np, int64_t img_row0, uint64_t pol) -> bool {
-    for (int p0 = 0; p0 < np;) {
-      const int nb = min(NW, np - p0);
-      if (!f.claim(nb, NW, sm.u_empty, lane, abort_flag)) return false;
-      uint64_t* full = &sm.u_full[f.inst % kFifoBars];
-      if (leader && lane == 0) {
-        uint32_t total = 0;
-        for (int q = 0; q < nb; ++q) total += (ta.item[n + p0 + q] >> 26) << 12;
-        mbar_expect_tx(full, total);
-      }
-      __syncwarp();
-      if (lane < nb) {
-        const int sl = (f.head + lane) % NW;
-        const uint32_t it = ta.item[n + p0 + lane];
-        const uint32_t hrows = ((it >> 26) << 12) / 256;
-        const int64_t y = img_row0 + ((it & 0x03FFFFFFu) >> 7) + hr * hrows;
-        tma_load_2d_pair(sm.w[sl], &maps.im[im_map_of(hrows)], lead(full), 0, (int32_t)y, pol);
-      }
-      __syncwarp();
-      f.advance(nb);
-      p0 += nb;
-    }
-    return true;
-  };
   const int64_t img_seq_rows = ta.fimg_seq_bytes >> 7;
   // Programmatic dependent launch: every thread lets the absorption kernel
   // launch only after it has seen the preparation kernel complete, so that
@@ -361,26 +332,26 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
 
   if (warp == 0) {
     // ---- latent pieces (this CTA's 128 rows of each), issued as soon as their
-    // slots are free; in query-folded mode also the factor items of MMA thread
-    // 1, in the order that thread consumes them (a group's pieces, then its
-    // units' items) ---------------------------------------------------------
+    // slots are free ---------------------------------------------------------
     if (has_work) {
       const uint64_t pol = policy_evict_first();
-      SlotFifo ga;  // the latent ring
+      const bool el = elect_one();
+      int slot = 0, fills = 0;  // latent ring: next slot, times round
       bool ok = true;
       // L2 prefetch of this half's latent rows, prefetch_ahead() tiles ahead of the
       // loads (across segment boundaries): the TMA loads then find them in L2
-      PairWalker pwalk[2] = {walk_m, walk_x};
-      PSegment pseg;
+      PairWalker pwalk = sm.walk[0];
+      PSegment pseg = {};
       int pph = 0, pti = 0;
-      bool pvalid = false;
       auto prefetch_next = [&]() {
         if (lane != 0) return;
-        while (!pvalid || pti >= pseg.ntiles) {
-          while (pph < 2 && !pwalk[pph].next(a, pseg)) ++pph;
-          if (pph >= 2) return;
-          pvalid = true;
+        while (pti >= pseg.ntiles) {
           pti = 0;
+          if (pph >= 2) return;
+          if (!pwalk.next(a, pseg)) {
+            pseg.ntiles = 0;
+            if (++pph < 2) pwalk = sm.walk[pph];
+          }
         }
         const int64_t r0 = pseg.row0 + pseg.t0(pti++, hr);
         const int64_t nr = a.n_rows - r0 < kTile ? a.n_rows - r0 : (int64_t)kTile;
@@ -390,8 +361,7 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
       griddep_wait();  // the preparation launch may append the step's own latents
       griddep_launch();
       for (int ph = 0; ph < 2 && ok; ++ph)
-        for (PairWalker walk = ph ? walk_x : walk_m; ok && walk.next(a, seg);) {
-          const int64_t img_row0 = kFold ? (int64_t)seg.b * img_seq_rows : 0;
+        for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             const int64_t yrow = seg.row0 + seg.t0(i, hr);
             prefetch_next();
@@ -399,22 +369,20 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
             units_of(ph, seg.X0 + i, ua, ub);
             for (int g = 0; g < lt.G && ok; ++g) {
               const GroupSm& gs = sm.grp[g];
-              const int np = gs.np;
-              const int lo = max(ua - gs.u0, 0), hi = min(ub - gs.u0, (int)gs.nu);
-              if (lo >= hi) continue;  // none of the group's units in this piece of work
-              // the group's pieces: one instance of the latent ring
-              if (!(ok = ga.claim(np, kNA, sm.g_empty, lane, abort_flag))) break;
-              uint64_t* gfull = &sm.g_full[ga.inst % kFifoBars];
-              if (leader && lane == 0) mbar_expect_tx(gfull, 2 * kTile * 2 * gs.rank);
-              __syncwarp();
-              if (lane < np) {
-                const int sl = (ga.head + lane) % kNA;
-                const int w = gs.w[lane];
-                const CUtensorMap* m = w == 64 ? &maps.kc64 : (w == 32 ? &maps.kc32 : &maps.kc16);
-                tma_load_2d_pair(sm.a[sl], m, lead(gfull), gs.roff + gs.k[lane], (int32_t)yrow, pol);
+              if (max(ua - gs.u0, 0) >= min(ub - gs.u0, (int)gs.nu)) continue;  // none of the group's units here
+              for (int p = 0; p < gs.np; ++p) {
+                if (fills && !(ok = wwait(&sm.a_empty[slot], (fills - 1) & 1, abort_flag))) break;
+                if (el) {
+                  const int w = gs.w[p];
+                  if (leader) mbar_expect_tx(&sm.a_full[slot], 2 * kTile * 2 * w);
+                  const CUtensorMap* m = w == 64 ? &maps.kc64 : (w == 32 ? &maps.kc32 : &maps.kc16);
+                  tma_load_2d_pair(sm.a[slot], m, lead(&sm.a_full[slot]), gs.roff + gs.k[p], (int32_t)yrow, pol);
+                }
+                if (++slot == kNA) {
+                  slot = 0;
+                  ++fills;
+                }
               }
-              __syncwarp();
-              ga.advance(np);
             }
           }
         }
@@ -423,47 +391,66 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
       griddep_wait();
       griddep_launch();
     }
-  } else if (warp == 10) {
-    // ---- factor items: several TMA copies per instruction (query-folded
-    // mode: the ring of MMA thread 0 only) --------------------------------------
+  } else if (warp == 2) {
+    // ---- factor items: this CTA's head of each (or its half of a lone head's),
+    // one slot and one pair of barriers each, so that a unit's first MMAs start
+    // when its first item is there and a slot refills as soon as it is read -----
     if (has_work) {
       const uint64_t pol = policy_evict_last();
-      SlotFifo fw;         // the factor ring
+      const bool el = elect_one();
+      int slot = 0, fills = 0, pos = 0;  // factor ring: next slot, times round, items so far
       bool ok = true;
       for (int ph = 0; ph < 2 && ok; ++ph)
-        for (PairWalker walk = ph ? walk_x : walk_m; ok && walk.next(a, seg);) {
+        for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
           const int64_t img_row0 = kFold ? (int64_t)seg.b * img_seq_rows : 0;
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             int ua, ub;
             units_of(ph, seg.X0 + i, ua, ub);
-            for (int g = 0; g < lt.G && ok; ++g) {
-              const GroupSm& gs = sm.grp[g];
-              const int np = gs.np;
-              const int lo = max(ua - gs.u0, 0), hi = min(ub - gs.u0, (int)gs.nu);
-              for (int u = lo; u < hi && ok; ++u) ok = put_unit(fw, gs.i0 + u * np, np, img_row0, pol);
+            const int n1 = ta.uitem[ub];
+            for (int n = ta.uitem[ua]; n < n1; ++n) {
+              if (fills && !(ok = wwait(&sm.w_empty[slot], (fills - 1) & 1, abort_flag))) break;
+              if (el) {
+                const uint32_t it = ta.item[n];
+                const uint32_t hrows = ((it >> 26) << 12) / 256;
+                uint64_t* full = &sm.w_full[pos % kItemBars];
+                if (leader) mbar_expect_tx(full, (it >> 26) << 12);
+                const int64_t y = img_row0 + ((it & 0x03FFFFFFu) >> 7) + hr * hrows;
+                tma_load_2d_pair(sm.w[slot], &maps.im[im_map_of(hrows)], lead(full), 0, (int32_t)y, pol);
+              }
+              ++pos;
+              if (++slot == NW) {
+                slot = 0;
+                ++fills;
+              }
             }
           }
         }
       if (!ok && lane == 0) stop_peer();
     }
-  } else if (warp == 1 || (kMma == 2 && warp == 11)) {
-    // ---- MMA issuers (even CTA only): lane 0 of warp 1 (and of warp 11 in
-    // query-folded mode) runs the schedule of every kMma-th unit into its own
-    // accumulator, so one thread's barrier waits and commits overlap the
-    // other's MMAs.  Each thread owns a factor ring (single consumer).  Per
-    // unit: one wait for its items, one for its accumulator, its MMAs, one
-    // commit for the items and one for the accumulator; per key group one
-    // wait for all its latent pieces and one release (commit, or arrivals in
-    // both CTAs when the thread has no unit in the group, after the fill so
-    // that no barrier phase is passed early). ---------------------------------
-    if (leader && lane == 0 && has_work) {
+  } else if (warp == 1 || (kMma == 2 && warp == 3)) {
+    // ---- MMA issuers (even CTA only): warp 1 (and warp 3 in query-folded mode)
+    // runs the schedule of every kMma-th unit into its own accumulator, so one
+    // warp's barrier waits and commits overlap the other's MMAs.  The whole warp
+    // runs it and an elected lane issues (see elect_one), with descriptors as a
+    // base per piece width plus a slot and a constant per k-step.  Per item: a
+    // wait for it, its MMAs and the commit that frees its slot; per unit a wait
+    // for the accumulator and its commit; per key group and warp a wait for each
+    // latent piece and its release (commit, or arrivals in both CTAs when the warp
+    // has no unit in the group, after the fill so that no barrier phase is passed
+    // early). --------------------------------------------------------------------
+    if (leader && has_work) {
+      const bool el = elect_one();
       const int t = warp == 1 ? 0 : 1;
-      int gi = 0, ghead = 0;  // latent-ring instances (groups) and slots handed out so far
-      int ui = 0, uhead = 0;  // factor-ring instances (item batches of every unit) and slots
-      int kc = 0, own = 0;    // units of the pair so far, units in this thread's accumulator
+      const uint32_t sa0 = smem_u32(sm.a[0]), sw0 = smem_u32(sm.w[0]);
+      const uint64_t da64 = sdesc(sa0, 16, 16 * 64, kSw128), dw64 = sdesc(sw0, 128 * 64, 1024, kSw128);
+      const uint64_t da32 = sdesc(sa0, 16, 16 * 32, kSw64), dw32 = sdesc(sw0, 128 * 32, 1024, kSw128);
+      const uint64_t da16 = sdesc(sa0, 16, 16 * 16, kSw32), dw16 = sdesc(sw0, 128 * 16, 1024, kSw128);
+      int as = 0, aph = 0;  // latent ring: slot and phase of the next group's first piece
+      int ws = 0, pos = 0;  // factor ring: slot and number of the next unit's first item
+      int kc = 0, own = 0;  // units of the pair so far, units in this warp's accumulator
       bool ok = true;
       for (int ph = 0; ph < 2 && ok; ++ph)
-        for (PairWalker walk = ph ? walk_x : walk_m; ok && walk.next(a, seg);) {
+        for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             int ua, ub;
             units_of(ph, seg.X0 + i, ua, ub);
@@ -472,77 +459,93 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
               const int np = gs.np;
               const int lo = max(ua - gs.u0, 0), hi = min(ub - gs.u0, (int)gs.nu);  // the group's units here
               if (lo >= hi) continue;
-              const int gb = gi % kFifoBars;
-              const uint32_t gpar = (gi / kFifoBars) & 1;
-              const int uf = lo + (kMma == 2 ? (((kc & 1) == t) ? 0 : 1) : 0);  // this thread's first unit of the group
-              // all the group's latent pieces (both CTAs' rows) are there
-              if (!(ok = mbar_wait(&sm.g_full[gb], gpar, abort_flag))) break;
-              if (uf >= hi) {  // no unit of this thread in the group: release its pieces in both CTAs
-                mbar_arrive(&sm.g_empty[gb]);
-                mbar_arrive_cluster(peer(&sm.g_empty[gb]));
-              }
-              for (int u = lo; u < hi && ok; ++u) {
-                if (u < uf || (u - uf) % kMma != 0) {  // the other thread's unit: skip its item batches
-                  ui += (np + NW - 1) / NW;
-                  uhead += np;
-                  continue;
-                }
-                const int nh = min(2, gs.nh - 2 * u);
-                const uint32_t idesc_k = idesc_bf16(256, kD * nh, false, true);
-                const int kg = kc + (u - lo);                        // unit index of the pair
-                const int buf = kMma == 2 ? t : (kg & 1);
-                const int use = kMma == 2 ? own : (kg >> 1);         // earlier units in this accumulator
-                const uint32_t dcol = tmem + buf * kKCols;
-                for (int p0 = 0; p0 < np && ok;) {  // the unit's item batches (ring instances)
-                  const int nb = min(NW, np - p0);
-                  const int ub_ = ui % kFifoBars;
-                  if (!(ok = mbar_wait(&sm.u_full[ub_], (ui / kFifoBars) & 1, abort_flag))) break;
-                  if (p0 == 0 && use >= 1) {  // both CTAs' epilogues have read this accumulator's previous unit
-                    if (!(ok = mbar_wait(&sm.k_empty[buf], (use - 1) & 1, abort_flag))) break;
+              const int uf = lo + (kMma == 2 ? (((kc & 1) == t) ? 0 : 1) : 0);  // this warp's first unit of the group
+              if (uf >= hi) {  // no unit of this warp in the group: release its pieces in both CTAs
+                for (int p = 0, sl = as, sp_ = aph; p < np; ++p) {
+                  if (!(ok = wwait(&sm.a_full[sl], sp_, abort_flag))) break;
+                  if (el) {
+                    mbar_arrive(&sm.a_empty[sl]);
+                    mbar_arrive_cluster(peer(&sm.a_empty[sl]));
                   }
-                  tc_fence_after();
-                  for (int q = 0; q < nb; ++q) {
-                    const int p = p0 + q;
-                    const int w = gs.w[p];
-                    const uint32_t ab0 = smem_u32(sm.a[(ghead + p) % kNA]);
-                    const uint32_t bb = smem_u32(sm.w[(uhead + q) % NW]);
-                    const uint32_t swz = swz_of(w);
-                    for (int k = 0; k < w / 16; ++k) {
-                      const uint64_t ad = sdesc(ab0 + k * 32, 16, 16 * w, swz);
-                      const uint64_t bd = sdesc(bb + k * 2048, 128 * w, 1024, kSw128);
-                      umma_f16_pair(dcol, ad, bd, idesc_k, (p > 0 || k > 0) ? 1u : 0u);
-                    }
+                  if (++sl == kNA) {
+                    sl = 0;
+                    sp_ ^= 1;
                   }
-                  umma_commit_pair(&sm.u_empty[ub_]);  // the batch's slots, once its MMAs are done
-                  ++ui;
-                  uhead += nb;
-                  p0 += nb;
                 }
                 if (!ok) break;
-                umma_commit_pair(&sm.k_full[buf]);
-                if (u + kMma >= hi) umma_commit_pair(&sm.g_empty[gb]);  // this thread is done with the pieces
+              }
+              for (int u = lo; u < hi; ++u) {
+                if (kMma == 2 && ((u - uf) & 1)) {  // the other warp's unit: skip its items
+                  ws = ws + np >= NW ? ws + np - NW : ws + np;
+                  pos += np;
+                  continue;
+                }
+                const uint32_t idesc_k = 2 * u + 1 < gs.nh ? idesc_bf16(256, 2 * kD, false, true)
+                                                           : idesc_bf16(256, kD, false, true);
+                const int kg = kc + (u - lo);                 // unit index of the pair
+                const int buf = kMma == 2 ? t : (kg & 1);
+                const int use = kMma == 2 ? own : (kg >> 1);  // earlier units in this accumulator
+                const uint32_t dcol = tmem + buf * kKCols;
+                const bool first = u == uf, last = u + kMma >= hi;  // of this warp's units in the group
+                for (int p = 0, sl = as, sp_ = aph; p < np; ++p) {
+                  if (!(ok = wwait(&sm.w_full[pos % kItemBars], (pos / kItemBars) & 1, abort_flag))) break;
+                  ++pos;
+                  if (first && !(ok = wwait(&sm.a_full[sl], sp_, abort_flag))) break;
+                  // both CTAs' epilogues have read this accumulator's previous unit
+                  if (p == 0 && use >= 1 && !(ok = wwait(&sm.k_empty[buf], (use - 1) & 1, abort_flag))) break;
+                  tc_fence_after();
+                  const int w = gs.w[p];
+                  const uint64_t ao = (uint64_t)(sl * (kSlot >> 4)), wo = (uint64_t)(ws * (kSlotW >> 4));
+                  if (el) {
+                    const uint32_t acc = p > 0 ? 1u : 0u;
+                    if (w == 64) {
+#pragma unroll
+                      for (int k = 0; k < 4; ++k)
+                        umma_f16_pair(dcol, da64 + ao + 2 * k, dw64 + wo + 128 * k, idesc_k, k ? 1u : acc);
+                    } else if (w == 32) {
+#pragma unroll
+                      for (int k = 0; k < 2; ++k)
+                        umma_f16_pair(dcol, da32 + ao + 2 * k, dw32 + wo + 128 * k, idesc_k, k ? 1u : acc);
+                    } else {
+                      umma_f16_pair(dcol, da16 + ao, dw16 + wo, idesc_k, acc);
+                    }
+                    umma_commit_pair(&sm.w_empty[ws]);
+                    if (last) umma_commit_pair(&sm.a_empty[sl]);
+                  }
+                  ws = ws + 1 == NW ? 0 : ws + 1;
+                  if (++sl == kNA) {
+                    sl = 0;
+                    sp_ ^= 1;
+                  }
+                }
+                if (!ok) break;
+                if (el) umma_commit_pair(&sm.k_full[buf]);
                 ++own;
               }
-              ++gi;
-              ghead += np;
+              as += np;
+              if (as >= kNA) {
+                as -= kNA;
+                aph ^= 1;
+              }
               kc += hi - lo;
             }
           }
         }
-      if (!ok) stop_peer();
+      if (!ok && lane == 0) stop_peer();
     }
     __syncwarp();
-  } else if (warp >= 2 && warp <= 9) {
+  } else if (warp >= kCtlWarps) {
     // ---- epilogue: RoPE, scores, softmax, P of this CTA's 128-token halves ----
-    const int e = tid - 64;              // 0 .. 255
-    const int quad = warp & 3;           // TMEM lane quadrant
-    const int hf = (warp - 2) >> 2;      // frequency half, then head half
-    const int tau = quad * 32 + lane;    // token row inside the half tile
+    const int e = tid - 32 * kCtlWarps;            // 0 .. 511
+    const int quad = warp & 3;                     // TMEM lane quadrant
+    const int fq = (warp - kCtlWarps) >> 2;        // frequency quarter: pairs [16 fq, 16 fq + 16)
+    const int gid = lane >> 2, tig = lane & 3;     // key mode: rows and columns of the 16 x 256-bit fragments
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-    // tile and segment ends: thread e owns head jt and the 16 tokens [16 ct, 16 ct + 16)
-    // of every half tile; the 8 owners of a head are adjacent lanes of one warp
-    const int jt = e >> 3, ct = e & 7;
-    int kc = 0, round = 0;
+    float* const xq = sm.x + fq * (kMaxHqTc * 128);  // this quarter's scores
+    // tile and segment ends: thread e owns head jt and the 8 tokens [8 ct, 8 ct + 8)
+    // of every half tile; the 16 owners of a head are adjacent lanes of one warp
+    const int jt = e >> 4, ct = e & 15;
+    int kc = 0, round = 0, tiles = 0;
     bool ok = true;
 #define EPI_SYNC()                                  \
   do {                                              \
@@ -561,36 +564,24 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
       }
     };
     for (int ph = 0; ph < 2 && ok; ++ph)
-      for (PairWalker walk = ph ? walk_x : walk_m; ok && walk.next(a, seg);) {
+      for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
         if (!kFold) {
           // rotated queries of this sequence at position L-1, scaled to log2 units
-          // (the 64 angles reduced mod 2 pi in fp64 once, sine and cosine in fp32;
-          // every query head uses them)
-          if (e < kD / 2) {
-            const double ang = (double)(seg.L - 1) * sm.om64[e];
-            sincosf((float)(ang - 6.283185307179586 * rint(ang * 0.15915494309189535)), &sm.qsn[e], &sm.qcs[e]);
-          }
-          EPI_SYNC();
-          if (!ok) break;
+          // (its last tile's scores have been formed: that tile's EPI_SYNC)
           const float qscale = kLog2e * rsqrtf((float)kD);
           const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(a.q) + (int64_t)seg.b * Hq * kD;
-          for (int i = e; i < Hq * (kD / 2); i += kEpiThreads) {
-            const int j = i / (kD / 2), pi = i % (kD / 2);
-            const float sn = sm.qsn[pi], cs = sm.qcs[pi];
+          const int pi = e & (kD / 2 - 1);
+          float sn, cs;
+          rope_sincos(sm.freq[pi], (uint32_t)(seg.L - 1), sn, cs);
+          for (int j = e >> 6; j < Hq; j += kEpiThreads / (kD / 2)) {
             const float x1v = __bfloat162float(qb[j * kD + pi]), x2v = __bfloat162float(qb[j * kD + pi + kD / 2]);
             sm.qr[j * kD + pi] = __float2bfloat16_rn((x1v * cs - x2v * sn) * qscale);
             sm.qr[j * kD + pi + kD / 2] = __float2bfloat16_rn((x1v * sn + x2v * cs) * qscale);
           }
+          EPI_SYNC();
+          if (!ok) break;
         }
-        // RoPE angle of token t0+tau and pair p: (t0*w_p mod 2pi, fp64) + tau*w_p (fp32);
-        // the offsets beta of later tiles are written at the previous tile's end
-        if (e < kD / 2) {
-          const double ang = (double)seg.t0(0, hr) * sm.om64[e];
-          sm.beta[e] = (float)(ang - 6.283185307179586 * floor(ang * 0.15915494309189535));
-        }
-        EPI_SYNC();
-        if (!ok) break;
-        // head jt's reference max (log2 units; the same in all 8 owners) and this
+        // head jt's reference max (log2 units; the same in all 16 owners) and this
         // owner's share of its row sum, rescaled whenever the reference moves
         float m_run = -INFINITY, l_part = 0.f;
         int ua = 0, ub = 0;  // units of the current tile
@@ -599,121 +590,94 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
           const bool has = seg.has(i, hr);    // this half holds tokens of the sequence
           const int64_t x = seg.x128(i, hr);  // its flattened 128-token tile (when it has)
           units_of(ph, seg.X0 + i, ua, ub);
-          float cs[32], sn[32];
+          // sines and cosines of this thread's accumulator elements: query-folded
+          // mode, token `lane` of the quadrant at the quarter's 16 frequencies; key
+          // mode, tokens gid + 8 k (k < 4) at frequencies 8 j + 2 tig + c (index 4 k + 2 j + c)
+          float cs[kFreqW], sn[kFreqW];
 #pragma unroll
-          for (int ip = 0; ip < 32; ++ip) {
-            const int pi = 32 * hf + ip;
-            float phs = fmaf((float)tau, sm.om32[pi], sm.beta[pi]);
-            phs = fmaf(-kTwoPi, rintf(phs * kInvTwoPi), phs);
-            __sincosf(phs, &sn[ip], &cs[ip]);
+          for (int ip = 0; ip < kFreqW; ++ip) {
+            const int fi = kFreqW * fq + (kFold ? ip : 8 * ((ip >> 1) & 1) + 2 * tig + (ip & 1));
+            const uint32_t pos = (uint32_t)(t0 + quad * 32 + (kFold ? lane : gid + 8 * (ip >> 2)));
+            const uint2 f = sm.freq[fi];
+            const float ang = (float)(int32_t)(__umulhi(pos, f.x) + pos * f.y) * kTurn32;
+            __sincosf(ang, &sn[ip], &cs[ip]);
           }
-          // per unit (one or two KV heads), in MMA order: partial scores of this frequency half
-          for (int g = 0; g < lt.G && ok; ++g) {
-            const GroupSm& gs = sm.grp[g];
-            const int lo = max(ua - gs.u0, 0), hi = min(ub - gs.u0, (int)gs.nu);
-            for (int u = lo; u < hi; ++u) {
-              const int nh = min(2, gs.nh - 2 * u);
-              const int buf = kc & 1;
-              if (!(ok = wwait(&sm.k_full[buf], (kc >> 1) & 1, abort_flag))) break;
-              tc_fence_after();
-              if (kFold) {
-                // Y columns [64 hf, 64 hf + 64) of both heads: pairs (2i, 2i+1) of my 32
-                // frequencies, in two passes of 16 pairs; each pass loads both heads
-                // before its one wait, so a unit costs two TMEM round trips
-                const uint32_t cb = tmem + lane_base + buf * kKCols + 64 * hf;
-                float pa[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};  // independent chains
+          if (tiles >= 1 && !(ok = wwait(&sm.x_free, (tiles - 1) & 1, abort_flag))) break;  // the last tile's scores
+          ++tiles;                                                                          // have been read
+          // per unit (one or two KV heads), in MMA order: partial scores of this frequency quarter
+          for (int u = ua; u < ub; ++u) {
+            const uint32_t ui = sm.uinfo[u];
+            const int h0 = ui & 0xFF, h1 = (ui >> 8) & 0xFF;
+            const bool two = (ui >> 17) != 0;
+            const int buf = kc & 1;
+            if (!(ok = wwait(&sm.k_full[buf], (kc >> 1) & 1, abort_flag))) break;
+            tc_fence_after();
+            if (kFold) {
+              // Y columns [32 fq, 32 fq + 32) of both heads: pairs (2i, 2i+1) of the 16 frequencies
+              const uint32_t cb = tmem + lane_base + buf * kKCols + 2 * kFreqW * fq;
 #pragma unroll
-                for (int ps = 0; ps < 2; ++ps) {
-                  float y0[32], y1[32];
-                  tmem_ld32(cb + 32 * ps, y0);
-                  if (nh == 2) tmem_ld32(cb + kD + 32 * ps, y1);
-                  tmem_wait_ld();
-                  if (ps == 1) release_acc(buf);
+              for (int hh = 0; hh < 2; ++hh) {
+                if (hh == 1 && !two) break;
+                float y[32];
+                tmem_ld32(cb + hh * kD, y);
+                tmem_wait_ld();
+                if (hh == 1 || !two) release_acc(buf);
+                float pa[4] = {0.f, 0.f, 0.f, 0.f};  // independent chains
 #pragma unroll
-                  for (int i2 = 0; i2 < 16; ++i2)
-                    pa[0][i2 & 3] =
-                        fmaf(cs[16 * ps + i2], y0[2 * i2], fmaf(sn[16 * ps + i2], y0[2 * i2 + 1], pa[0][i2 & 3]));
-                  if (nh == 2)
+                for (int i2 = 0; i2 < kFreqW; ++i2)
+                  pa[i2 & 3] = fmaf(cs[i2], y[2 * i2], fmaf(sn[i2], y[2 * i2 + 1], pa[i2 & 3]));
+                xq[(hh ? h1 : h0) * 128 + quad * 32 + lane] = (pa[0] + pa[1]) + (pa[2] + pa[3]);
+              }
+            } else {
+              // per head: the key's 16 frequency pairs of this quarter, read from TMEM
+              // in the layout of the score MMA's A operand (m16n8k16: rows the warp's
+              // 32 tokens in two m-tiles, k the 16 x-halves, then the 16 y-halves, n the
+              // query heads padded to 8), rotated and rounded to bf16 in place
 #pragma unroll
-                    for (int i2 = 0; i2 < 16; ++i2)
-                      pa[1][i2 & 3] =
-                          fmaf(cs[16 * ps + i2], y1[2 * i2], fmaf(sn[16 * ps + i2], y1[2 * i2 + 1], pa[1][i2 & 3]));
+              for (int hh = 0; hh < 2; ++hh) {
+                if (hh == 1 && !two) break;
+                const int j0 = (hh ? h1 : h0) * qpg;
+                const uint32_t cb = tmem + lane_base + buf * kKCols + hh * kD + kFreqW * fq;
+                float xv[2][8], yv[2][8];
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                  tmem_ld_16x256b_x2(cb + ((uint32_t)(16 * mt) << 16), xv[mt]);
+                  tmem_ld_16x256b_x2(cb + kD / 2 + ((uint32_t)(16 * mt) << 16), yv[mt]);
                 }
-                float* xh = sm.x + hf * (kMaxHqTc * 128);  // this frequency half's scores
-                xh[sm.order[gs.h0 + 2 * u] * 128 + tau] = (pa[0][0] + pa[0][1]) + (pa[0][2] + pa[0][3]);
-                if (nh == 2)
-                  xh[sm.order[gs.h0 + 2 * u + 1] * 128 + tau] = (pa[1][0] + pa[1][1]) + (pa[1][2] + pa[1][3]);
-              } else {
-                // per head: rotate the key's 32 frequency pairs of this half (two
-                // passes of 16), stage them as bf16, and form the scores of the
-                // head's qpg query heads with mma m16n8k16 (rows: the warp's 32
-                // tokens in two m-tiles; k: 16 rotated x-halves, then 16 y-halves
-                // per pass; n: query heads, padded to 8)
-                const int gid = lane >> 2, tig = lane & 3;
-                uint8_t* st = sm.kst[warp - 2];
-                const uint32_t st_addr = smem_u32(st);
-                for (int hh = 0; hh < nh; ++hh) {
-                  const int j0 = sm.order[gs.h0 + 2 * u + hh] * qpg;
-                  const uint32_t cb = tmem + lane_base + buf * kKCols + hh * kD;
-                  const bool last = hh == nh - 1;
-                  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+                // B operand: query head n = gid (zero past qpg), k = 2 tig .. and 2 tig + 8 ..
+                uint32_t bq[2][2] = {{0u, 0u}, {0u, 0u}};
+                if (gid < qpg) {
+                  const __nv_bfloat16* qrow = sm.qr + (j0 + gid) * kD + kFreqW * fq + 2 * tig;
 #pragma unroll
-                  for (int ps = 0; ps < 2; ++ps) {
-                    float k1v[16], k2v[16];
-                    tmem_ld16(cb + 32 * hf + 16 * ps, k1v);
-                    tmem_ld16(cb + 64 + 32 * hf + 16 * ps, k2v);
-                    tmem_wait_ld();
-                    if (last && ps == 1) release_acc(buf);
-                    // this lane's token: rotated x-halves (chunks 0, 1) and y-halves (2, 3)
-                    uint32_t rw[16];
+                  for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
-                    for (int w = 0; w < 8; ++w) {
-                      const int ip = 16 * ps + 2 * w;
-                      const float a0 = fmaf(k1v[2 * w], cs[ip], -k2v[2 * w] * sn[ip]);
-                      const float a1 = fmaf(k1v[2 * w + 1], cs[ip + 1], -k2v[2 * w + 1] * sn[ip + 1]);
-                      const float b0 = fmaf(k1v[2 * w], sn[ip], k2v[2 * w] * cs[ip]);
-                      const float b1 = fmaf(k1v[2 * w + 1], sn[ip + 1], k2v[2 * w + 1] * cs[ip + 1]);
-                      rw[w] = pack_bf16x2(a0, a1);
-                      rw[8 + w] = pack_bf16x2(b0, b1);
-                    }
-                    __syncwarp();  // the previous pass's fragments have been read
+                    for (int j = 0; j < 2; ++j) bq[ks][j] = *reinterpret_cast<const uint32_t*>(qrow + 64 * ks + 8 * j);
+                }
+                tmem_wait_ld();
+                if (hh == 1 || !two) release_acc(buf);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                      *reinterpret_cast<uint4*>(st + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) =
-                          make_uint4(rw[4 * c], rw[4 * c + 1], rw[4 * c + 2], rw[4 * c + 3]);
-                    __syncwarp();
+                for (int mt = 0; mt < 2; ++mt) {
+                  uint32_t ax[4], ay[4];
 #pragma unroll
-                    for (int ks = 0; ks < 2; ++ks) {  // x-halves, then y-halves
-                      // B: query head n = gid (zero past qpg), k = 2 tig .. and 2 tig + 8 ..
-                      uint32_t bq0 = 0u, bq1 = 0u;
-                      if (gid < qpg) {
-                        const __nv_bfloat16* qrow = sm.qr + (j0 + gid) * kD + 64 * ks + 32 * hf + 16 * ps;
-                        bq0 = *reinterpret_cast<const uint32_t*>(qrow + 2 * tig);
-                        bq1 = *reinterpret_cast<const uint32_t*>(qrow + 2 * tig + 8);
-                      }
-#pragma unroll
-                      for (int mt = 0; mt < 2; ++mt) {
-                        // A: tokens 16 mt .. +15, k chunks 2 ks and 2 ks + 1 of the staged rows
-                        const int r = 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1), ch = 2 * ks + (lane >> 4);
-                        uint32_t af[4];
-                        ldmatrix_x4(af, st_addr + r * 64 + ((ch ^ ((r >> 1) & 3)) << 4));
-                        mma_bf16_16816(acc[mt], af, bq0, bq1);
-                      }
-                    }
+                  for (int r = 0; r < 4; ++r) {  // rows gid + 8 (r & 1), frequencies 8 (r >> 1) + 2 tig, + 1
+                    const int vi = 4 * (r >> 1) + 2 * (r & 1), ci = 4 * (2 * mt + (r & 1)) + 2 * (r >> 1);
+                    const float x0 = xv[mt][vi], x1 = xv[mt][vi + 1], y0 = yv[mt][vi], y1 = yv[mt][vi + 1];
+                    ax[r] = pack_bf16x2(fmaf(x0, cs[ci], -y0 * sn[ci]), fmaf(x1, cs[ci + 1], -y1 * sn[ci + 1]));
+                    ay[r] = pack_bf16x2(fmaf(x0, sn[ci], y0 * cs[ci]), fmaf(x1, sn[ci + 1], y1 * cs[ci + 1]));
                   }
+                  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                  mma_bf16_16816(acc, ax, bq[0][0], bq[0][1]);
+                  mma_bf16_16816(acc, ay, bq[1][0], bq[1][1]);
                   // scores: token (16 mt + gid [+ 8]) of this quadrant, query heads 2 tig, 2 tig + 1
-                  float* xh = sm.x + hf * (kMaxHqTc * 128);  // this frequency half's scores
 #pragma unroll
-                  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                      const int jj = 2 * tig + (q & 1), tt = quad * 32 + 16 * mt + gid + 8 * (q >> 1);
-                      if (jj < qpg) xh[(j0 + jj) * 128 + tt] = acc[mt][q];
-                    }
+                  for (int q = 0; q < 4; ++q) {
+                    const int jj = 2 * tig + (q & 1), tt = quad * 32 + 16 * mt + gid + 8 * (q >> 1);
+                    if (jj < qpg) xq[(j0 + jj) * 128 + tt] = acc[q];
+                  }
                 }
               }
-              ++kc;
             }
+            ++kc;
           }
           if (!ok) break;
           // ---- tile end: reference max, P ------------------------------------
@@ -721,32 +685,34 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
           if (!ok) break;
           {
             const bool own = jt < Hq && sm.hunit[jt] >= ua && sm.hunit[jt] < ub;  // head computed here
-            const int tb = 16 * ct;  // first token of this owner
-            float sc[16];
+            const int tb = 8 * ct;  // first token of this owner
+            float sc[8];
             const float4* xr = reinterpret_cast<const float4*>(&sm.x[jt * 128 + tb]);
-            const float4* xr2 = reinterpret_cast<const float4*>(&sm.x[kMaxHqTc * 128 + jt * 128 + tb]);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float4 v = own ? xr[q] : make_float4(0.f, 0.f, 0.f, 0.f);
-              if (own) {  // plus the other frequency half (every score is stored each tile)
-                const float4 w = xr2[q];
-                v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+            for (int q = 0; q < 2; ++q) {  // the sum of the four frequency quarters (every score is stored each tile)
+              float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (own) {
+                const float4 w0 = xr[q], w1 = xr[kMaxHqTc * 32 + q], w2 = xr[2 * kMaxHqTc * 32 + q],
+                             w3 = xr[3 * kMaxHqTc * 32 + q];
+                v = make_float4((w0.x + w1.x) + (w2.x + w3.x), (w0.y + w1.y) + (w2.y + w3.y),
+                                (w0.z + w1.z) + (w2.z + w3.z), (w0.w + w1.w) + (w2.w + w3.w));
               }
               sc[4 * q] = v.x;
               sc[4 * q + 1] = v.y;
               sc[4 * q + 2] = v.z;
               sc[4 * q + 3] = v.w;
             }
-            const int nv = max(0, min(16, seg.L - (t0 + tb)));  // tokens inside the sequence
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.x_free);  // the next tile's scores may be stored
+            const int nv = max(0, min(8, seg.L - (t0 + tb)));  // tokens inside the sequence
             float mx = -INFINITY;
 #pragma unroll
-            for (int k = 0; k < 16; ++k) {
+            for (int k = 0; k < 8; ++k) {
               if (k >= nv || !own) sc[k] = -INFINITY;
               mx = fmaxf(mx, sc[k]);
             }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
             // the reference moves only when the tile's max exceeds it by the threshold
             if (own && (m_run == -INFINITY || mx > m_run + kRescaleThr)) {
               l_part *= exp2f(m_run - mx);
@@ -755,9 +721,9 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
             if (has && own && ct == 0) ta.mglob[x * Hq + jt] = m_run;
             // probabilities (bf16, the absorption's operand) straight into this tile's
             // P image; the row sum uses the rounded values
-            uint32_t pk[8];
+            uint32_t pk[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < 4; ++k) {
               const __nv_bfloat162 pv = __floats2bfloat162_rn(own ? ex2_approx(sc[2 * k] - m_run) : 0.f,
                                                               own ? ex2_approx(sc[2 * k + 1] - m_run) : 0.f);
               const float2 pf = __bfloat1622float2(pv);
@@ -768,23 +734,14 @@ __global__ void __launch_bounds__(Ring<kFold>::kThreads, 1)
               // image: [token atom (64)][head row][64 tokens], 128B rows, 16-byte chunks swizzled by row % 8
               uint8_t* img = ta.pglob + x * (hq_pad * 256) + (tb >> 6) * (hq_pad * 128) + (jt >> 3) * 1024 +
                              (jt & 7) * 128;
-              const int ch = (tb & 63) >> 3;
-              *reinterpret_cast<uint4*>(img + ((ch ^ (jt & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-              *reinterpret_cast<uint4*>(img + (((ch + 1) ^ (jt & 7)) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+              *reinterpret_cast<uint4*>(img + (((ct & 7) ^ (jt & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             }
           }
-          if (e < kD / 2 && i + 1 < seg.ntiles) {  // RoPE phase offsets of the next pair tile
-            const double ang = (double)(t0 + kPTile) * sm.om64[e];
-            sm.beta[e] = (float)(ang - 6.283185307179586 * floor(ang * 0.15915494309189535));
-          }
-          EPI_SYNC();  // x is clear and the next tile's phase offsets are in place
-          if (!ok) break;
         }
         if (!ok) break;
         // ---- segment end: reference max and row sum -> this half's partial slot ----
-        l_part += __shfl_xor_sync(0xffffffffu, l_part, 1);
-        l_part += __shfl_xor_sync(0xffffffffu, l_part, 2);
-        l_part += __shfl_xor_sync(0xffffffffu, l_part, 4);
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) l_part += __shfl_xor_sync(0xffffffffu, l_part, o);
         if (jt < Hq && ct == 0 && sm.hunit[jt] >= ua && sm.hunit[jt] < ub) {
           const int64_t slot = ph ? pair_xslot(P, a.B, seg.X0 - sp.NPm, hr) : pair_slot(pair, seg.b, hr);
           a.part_ml[(slot * Hq + jt) * 2] = m_run;
@@ -1123,8 +1080,9 @@ bool build_maps(const LayerTable& lt, const DecodeArgs& a, const void* img, int6
   return true;
 }
 
-static_assert(sizeof(Smem<true>) + 1024 <= 232448, "shared memory of the query-folded kernel");
-static_assert(sizeof(Smem<false>) + 1024 <= 232448, "shared memory of the key-mode kernel");
+static_assert(kMaxPieces <= Ring<true>::NW && Ring<true>::NW <= 5 && kMaxPieces <= 5, "see kItemBars");
+static_assert(sizeof(Smem<true>) + 1024 + 384 <= 232448, "shared memory of the query-folded kernel");
+static_assert(sizeof(Smem<false>) + 1024 + 384 <= 232448, "shared memory of the key-mode kernel");
 
 template <bool kFold>
 cudaError_t set_smem_attr() {
@@ -1152,7 +1110,7 @@ int pairs_of_device() {
   if (set_smem_attr<kFold>() != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * (sms / 2));
-  cfg.blockDim = dim3(Ring<kFold>::kThreads);
+  cfg.blockDim = dim3(kThreadsTc);
   cfg.dynamicSmemBytes = sizeof(Smem<kFold>) + 1024;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1188,7 +1146,7 @@ cudaError_t launch_mode(const LayerTable& lt, const DecodeArgs& a, const Maps& m
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * ta.n_pairs);
-  cfg.blockDim = dim3(Ring<kFold>::kThreads);
+  cfg.blockDim = dim3(kThreadsTc);
   cfg.dynamicSmemBytes = sizeof(Smem<kFold>) + 1024;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -1231,6 +1189,7 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
   if (lt.G > kMaxGroupsTc) return false;
   int gorder[kMaxGroupsTc];
   group_order(lt, gorder);
+  int order[kMaxHqTc];  // KV head at each MMA position (group-major, slot order)
   int pos = 0, item = 0, off = 0, unit = 0;
   for (int gi = 0; gi < lt.G; ++gi) {
     const int g = gorder[gi];
@@ -1250,13 +1209,14 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
       for (int h = 0; h < lt.Hkv; ++h)
         if (lt.head_group[h] == g && lt.head_slot[h] == sl) {
           if (pos >= kMaxHqTc) return false;
-          ta.order[pos++] = (int16_t)h;
+          order[pos++] = h;
           for (int jj = 0; jj < lt.qpg; ++jj) ta.hunit[h * lt.qpg + jj] = (int8_t)(unit + sl / 2);
         }
     for (int s0 = 0; s0 < lt.grp_nh[g]; s0 += 2) {
       const int nh = std::min(2, lt.grp_nh[g] - s0);
       if (unit >= kMaxUnits) return false;
-      ta.uitem[unit++] = (int16_t)item;
+      ta.uitem[unit] = (int16_t)item;
+      ta.uinfo[unit++] = (uint32_t)(order[gs.h0 + s0] | (nh == 2 ? order[gs.h0 + s0 + 1] << 8 : 0) | nh << 16);
       for (int p = 0; p < gs.np; ++p) {
         if (item >= kMaxItems) return false;
         const int w = gs.w[p], bytes = nh * w * 256;
@@ -1351,8 +1311,8 @@ cudaError_t launch_decode_tc(const LayerTable& lt, const DecodeArgs& a, const Tc
     pa.app.D = app->D;
     pa.app.n_blocks = (lt.Rk + lt.rv) / kAppCols;
   }
-  rope_freqs(a.theta, ta.om);
-  std::memcpy(pa.om, ta.om, sizeof(ta.om));
+  ta.rf = rope_freqs_of(a.theta, kD);
+  rope_freqs(a.theta, pa.om);
   const ExtraLayout xl = extra_layout(lt, a.B, a.n_rows);
   uint8_t* base = static_cast<uint8_t*>(a.extra);
   ta.n_pairs = a.n_items / 2;

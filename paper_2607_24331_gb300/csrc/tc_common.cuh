@@ -58,61 +58,6 @@ __device__ __forceinline__ bool wait_slots(uint64_t* empty, int depth, int cnt, 
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
-// Lane 0 waits for ring position `cnt` to be free, then counts how many of the
-// following positions (up to `max_n` in all, at most one ring turn) are free
-// already, without waiting.  Returns that count to the whole warp, 0 if the
-// wait gave up.  (A position within one turn is at most one use ahead of its
-// release, so the parity test cannot see a stale phase.)
-__device__ __forceinline__ int claim_slots(uint64_t* empty, int depth, int cnt, int max_n, int lane,
-                                           volatile int* abort_flag) {
-  int n = 0;
-  if (lane == 0 && (cnt < depth || mbar_wait(&empty[cnt % depth], ((cnt / depth) - 1) & 1, abort_flag))) {
-    n = 1;
-    while (n < max_n && n < depth) {
-      const int c = cnt + n;
-      if (c >= depth && !mbar_test(&empty[c % depth], ((c / depth) - 1) & 1)) break;
-      ++n;
-    }
-  }
-  return __shfl_sync(0xffffffffu, n, 0);
-}
-
-// A ring of `depth` shared-memory slots handed out in FIFO order to
-// instances of variable size (a key group's latent pieces, a unit's factor
-// items), each instance with one full and one empty mbarrier (index
-// instance % kFifoBars; phase (instance / kFifoBars) & 1).  One warp fills the
-// ring; its lanes all keep the same state.  Since every instance holds at
-// least one slot and depth <= kFifoBars, an instance is allocated only after
-// the one kFifoBars before it (same barriers) has been released, so no
-// barrier phase can be confused with another.
-constexpr int kFifoBars = 8;
-struct SlotFifo {
-  int head = 0;       // slots handed out so far (the next instance starts at head % depth)
-  int used = 0;       // slots held by instances not yet released
-  int tail = 0;       // oldest instance not yet released
-  int inst = 0;       // instances handed out so far
-  uint32_t hist = 0;  // slot counts of the last kFifoBars instances, 4 bits each
-  // Waits (lane 0) for the oldest instances' empty barriers until n slots are
-  // free, then records the next instance; false (in every lane) if a wait gave up.
-  __device__ bool claim(int n, int depth, uint64_t* empty, int lane, volatile int* abort_flag) {
-    while (depth - used < n) {
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&empty[tail % kFifoBars], (tail / kFifoBars) & 1, abort_flag);
-      if (__shfl_sync(0xffffffffu, ok ? 1 : 0, 0) == 0) return false;
-      used -= (hist >> (4 * (tail % kFifoBars))) & 0xFu;
-      ++tail;
-    }
-    const int sh = 4 * (inst % kFifoBars);
-    hist = (hist & ~(0xFu << sh)) | ((uint32_t)n << sh);
-    used += n;
-    return true;
-  }
-  __device__ void advance(int n) {
-    head += n;
-    ++inst;
-  }
-};
-
 // ---------------------------------------------------------------------------
 // Work plan of the tensor-core decode path.
 //
@@ -210,8 +155,8 @@ struct PairWalker {
   }
 };
 
-// Block-wide count of pair tiles over the batch (every thread of the block
-// calls it; s256 and s128 are shared scratch of blockDim.x ints each and keep
+// Block-wide count of pair tiles over the batch (every thread of the block, of
+// whole warps, calls it; s256 and s128 are shared scratch of blockDim.x ints each and keep
 // every thread's inclusive prefixes of pair tiles and of 128-token tiles for
 // pair_tile_find).  Block 0 of the grid reports sequences whose rows fall
 // outside the cache.  Returns NP.
@@ -228,17 +173,29 @@ __device__ __forceinline__ int pair_tile_count(const DecodeArgs& a, int* s256, i
       if (L < 0 || st < 0 || st + L > a.n_rows) atomicOr(a.err, kErrBadSeq);
     }
   }
+  // inclusive scan: shuffles inside each warp, then the totals of the warps before
+  __shared__ int w256[32], w128[32];
+  const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, l256, o), w = __shfl_up_sync(0xffffffffu, l128, o);
+    if (lane >= o) {
+      l256 += v;
+      l128 += w;
+    }
+  }
+  if (lane == 31) {
+    w256[warp] = l256;
+    w128[warp] = l128;
+  }
+  __syncthreads();
+  for (int w = 0; w < warp; ++w) {
+    l256 += w256[w];
+    l128 += w128[w];
+  }
   s256[tid] = l256;
   s128[tid] = l128;
   __syncthreads();
-  for (int off = 1; off < nthr; off <<= 1) {
-    const int v = tid >= off ? s256[tid - off] : 0;
-    const int w = tid >= off ? s128[tid - off] : 0;
-    __syncthreads();
-    s256[tid] += v;
-    s128[tid] += w;
-    __syncthreads();
-  }
   return s256[nthr - 1];
 }
 
