@@ -7,13 +7,10 @@
 // 64-wide stages staged by TMA (x: K-major, 128B swizzle; A: MN-major, 128B
 // swizzle) through a 4-deep mbarrier ring.  Warp 0 issues TMA, warp 1 owns
 // TMEM and issues tcgen05.mma, warps 2-5 drain the accumulator (one TMEM lane
-// quadrant each).  Small batches (<= 256 tokens, the decode-step append) split
-// K over CTAs, each storing its fp32 partial in its own slice of the caller's
-// workspace; a second kernel sums the slices, rounds and scatters.  The ring
-// has only as many stages as a CTA has K blocks, so split CTAs of two K blocks
-// fit two to an SM and the whole split runs in one wave.  Longer appends (a
-// prefill) with R_k and r_v multiples of 64 run on persistent CTA pairs
-// (append_pair_kernel below).
+// quadrant each).  Small batches (<= 256 tokens) split K over a cluster of four
+// CTAs that add their partial sums through distributed shared memory
+// (append_few_kernel below).  Longer appends (a prefill) with R_k and r_v
+// multiples of 64 run on persistent CTA pairs (append_pair_kernel below).
 #include <algorithm>
 #include <cstring>
 
@@ -32,19 +29,16 @@ constexpr int kBBytes = kBK * kMaxBN * 2;       // 32 KB
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kThreads = 192;
 constexpr int kSplitMaxTok = 256;
-constexpr int kMaxSplit = 32;  // K splits of a small batch
+constexpr int kMaxSplit = 32;  // slices of a small batch that the workspace query has always allowed for
 
 struct AppendParams {
   int n_tok, D, Rk, rv;
   int nt_k;      // N tiles over the key output
   int kblocks;   // ceil(D / 64)
-  int ksplit;
-  int stages;    // ring depth: min(kStages, K blocks of one CTA)
   const int64_t* rows;  // cache row of each token
   __nv_bfloat16* kc;
   __nv_bfloat16* vc;
   int64_t n_rows;
-  float* ws;     // split-K partials [ksplit][n_tok][Rk + rv] (ksplit > 1)
   int* err;
 };
 
@@ -60,7 +54,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int nst = p.stages;
+  constexpr int nst = kStages;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + nst * kStageBytes);
   uint64_t* empty = full + kStages;
   uint64_t* acc_bar = empty + kStages;
@@ -72,8 +66,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   int n0, nt;
   tile_of(p, blockIdx.x, is_k, n0, nt);
   const int m0 = blockIdx.y * kBM;
-  const int kb0 = (int)((int64_t)blockIdx.z * p.kblocks / p.ksplit);
-  const int kb1 = (int)((int64_t)(blockIdx.z + 1) * p.kblocks / p.ksplit);
+  const int kb0 = 0, kb1 = p.kblocks;
   const int nboxes = (nt + 63) / 64;
 
   if (threadIdx.x == 0) {
@@ -134,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool ok = mbar_wait(acc_bar, 0, abort_flag);
     tc_fence_after();
     int64_t row = -1;
-    if (ok && m < p.n_tok && p.ksplit == 1) {
+    if (ok && m < p.n_tok) {
       row = p.rows[m];
       if (row < 0 || row >= p.n_rows) {
         atomicOr(p.err, kErrBadRow);
@@ -147,22 +140,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       float v[16];
       tmem_ld16(tmem_addr(tmem, quad * 32, c), v);
       tmem_wait_ld();
-      if (m >= p.n_tok) continue;
-      if (p.ksplit == 1) {
-        if (row >= 0) {
-          uint4 pk[2];
-          __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(pk);
+      if (row >= 0) {
+        uint4 pk[2];
+        __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(pk);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) h2[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-          uint4* o = reinterpret_cast<uint4*>(dst + row * N + n0 + c);
-          o[0] = pk[0];
-          o[1] = pk[1];
-        }
-      } else {
-        float4* w = reinterpret_cast<float4*>(p.ws + ((int64_t)blockIdx.z * p.n_tok + m) * (p.Rk + p.rv) +
-                                              (is_k ? 0 : p.Rk) + n0 + c);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        for (int i = 0; i < 8; ++i) h2[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        uint4* o = reinterpret_cast<uint4*>(dst + row * N + n0 + c);
+        o[0] = pk[0];
+        o[1] = pk[1];
       }
     }
   }
@@ -175,35 +160,157 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (threadIdx.x == 0 && *abort_flag) atomicOr(p.err, kErrTimeout);
 }
 
-__global__ void append_finalize_kernel(const float* __restrict__ ws, int n_tok, int Rk, int rv, int ksplit,
-                                       const int64_t* __restrict__ rows, __nv_bfloat16* kc, __nv_bfloat16* vc,
-                                       int64_t n_rows, int* err) {
-  pdl_wait();  // the split partials come from the kernel before
-  pdl_launch_dependents();
-  const int N = Rk + rv;
-  const int m = blockIdx.y;
-  const int64_t row = rows[m];
-  if (row < 0 || row >= n_rows) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) atomicOr(err, kErrBadRow);
-    return;
-  }
-  const int64_t zs = (int64_t)n_tok * N;  // stride between the splits' slices
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
-    const float* w = ws + (int64_t)m * N + c;
-    float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;  // four loads in flight, summed in split order per chain
-    int z = 0;
-    for (; z + 4 <= ksplit; z += 4) {
-      const float a0 = w[z * zs], a1 = w[(z + 1) * zs], a2 = w[(z + 2) * zs], a3 = w[(z + 3) * zs];
-      v0 += a0;
-      v1 += a1;
-      v2 += a2;
-      v3 += a3;
+// ---------------------------------------------------------------------------
+// Small batches (<= 256 tokens): a cluster of four CTAs per 128 tokens x 64
+// output columns, CTA `rank` taking a quarter of K.  Bound by the latency of one
+// pass over the factors (HBM, 2.5 us on the 32-head layer) and by each CTA's x
+// stream from L2 (64 columns re-read it once per tile); seven 24 KB stages per
+// CTA keep both in flight.  The CTAs push each 16-column slice of their partial
+// sums into its owner rank's shared memory, meet at a cluster barrier, and every
+// rank adds its slice's four partials and writes the rows.  (Partials through
+// global memory, 19 slices written and read back by a second launch, took as long
+// as the products: 19.4 us for 100 tokens on the 32-head layer.)
+// ---------------------------------------------------------------------------
+
+constexpr int kFN = 64;        // output columns of a cluster
+constexpr int kFSplit = 4;     // K quarters = CTAs of a cluster; 16 columns of the sum each
+constexpr int kFStages = 7;
+constexpr int kFBBytes = kBK * kFN * 2;             // 8 KB
+constexpr int kFStageBytes = kABytes + kFBBytes;
+constexpr int kFRecvBytes = kFSplit * kBM * 16 * 4; // partial sums received: [source rank][token][16] fp32
+static_assert(kFN == 16 * kFSplit, "a rank owns one 16-column slice");
+
+// 16-byte chunk q of token row r in a slice: rotated over the rows, so that the
+// pushes of a warp (one row per lane) spread over the banks.
+__device__ __forceinline__ int few_chunk(int r, int q) { return (r * 4 + (q ^ ((r >> 1) & 3))) * 16; }
+
+__global__ void __launch_bounds__(kThreads, 1)
+    append_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_ak,
+                      const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* recv = smem + kFStages * kFStageBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(recv + kFRecvBytes);
+  uint64_t* empty = full + kFStages;
+  uint64_t* acc_bar = empty + kFStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_bar + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)cluster_ctarank();
+  const int t = blockIdx.x / kFSplit;
+  const bool is_k = t < p.nt_k;
+  const int N = is_k ? p.Rk : p.rv, n0 = (is_k ? t : t - p.nt_k) * kFN;
+  const int m0 = blockIdx.y * kBM;
+  const int kb0 = rank * p.kblocks / kFSplit, kb1 = (rank + 1) * p.kblocks / kFSplit;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kFStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
     }
-    for (; z < ksplit; ++z) v0 += w[z * zs];
-    const float v = (v0 + v1) + (v2 + v3);
-    if (c < Rk) kc[row * Rk + c] = __float2bfloat16_rn(v);
-    else vc[row * rv + (c - Rk)] = __float2bfloat16_rn(v);
+    mbar_init(acc_bar, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
   }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, kFN);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  cluster_sync();  // every CTA of the cluster runs: its shared memory may be written
+  tc_fence_after();
+  pdl_wait();
+  pdl_launch_dependents();
+  const uint32_t tmem = *tmem_slot;
+  const CUtensorMap* tmb = is_k ? &tm_ak : &tm_av;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      for (int kb = kb0; kb < kb1; ++kb) {
+        const int i = kb - kb0, s = i % kFStages;
+        if (i >= kFStages && !mbar_wait(&empty[s], ((i / kFStages) - 1) & 1, abort_flag)) break;
+        uint8_t* a = smem + s * kFStageBytes;
+        mbar_expect_tx(&full[s], kFStageBytes);
+        tma_load_2d(a + kABytes, tmb, &full[s], n0, kb * kBK);
+        tma_load_2d(a, &tm_x, &full[s], kb * kBK, m0);
+      }
+    }
+  } else if (warp == 1) {
+    const bool el = elect_one();
+    const uint32_t idesc = idesc_bf16(kBM, kFN, false, true), s0 = smem_u32(smem);
+    const uint64_t da = sdesc(s0, 16, 1024, kSw128), db = sdesc(s0 + kABytes, kFBBytes, 1024, kSw128);
+    bool ok = true;
+    for (int i = 0; i < kb1 - kb0; ++i) {
+      const int s = i % kFStages;
+      ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (i / kFStages) & 1, abort_flag));
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t o = (uint64_t)(s * (kFStageBytes >> 4));
+      if (el) {
+#pragma unroll
+        for (int k = 0; k < kBK / 16; ++k)
+          umma_f16(tmem, da + o + 2 * k, db + o + 128 * k, idesc, (i > 0 || k > 0) ? 1u : 0u);
+        umma_commit(&empty[s]);
+      }
+    }
+    if (el) umma_commit(acc_bar);
+  } else {
+    const int quad = warp & 3, r = quad * 32 + lane;
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_bar, 0, abort_flag));
+    tc_fence_after();
+    if (ok) {
+#pragma unroll
+      for (int c = 0; c < kFSplit; ++c) {
+        float v[16];
+        if (kb0 < kb1) {
+          tmem_ld16(tmem_addr(tmem, quad * 32, 16 * c), v);
+          tmem_wait_ld();
+        } else {  // fewer K blocks than ranks
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        }
+        if (m0 + r < p.n_tok) {
+          const uint32_t dst = mapa_shared(smem_u32(recv + rank * (kBM * 64)), (uint32_t)c);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + few_chunk(r, q)),
+                         "f"(v[4 * q]), "f"(v[4 * q + 1]), "f"(v[4 * q + 2]), "f"(v[4 * q + 3])
+                         : "memory");
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync();  // every partial sum of this rank's slice has arrived
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kFN);
+  }
+  const int col = n0 + 16 * rank;
+  __nv_bfloat16* dst = is_k ? p.kc : p.vc;
+  for (int i = threadIdx.x; i < kBM * 4; i += kThreads) {
+    const int r = i >> 2, q = i & 3;
+    if (m0 + r >= p.n_tok) break;
+    const int64_t row = p.rows[m0 + r];
+    if (row < 0 || row >= p.n_rows) {
+      atomicOr(p.err, kErrBadRow);
+      continue;
+    }
+    if (col >= N) continue;  // the last tile of an output whose width is no multiple of 64
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int z = 0; z < kFSplit; ++z) {
+      const float4 w = *reinterpret_cast<const float4*>(recv + z * (kBM * 64) + few_chunk(r, q));
+      v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+    }
+    uint2 o;
+    *reinterpret_cast<__nv_bfloat162*>(&o.x) = __floats2bfloat162_rn(v.x, v.y);
+    *reinterpret_cast<__nv_bfloat162*>(&o.y) = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(dst + row * N + col + 4 * q) = o;
+  }
+  if (threadIdx.x == 0 && *abort_flag) atomicOr(p.err, kErrTimeout);
 }
 
 // ---------------------------------------------------------------------------
@@ -465,17 +572,6 @@ int append_pairs_of_device(size_t smem) {
   return cache[dev];
 }
 
-int plan_ksplit(int n_tok, int D, int Rk, int rv, int sms) {
-  if (n_tok > kSplitMaxTok) return 1;
-  const int mt = (n_tok + kBM - 1) / kBM;
-  const int ntiles = (Rk + kMaxBN - 1) / kMaxBN + (rv + kMaxBN - 1) / kMaxBN;
-  const int kblocks = (D + kBK - 1) / kBK;
-  // up to two CTAs per SM (split CTAs of at most two K blocks take 96 KB of shared memory)
-  int ks = 2 * sms / max(1, mt * ntiles);
-  ks = max(1, min(ks, min(kMaxSplit, kblocks)));
-  return ks;
-}
-
 }  // namespace
 
 bool tc_append_supports(int D, int Rk, int rv, int dtype) {
@@ -487,11 +583,9 @@ size_t tc_append_workspace(int n_tok, int Rk, int rv) {
 }
 
 cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
-                             const int64_t* rows, void* kc, void* vc, int64_t n_rows, void* ws, size_t ws_bytes,
-                             int* err, cudaStream_t s, int* n_launches) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+                             const int64_t* rows, void* kc, void* vc, int64_t n_rows, int* err, cudaStream_t s,
+                             int* n_launches) {
+  *n_launches = 1;
   AppendParams p;
   p.n_tok = n_tok;
   p.D = D;
@@ -499,15 +593,11 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
   p.rv = rv;
   p.nt_k = (Rk + kMaxBN - 1) / kMaxBN;
   p.kblocks = (D + kBK - 1) / kBK;
-  p.ksplit = plan_ksplit(n_tok, D, Rk, rv, sms);
-  p.stages = std::min(kStages, (p.kblocks + p.ksplit - 1) / p.ksplit);
   p.rows = rows;
   p.kc = static_cast<__nv_bfloat16*>(kc);
   p.vc = static_cast<__nv_bfloat16*>(vc);
   p.n_rows = n_rows;
-  p.ws = static_cast<float*>(ws);
   p.err = err;
-  if (n_tok <= kSplitMaxTok && (!ws || ws_bytes < tc_append_workspace(n_tok, Rk, rv))) return cudaErrorInvalidValue;
   CUtensorMap tx, tk, tv;
   if (!make_tmap_2d_bf16(&tx, x, D, n_tok, (uint64_t)D * 2, kBK, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_tmap_2d_bf16(&tk, A_k, Rk, D, (uint64_t)Rk * 2, 64, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -537,23 +627,35 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
       attr[1].val.programmaticStreamSerializationAllowed = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 2;
-      *n_launches = 1;
       return cudaLaunchKernelEx(&cfg, append_pair_kernel, tx, tk, tv, p);
     }
   }
+  if (n_tok <= kSplitMaxTok) {
+    p.nt_k = (Rk + kFN - 1) / kFN;
+    const size_t fsmem = (size_t)kFStages * kFStageBytes + kFRecvBytes + 1024 + 256;
+    cudaError_t e = cudaFuncSetAttribute(append_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kFSplit * (p.nt_k + (rv + kFN - 1) / kFN), (n_tok + kBM - 1) / kBM);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = fsmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kFSplit;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, append_few_kernel, tx, tk, tv, p);
+  }
   const int ntiles = p.nt_k + (rv + kMaxBN - 1) / kMaxBN;
-  const size_t smem = (size_t)p.stages * kStageBytes + 1024 + 256;
-  // the attribute is an upper bound for every launch (prefill uses all kStages stages)
-  cudaError_t e = cudaFuncSetAttribute(append_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(kStages * kStageBytes + 1024 + 256));
+  const size_t smem = (size_t)kStages * kStageBytes + 1024 + 256;
+  cudaError_t e = cudaFuncSetAttribute(append_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid(ntiles, (n_tok + kBM - 1) / kBM, p.ksplit);
-  *n_launches = p.ksplit > 1 ? 2 : 1;
-  e = launch_pdl(append_tc_kernel, grid, dim3(kThreads), smem, s, tx, tk, tv, p);
-  if (e != cudaSuccess || p.ksplit == 1) return e;
-  dim3 g2((Rk + rv + 255) / 256, n_tok);
-  return launch_pdl(append_finalize_kernel, g2, dim3(256), 0, s, (const float*)p.ws, n_tok, Rk, rv, p.ksplit, rows,
-                    p.kc, p.vc, n_rows, err);
+  return launch_pdl(append_tc_kernel, dim3(ntiles, (n_tok + kBM - 1) / kBM), dim3(kThreads), smem, s, tx, tk, tv, p);
 }
 
 }  // namespace dck

@@ -28,8 +28,8 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
                               void* out, void* ws, int* err, LaunchHook* hook, cudaStream_t s);
 cudaError_t launch_bounded_wait_selftest(long long limit_cycles, int* err, cudaStream_t s);
 cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
-                             const int64_t* rows, void* kc, void* vc, int64_t n_rows, void* ws, size_t ws_bytes,
-                             int* err, cudaStream_t s, int* n_launches);
+                             const int64_t* rows, void* kc, void* vc, int64_t n_rows, int* err, cudaStream_t s,
+                             int* n_launches);
 }  // namespace dck
 
 using namespace dck;
@@ -407,8 +407,8 @@ dck_status dck_latent_append(const dck_layer_desc* desc, const void* x, int32_t 
   if (tc_append_supports(desc->hidden, lt.Rk, lt.rv, desc->dtype)) {
     const size_t need = tc_append_workspace(n_tok, lt.Rk, lt.rv);
     if (need && (!workspace || ws_bytes < need || !aligned(workspace, 256))) return DCK_ERR_WORKSPACE;
-    e = launch_append_tc(x, n_tok, desc->hidden, A_k, A_v, lt.Rk, lt.rv, d_rows, kcache, vcache, n_rows, workspace,
-                         ws_bytes, err, s, &launches);
+    e = launch_append_tc(x, n_tok, desc->hidden, A_k, A_v, lt.Rk, lt.rv, d_rows, kcache, vcache, n_rows, err, s,
+                         &launches);
   } else {
     e = launch_append_simt(x, n_tok, desc->hidden, A_k, A_v, lt.Rk, lt.rv, d_rows, kcache, vcache, n_rows,
                            desc->dtype, err, s);
