@@ -148,7 +148,7 @@ struct AWalk {
 __global__ void __launch_bounds__(kAThreads, 1)
     absorb_tc_kernel(const __grid_constant__ AMaps maps, const LayerTable lt, const DecodeArgs a, const AbsArgs aa) {
   extern __shared__ uint8_t smem_raw[];
-  ASmem& sm = *reinterpret_cast<ASmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  ASmem& sm = *reinterpret_cast<ASmem*>(align_1024(smem_raw));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* abort_flag = &sm.abort_flag;
   const int Hq = lt.Hq, hq_pad = aa.hq_pad, n_chunks = aa.n_chunks;

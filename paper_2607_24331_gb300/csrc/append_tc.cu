@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     append_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_ak,
                      const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_1024(smem_raw);
   constexpr int nst = kStages;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + nst * kStageBytes);
   uint64_t* empty = full + kStages;
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     append_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_ak,
                       const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_1024(smem_raw);
   uint8_t* recv = smem + kFStages * kFStageBytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(recv + kFRecvBytes);
   uint64_t* empty = full + kFStages;
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
     append_pair_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_ak,
                        const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_1024(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kPStages * kPStageBytes);
   uint64_t* empty = full + kPStages;
   uint64_t* acc_full = empty + kPStages;

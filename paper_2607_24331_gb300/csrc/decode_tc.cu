@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   constexpr int kThreads = kThreadsTc;
   extern __shared__ uint8_t smem_raw[];
   Smem<kFold>& sm =
-      *reinterpret_cast<Smem<kFold>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+      *reinterpret_cast<Smem<kFold>*>(align_1024(smem_raw));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* abort_flag = &sm.abort_flag;
   const int hq_pad = ta.hq_pad;

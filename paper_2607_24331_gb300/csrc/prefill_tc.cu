@@ -122,7 +122,7 @@ __device__ __forceinline__ float2 unpack2(uint32_t v) {
 __global__ void __launch_bounds__(kRThreads, 1)
     recon_kernel(const __grid_constant__ RMaps maps, const __grid_constant__ RArgs ra) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = align_1024(smem_raw);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRStages * kRStageBytes);
   uint64_t* empty = full + kRStages;
   uint64_t* acc_full = empty + kRStages;
@@ -570,7 +570,7 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 __global__ void __launch_bounds__(kAThreadsP, 1)
     prefill_attn_kernel(const __grid_constant__ AMapsP maps, const __grid_constant__ AArgsP aa) {
   extern __shared__ uint8_t smem_raw[];
-  ASmemP& sm = *reinterpret_cast<ASmemP*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  ASmemP& sm = *reinterpret_cast<ASmemP*>(align_1024(smem_raw));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* abort_flag = &sm.abort_flag;
   const int qpg = aa.qpg, pp = 128 / qpg;

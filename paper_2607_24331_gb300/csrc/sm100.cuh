@@ -14,6 +14,11 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The first 1024-byte boundary (the swizzle atom) of dynamic shared memory.  As
+// an offset from the array, not a rounded pointer: the compiler then knows every
+// access for shared memory, where it would use generic ones.
+__device__ __forceinline__ uint8_t* align_1024(uint8_t* raw) { return raw + ((0u - smem_u32(raw)) & 1023u); }
+
 __device__ __forceinline__ uint64_t global_timer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
