@@ -76,7 +76,7 @@ struct ASmem {
   uint64_t v_full[2 * kNVr], v_empty[2 * kNVr], p_full[kNP], p_empty[kNP];
   uint64_t drain, tile_ok, u_ready[2], u_free[2];
   int pneed[kNP];  // P slot's tile raises some head's reference max (set by the producer before the slot fills)
-  int s256[kAThreads], s128[kAThreads];
+  PairScratch sc;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -156,22 +156,25 @@ __global__ void __launch_bounds__(kAThreads, 1)
   DCK_AB_TRACE(99);
   griddep_launch();  // the combine kernel may stage its factors as CTAs finish
 
-  if (tid == 0) {
-    for (int i = 0; i < 2 * kNVr; ++i) {
-      mbar_init(&sm.v_full[i], 1);
-      mbar_init(&sm.v_empty[i], 1);
+  if (warp == 0) {  // a barrier per lane
+    if (lane < 2 * kNVr) {
+      mbar_init(&sm.v_full[lane], 1);
+      mbar_init(&sm.v_empty[lane], 1);
     }
-    for (int i = 0; i < kNP; ++i) {
-      mbar_init(&sm.p_full[i], 1);
-      mbar_init(&sm.p_empty[i], 2);  // released by both MMA threads
+    if (lane < kNP) {
+      mbar_init(&sm.p_full[lane], 1);
+      mbar_init(&sm.p_empty[lane], 2);  // released by both MMA threads
     }
-    mbar_init(&sm.drain, 2);
-    mbar_init(&sm.tile_ok, kEpiWarpsA);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&sm.u_ready[i], 2);
-      mbar_init(&sm.u_free[i], kEpiWarpsA);
+    if (lane < 2) {
+      mbar_init(&sm.u_ready[lane], 2);
+      mbar_init(&sm.u_free[lane], kEpiWarpsA);
     }
-    sm.abort_flag = 0;
+    if (lane == 0) {
+      mbar_init(&sm.drain, 2);
+      mbar_init(&sm.tile_ok, kEpiWarpsA);
+      sm.abort_flag = 0;
+      tma_prefetch_desc(&maps.vc);
+    }
     fence_mbar_init();
   }
   if (warp == 1) {
@@ -187,27 +190,30 @@ __global__ void __launch_bounds__(kAThreads, 1)
   pl.hh = blockIdx.x & 1;
   pl.nc = n_chunks;
   DCK_AB_TRACE(3);
-  const int NP = pair_tile_count(a, sm.s256, sm.s128);
+  const PairScan scan = pair_scan(a, sm.sc);
+  const int NP = scan.total256;
   DCK_AB_TRACE(4);
   const PSplit sp(NP, pl.P);
   pl.NPm = sp.NPm;
-  const bool fits = sm.s128[kAThreads - 1] <= aa.max_tiles;  // else the scores kernel has reported the input
+  const bool fits = scan.total128 <= aa.max_tiles;  // else the scores kernel has reported the input
   const int X0 = fits ? sp.main_begin(pl.pr, pl.P) : 0;
   const int X1 = fits ? sp.main_begin(pl.pr + 1, pl.P) : 0;
   const int xc = 2 * sp.R * n_chunks;
-  pl.c_lo = fits ? (int)((int64_t)blockIdx.x * xc / a.n_items) : 0;
-  pl.c_hi = fits ? (int)((int64_t)(blockIdx.x + 1) * xc / a.n_items) : 0;
+  pl.c_lo = fits ? (int)blockIdx.x * xc / a.n_items : 0;  // (fewer than P extra pair tiles)
+  pl.c_hi = fits ? (int)(blockIdx.x + 1) * xc / a.n_items : 0;
   const int q0 = pl.c_lo < pl.c_hi ? pl.c_lo / n_chunks : 0;
   const int q1 = pl.c_lo < pl.c_hi ? (pl.c_hi - 1) / n_chunks + 1 : 0;
-  AWalk walk0;
-  walk0.wm = pair_walker_at(a, sm.s256, sm.s128, X0, X1, false);
-  walk0.wx = pair_walker_at(a, sm.s256, sm.s128, sp.NPm + q0 / 2, q0 < q1 ? sp.NPm + (q1 - 1) / 2 + 1 : sp.NPm, true);
+  const int xx0 = sp.NPm + q0 / 2, xx1 = q0 < q1 ? sp.NPm + (q1 - 1) / 2 + 1 : sp.NPm;
+  pair_find(a, scan, X0, xx0, sm.sc);
   const bool has_work = X0 < X1 || pl.c_lo < pl.c_hi;
   // the two MMA threads split a tile's chunks [ca, cb) at cm: thread 0 [ca, cm), thread 1 [cm, cb)
   auto chunk_mid = [](int ca, int cb) { return ca + (cb - ca + 1) / 2; };
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  AWalk walk0;
+  walk0.wm = pair_walker(sm.sc.at[0], X0, X1, false);
+  walk0.wx = pair_walker(sm.sc.at[1], xx0, xx1, true);
   const uint32_t tmem = sm.tmem_base;
   // U is double-buffered in TMEM where two copies fit: segment s accumulates in
   // buffer s % nub while the epilogue reads out segment s - 1

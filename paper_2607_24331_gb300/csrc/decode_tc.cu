@@ -199,7 +199,6 @@ struct Smem {
   uint64_t k_full[2], k_empty[2], epi_bar, x_free;
   GroupSm grp[kMaxGroupsTc];
   uint32_t uinfo[kMaxUnits];
-  PairWalker walk[2];  // main and extra pair tiles of this pair
   int8_t hunit[kMaxHqTc];
   uint32_t tmem_base;
   int abort_flag;
@@ -232,7 +231,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     decode_tc_kernel(const __grid_constant__ Maps maps, const LayerTable lt, const DecodeArgs a,
                      const __grid_constant__ TcArgs ta) {
   constexpr int kMma = Ring<kFold>::kMma, NW = Ring<kFold>::NW, kNA = Ring<kFold>::NA;
-  constexpr int kThreads = kThreadsTc;
   extern __shared__ uint8_t smem_raw[];
   Smem<kFold>& sm =
       *reinterpret_cast<Smem<kFold>*>(align_1024(smem_raw));
@@ -245,20 +243,24 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   const int P = ta.n_pairs, pair = blockIdx.x >> 1;
 
   // ---- setup -------------------------------------------------------------
-  if (tid == 0) {
-    for (int i = 0; i < kNA; ++i) {
-      mbar_init(&sm.a_full[i], 1);      // even CTA: its producer's expect_tx; both CTAs' copies complete on it
-      mbar_init(&sm.a_empty[i], kMma);  // released by every MMA warp (arrivals reach both CTAs)
+  if (warp == 0) {  // a barrier per lane
+    if (lane < kItemBars) mbar_init(&sm.w_full[lane], 1);
+    if (lane < kNA) {
+      mbar_init(&sm.a_full[lane], 1);      // even CTA: its producer's expect_tx; both CTAs' copies complete on it
+      mbar_init(&sm.a_empty[lane], kMma);  // released by every MMA warp (arrivals reach both CTAs)
     }
-    for (int i = 0; i < NW; ++i) mbar_init(&sm.w_empty[i], 1);
-    for (int i = 0; i < kItemBars; ++i) mbar_init(&sm.w_full[i], 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&sm.k_full[i], 1);
-      mbar_init(&sm.k_empty[i], 2 * kEpiWarps);  // even CTA: both CTAs' epilogue warps
+    if (lane < NW) mbar_init(&sm.w_empty[lane], 1);
+    if (lane < 2) {
+      mbar_init(&sm.k_full[lane], 1);
+      mbar_init(&sm.k_empty[lane], 2 * kEpiWarps);  // even CTA: both CTAs' epilogue warps
     }
-    mbar_init(&sm.epi_bar, kEpiWarps);
-    mbar_init(&sm.x_free, kEpiWarps);
-    sm.abort_flag = 0;
+    if (lane == 0) {
+      mbar_init(&sm.epi_bar, kEpiWarps);
+      mbar_init(&sm.x_free, kEpiWarps);
+      sm.abort_flag = 0;
+      tma_prefetch_desc(&maps.kc64);
+      tma_prefetch_desc(&maps.im[3]);
+    }
     fence_mbar_init();
   }
   if (warp == 1) {
@@ -273,11 +275,9 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   // [u_lo, u_hi) of the flattened (extra tile, unit) list, every extra tile a
   // segment of its own.
   const int U = ta.n_units;
-  // block-scan scratch in the latent ring: used only before the first copy is issued
-  int* const s256 = reinterpret_cast<int*>(sm.a[0]);
-  int* const s128 = s256 + kThreads;
-  const int NP = pair_tile_count(a, s256, s128);
-  const int NT128 = s128[kThreads - 1];
+  __shared__ PairScratch sc;
+  const PairScan scan = pair_scan(a, sc);
+  const int NP = scan.total256, NT128 = scan.total128;
   const PSplit sp(NP, P);
   // the per-tile stores are sized for non-overlapping sequences; more tiles
   // than that is reported as invalid input and nothing is computed
@@ -286,17 +286,10 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   const int X0 = fits ? sp.main_begin(pair, P) : 0;
   const int X1 = fits ? sp.main_begin(pair + 1, P) : 0;
   const int xu = sp.R * U;
-  const int u_lo = fits ? (int)((int64_t)pair * xu / P) : 0;
-  const int u_hi = fits ? (int)((int64_t)(pair + 1) * xu / P) : 0;
+  const int u_lo = fits ? pair * xu / P : 0;  // (fewer than P extra tiles)
+  const int u_hi = fits ? (pair + 1) * xu / P : 0;
   const int xe0 = sp.NPm + (u_lo < u_hi ? u_lo / U : 0), xe1 = sp.NPm + (u_lo < u_hi ? (u_hi - 1) / U + 1 : 0);
-  {
-    const PairWalker wm = pair_walker_at(a, s256, s128, X0, X1, false);
-    const PairWalker wx = pair_walker_at(a, s256, s128, xe0, xe1, true);
-    if (tid == 0) {
-      sm.walk[0] = wm;
-      sm.walk[1] = wx;
-    }
-  }
+  pair_find(a, scan, X0, xe0, sc);
   const bool has_work = X0 < X1 || xe0 < xe1;  // the same in both CTAs of the pair
   // units [ua, ub) of flattened pair tile X in phase ph (0: main, 1: extra)
   auto units_of = [&](int ph, int X, int& ua, int& ub) {
@@ -309,8 +302,11 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
     }
   };
   tc_fence_before();
-  cluster_sync();  // both CTAs' barriers initialised and TMEM allocated
+  cluster_sync();  // both CTAs' barriers initialised and TMEM allocated, the walkers' starts found
   tc_fence_after();
+  auto walker = [&](int ph) {  // main or extra pair tiles of this pair
+    return pair_walker(sc.at[ph], ph ? xe0 : X0, ph ? xe1 : X1, ph != 0);
+  };
   const uint32_t tmem = sm.tmem_base;
   // shared::cluster addresses: a barrier of the even CTA, or a word of the peer
   auto lead = [](const void* p) { return mapa_shared(smem_u32(p), 0); };
@@ -340,7 +336,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       bool ok = true;
       // L2 prefetch of this half's latent rows, prefetch_ahead() tiles ahead of the
       // loads (across segment boundaries): the TMA loads then find them in L2
-      PairWalker pwalk = sm.walk[0];
+      PairWalker pwalk = walker(0);
       PSegment pseg = {};
       int pph = 0, pti = 0;
       auto prefetch_next = [&]() {
@@ -350,7 +346,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
           if (pph >= 2) return;
           if (!pwalk.next(a, pseg)) {
             pseg.ntiles = 0;
-            if (++pph < 2) pwalk = sm.walk[pph];
+            if (++pph < 2) pwalk = walker(pph);
           }
         }
         const int64_t r0 = pseg.row0 + pseg.t0(pti++, hr);
@@ -361,7 +357,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       griddep_wait();  // the preparation launch may append the step's own latents
       griddep_launch();
       for (int ph = 0; ph < 2 && ok; ++ph)
-        for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
+        for (PairWalker walk = walker(ph); ok && walk.next(a, seg);) {
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             const int64_t yrow = seg.row0 + seg.t0(i, hr);
             prefetch_next();
@@ -401,7 +397,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       int slot = 0, fills = 0, pos = 0;  // factor ring: next slot, times round, items so far
       bool ok = true;
       for (int ph = 0; ph < 2 && ok; ++ph)
-        for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
+        for (PairWalker walk = walker(ph); ok && walk.next(a, seg);) {
           const int64_t img_row0 = kFold ? (int64_t)seg.b * img_seq_rows : 0;
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             int ua, ub;
@@ -450,7 +446,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       int kc = 0, own = 0;  // units of the pair so far, units in this warp's accumulator
       bool ok = true;
       for (int ph = 0; ph < 2 && ok; ++ph)
-        for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
+        for (PairWalker walk = walker(ph); ok && walk.next(a, seg);) {
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             int ua, ub;
             units_of(ph, seg.X0 + i, ua, ub);
@@ -564,7 +560,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
       }
     };
     for (int ph = 0; ph < 2 && ok; ++ph)
-      for (PairWalker walk = sm.walk[ph]; ok && walk.next(a, seg);) {
+      for (PairWalker walk = walker(ph); ok && walk.next(a, seg);) {
         if (!kFold) {
           // rotated queries of this sequence at position L-1, scaled to log2 units
           // (its last tile's scores have been formed: that tile's EPI_SYNC)
@@ -1081,8 +1077,8 @@ bool build_maps(const LayerTable& lt, const DecodeArgs& a, const void* img, int6
 }
 
 static_assert(kMaxPieces <= Ring<true>::NW && Ring<true>::NW <= 5 && kMaxPieces <= 5, "see kItemBars");
-static_assert(sizeof(Smem<true>) + 1024 + 384 <= 232448, "shared memory of the query-folded kernel");
-static_assert(sizeof(Smem<false>) + 1024 + 384 <= 232448, "shared memory of the key-mode kernel");
+static_assert(sizeof(Smem<true>) + 1024 + sizeof(PairScratch) <= 232448, "shared memory of the query-folded kernel");
+static_assert(sizeof(Smem<false>) + 1024 + sizeof(PairScratch) <= 232448, "shared memory of the key-mode kernel");
 
 template <bool kFold>
 cudaError_t set_smem_attr() {

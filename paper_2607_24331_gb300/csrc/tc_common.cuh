@@ -106,7 +106,10 @@ __host__ __device__ inline int64_t pair_slot_count(int P, int B, int64_t n_rows)
 struct PSplit {
   int NP, NPm, R;
   __host__ __device__ PSplit(int np, int P) : NP(np), NPm(np / P < kFineSplitBelow ? np / P * P : np), R(np - NPm) {}
-  __host__ __device__ int main_begin(int p, int P) const { return item_begin(p, NPm, P); }
+  // floor(p NPm / P): the tiles of caches of fewer than 2^31 rows times the pairs of a GPU stay below 2^32
+  __host__ __device__ int main_begin(int p, int P) const {
+    return (int)((uint32_t)p * (uint32_t)NPm / (uint32_t)P);
+  }
 };
 
 // A run of consecutive pair tiles of one sequence.
@@ -155,88 +158,92 @@ struct PairWalker {
   }
 };
 
-// Block-wide count of pair tiles over the batch (every thread of the block, of
-// whole warps, calls it; s256 and s128 are shared scratch of blockDim.x ints each and keep
-// every thread's inclusive prefixes of pair tiles and of 128-token tiles for
-// pair_tile_find).  Block 0 of the grid reports sequences whose rows fall
-// outside the cache.  Returns NP.
-__device__ __forceinline__ int pair_tile_count(const DecodeArgs& a, int* s256, int* s128) {
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int per = (a.B + nthr - 1) / nthr;
-  const int b0 = tid * per;
-  int l256 = 0, l128 = 0;
-  for (int b = b0; b < b0 + per && b < a.B; ++b) {
-    l256 += n256_of(a, b);
-    l128 += n128_of(a, b);
-    if (blockIdx.x == 0) {
-      const int64_t L = a.seq_len[b], st = a.seq_start[b];
-      if (L < 0 || st < 0 || st + L > a.n_rows) atomicOr(a.err, kErrBadSeq);
+// The batch's tile counts and where a thread's sequences lie in them: a block-wide
+// scan (every thread of the block, of whole warps, takes part) whose results stay
+// in registers.  Two barriers from the sequence lengths to the walkers: a CTA with
+// one unit of work spends most of its time before its first load otherwise.
+struct PairScan {
+  int total256, total128;  // pair tiles and 128-token tiles of the batch
+  int b0, per;             // this thread's sequences [b0, b0 + per)
+  int r256, r128;          // tiles before them
+  int n256, n128;          // tiles of them
+};
+struct PairFind {
+  int b, p256, p128;  // sequence of a flattened pair tile, tiles before that sequence
+};
+struct PairScratch {
+  int w256[32], w128[32];  // the warps' totals
+  PairFind at[2];
+};
+
+// Block 0 of the grid reports sequences whose rows fall outside the cache.
+__device__ __forceinline__ PairScan pair_scan(const DecodeArgs& a, PairScratch& sc) {
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  PairScan s;
+  s.per = (a.B + nthr - 1) / nthr;
+  s.b0 = tid * s.per;
+  s.n256 = s.n128 = 0;
+  for (int b = s.b0; b < s.b0 + s.per && b < a.B; ++b) {
+    int64_t L = a.seq_len[b];
+    const int64_t st = a.seq_start[b];
+    if (L < 0 || st < 0 || st + L > a.n_rows) {
+      if (blockIdx.x == 0) atomicOr(a.err, kErrBadSeq);
+      L = 0;
     }
+    s.n256 += (int)((L + kPTile - 1) / kPTile);
+    s.n128 += (int)((L + kTile - 1) / kTile);
   }
-  // inclusive scan: shuffles inside each warp, then the totals of the warps before
-  __shared__ int w256[32], w128[32];
-  const int lane = tid & 31, warp = tid >> 5;
+  int i256 = s.n256, i128 = s.n128;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, l256, o), w = __shfl_up_sync(0xffffffffu, l128, o);
+    const int v = __shfl_up_sync(0xffffffffu, i256, o), w = __shfl_up_sync(0xffffffffu, i128, o);
     if (lane >= o) {
-      l256 += v;
-      l128 += w;
+      i256 += v;
+      i128 += w;
     }
   }
   if (lane == 31) {
-    w256[warp] = l256;
-    w128[warp] = l128;
+    sc.w256[warp] = i256;
+    sc.w128[warp] = i128;
   }
   __syncthreads();
-  for (int w = 0; w < warp; ++w) {
-    l256 += w256[w];
-    l128 += w128[w];
+  int t256 = lane < (nthr >> 5) ? sc.w256[lane] : 0, t128 = lane < (nthr >> 5) ? sc.w128[lane] : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, t256, o), w = __shfl_up_sync(0xffffffffu, t128, o);
+    if (lane >= o) {
+      t256 += v;
+      t128 += w;
+    }
   }
-  s256[tid] = l256;
-  s128[tid] = l128;
-  __syncthreads();
-  return s256[nthr - 1];
+  s.total256 = __shfl_sync(0xffffffffu, t256, 31);
+  s.total128 = __shfl_sync(0xffffffffu, t128, 31);
+  const int b256 = __shfl_sync(0xffffffffu, t256, warp ? warp - 1 : 0);
+  const int b128 = __shfl_sync(0xffffffffu, t128, warp ? warp - 1 : 0);
+  s.r256 = i256 - s.n256 + (warp ? b256 : 0);
+  s.r128 = i128 - s.n128 + (warp ? b128 : 0);
+  return s;
 }
 
-// Block-wide lookup (after pair_tile_count, same scratch): a walker positioned
-// at flattened pair tile X over [X, X1).
-__device__ __forceinline__ PairWalker pair_walker_at(const DecodeArgs& a, const int* s256, const int* s128, int X,
-                                                     int X1, bool single) {
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int per = (a.B + nthr - 1) / nthr;
-  const int b0 = tid * per;
-  __shared__ int s_b, s_p256, s_p128;
-  if (tid == 0) {
-    s_b = a.B;
-    s_p256 = s256[nthr - 1];
-    s_p128 = s128[nthr - 1];
+// Looks up flattened pair tiles X0 and X1 (block-wide; a tile past the batch's
+// last leaves its walker with nothing to walk, as its range is empty) and returns
+// them in sc.at after a barrier that the caller passes next.
+__device__ __forceinline__ void pair_find(const DecodeArgs& a, const PairScan& s, int X0, int X1, PairScratch& sc) {
+  int r256 = s.r256, r128 = s.r128;
+  for (int b = s.b0; b < s.b0 + s.per && b < a.B; ++b) {
+    const int nt = s.per == 1 ? s.n256 : n256_of(a, b);
+    if (X0 >= r256 && X0 < r256 + nt) sc.at[0] = PairFind{b, r256, r128};
+    if (X1 >= r256 && X1 < r256 + nt) sc.at[1] = PairFind{b, r256, r128};
+    r256 += nt;
+    r128 += s.per == 1 ? s.n128 : n128_of(a, b);
   }
-  __syncthreads();
-  int r256 = tid ? s256[tid - 1] : 0, r128 = tid ? s128[tid - 1] : 0;
-  if (per == 1) {  // this thread's sequence (if any): its tile counts are the prefix steps
-    const int nt = s256[tid] - r256;
-    if (b0 < a.B && nt > 0 && X >= r256 && X < r256 + nt) {
-      s_b = b0;
-      s_p256 = r256;
-      s_p128 = r128;
-    }
-  } else {
-    for (int b = b0; b < b0 + per && b < a.B; ++b) {
-      const int nt = n256_of(a, b);
-      if (nt > 0 && X >= r256 && X < r256 + nt) {
-        s_b = b;
-        s_p256 = r256;
-        s_p128 = r128;
-      }
-      r256 += nt;
-      r128 += n128_of(a, b);
-    }
+  if (threadIdx.x == 0) {
+    if (X0 >= s.total256) sc.at[0] = PairFind{a.B, s.total256, s.total128};
+    if (X1 >= s.total256) sc.at[1] = PairFind{a.B, s.total256, s.total128};
   }
-  __syncthreads();
-  PairWalker w{s_b, s_p256, s_p128, X, X1, single};
-  __syncthreads();
-  return w;
+}
+__device__ __forceinline__ PairWalker pair_walker(const PairFind& f, int X, int X1, bool single) {
+  return PairWalker{f.b, f.p256, f.p128, X, X1, single};
 }
 
 // Most 128-token tiles a call can have with non-overlapping sequences: the
