@@ -768,13 +768,17 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
 // ---------------------------------------------------------------------------
 
 struct PrepItem {
-  int8_t g, s0, nh, ws;  // group, first head slot, heads, ranks
-  int16_t k0;            // first rank
-  int8_t kv[2];          // KV head of each of the item's heads
-  int32_t off;           // byte offset in a sequence's image
+  int32_t src;    // element of B_k at the item's first rank and head
+  int32_t off;    // byte offset in a sequence's image
+  int16_t ld;     // elements between ranks in B_k
+  int8_t ws;      // ranks
+  int8_t kv[2];   // KV head of each of the item's heads
 };
+// A warp's piece of the preparation: 8 ranks of one head (2 KB of image).
+constexpr int kUnitBytes = 8 * kD * 2;
+constexpr int kMaxPrepUnits = kMaxHqTc * 256 / 8;
 
-// The decode step's latent append, done by extra blocks of the preparation
+// The decode step's latent append, done by the first blocks of the preparation
 // launch: z_b = x_b [A_k | A_v] for the batch's new tokens, written to cache
 // row rows[b] (Sec. III-A z = x L; Sec. III-C L_g side by side; Sec. III-D L_v).
 struct StepAppend {
@@ -787,11 +791,12 @@ struct StepAppend {
 };
 
 struct PrepArgs {
-  int n_items;
+  int n_units;                  // pieces of one sequence's image
   int64_t seq_bytes;
-  double om[kD / 2];  // RoPE frequencies, fp64
-  PrepItem item[kMaxItems];
   StepAppend app;
+  RopeFreqs rf;
+  PrepItem item[kMaxItems];
+  uint8_t unit[kMaxPrepUnits];  // item of each piece
 };
 
 constexpr int kAppCols = 16;     // output columns of one GEMV block
@@ -832,9 +837,9 @@ __device__ __forceinline__ void ldmatrix_x4_plain(uint32_t (&r)[4], uint32_t add
 }
 
 constexpr int kAppStages = 6;    // k-steps of a warp in flight
-// Dynamic shared memory of the append blocks: per warp kAppStages stages of a
-// factor tile (512 B) and an x tile (16 tokens x 16 k per token m-tile), then
-// the warps' partial sums.
+// Dynamic shared memory of the append: per warp a ring of stages of a factor
+// tile (512 B) and an x tile (16 tokens x 16 k per token m-tile), then the
+// warps' partial sums.
 __host__ __device__ inline int app_stage_bytes(int batch) { return 512 + ((batch + 15) / 16) * 512; }
 __host__ __device__ inline size_t app_smem_bytes(int batch) {
   return (size_t)kAppWarps * kAppStages * app_stage_bytes(batch) + (size_t)kAppWarps * batch * kAppCols * 4;
@@ -935,87 +940,102 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
   }
 }
 
-// One block writes one factor item: [nh heads][2 halves][ws rank rows]
-// [64 columns] bf16, 128B-swizzled (16-byte chunk c of row r stored at chunk
-// c ^ (r % 8); every half starts on a 1024-byte swizzle atom).
-// Key mode: columns of B_g[:, slot].  Query-folded mode (the block's row of
-// the grid covers kPrepSeqs sequences b): columns 2i and 2i+1 are
+// Factor images: items of [nh heads][2 halves][ws rank rows][64 columns] bf16,
+// 128B-swizzled (16-byte chunk c of row r stored at chunk c ^ (r % 8); every half
+// starts on a 1024-byte swizzle atom).
+// Key mode: columns of B_g[:, slot].  Query-folded mode: columns 2i and 2i+1 are
 //   a_i B[:, i] + b_i B[:, i+64]  and  b_i B[:, i] - a_i B[:, i+64]
-// with (a, b) the halves of RoPE(q_{b,h}, L_b - 1) * log2(e)/sqrt(d); each
-// thread loads its B_g values once and writes them folded for every sequence.
-// Blocks in rows after the preparation rows do the decode step's latent
-// append (step_append_block), when the call has one.
+// with (a, b) the halves of RoPE(q_{b,h}, L_b - 1) * log2(e)/sqrt(d).
+// The launch's first blocks do the fused append, if there is one (16 output
+// columns each), the others write eight pieces each: 8 ranks of one head per
+// warp, in query-folded mode for kPrepSeqs sequences.  A warp's loads (factors,
+// queries) are all issued before the first is used, and a lane rotates the four
+// frequency pairs that its columns need.  Bound by latency and the launch: with a
+// whole item per block, fp64 angles and the loads in series it took 10.3 us for
+// one sequence of the 32-head layer and 13 us for 16 (18 MB of images, written to
+// L2).  Small blocks, not one per SM: SMs that have none left take the scores
+// kernel's CTAs, whose set-up then overlaps (one 512-thread block per SM cost the
+// step 4 to 10 us).
 constexpr int kPrepSeqs = 4;
+constexpr int kPrepThreads = 256;
 template <bool kFold>
-__global__ void __launch_bounds__(256) factor_prep_kernel(const LayerTable lt, const DecodeArgs a, const PrepArgs pa,
-                                                          uint8_t* __restrict__ img) {
+__global__ void __launch_bounds__(kPrepThreads, 2)
+    factor_prep_kernel(const LayerTable lt, const DecodeArgs a, const __grid_constant__ PrepArgs pa,
+                       uint8_t* __restrict__ img) {
   griddep_launch();
-  const int prep_rows = kFold ? (a.B + kPrepSeqs - 1) / kPrepSeqs : 1;
-  if ((int)blockIdx.y >= prep_rows) {  // a block of the fused decode-step append
-    const int blk = (blockIdx.y - prep_rows) * gridDim.x + blockIdx.x;
-    if (blk < pa.app.n_blocks) step_append_block(lt, a, pa.app, blk);
+  if ((int)blockIdx.x < pa.app.n_blocks) {
+    step_append_block(lt, a, pa.app, blockIdx.x);
     return;
   }
-  const int n = blockIdx.x, bs0 = blockIdx.y * kPrepSeqs;
-  const int nbs = kFold ? min(kPrepSeqs, a.B - bs0) : 1;
-  const PrepItem it = pa.item[n];
-  const int g = it.g, ws = it.ws, nh = it.nh;
-  __shared__ float qa[kPrepSeqs][2][kD / 2], qb[kPrepSeqs][2][kD / 2];
-  __shared__ int live[kPrepSeqs];
-  if (kFold) {
-    for (int e = threadIdx.x; e < nbs * nh * (kD / 2); e += blockDim.x) {
-      const int sb = e / (nh * (kD / 2)), hh = (e / (kD / 2)) % nh, i = e % (kD / 2);
-      const int b = bs0 + sb;
-      const int L = valid_len(a.seq_len, a.seq_start, b, a.n_rows);
-      if (hh == 0 && i == 0) live[sb] = L > 0;  // no tile of an empty sequence is ever processed
-      const int kv = it.kv[hh];
-      // angle (L-1) w_i reduced mod 2 pi in fp64, sine and cosine in fp32
-      const double ang = (double)max(L - 1, 0) * pa.om[i];
-      float sn, cs;
-      sincosf((float)(ang - 6.283185307179586 * rint(ang * 0.15915494309189535)), &sn, &cs);
-      const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(a.q) + ((int64_t)b * lt.Hq + kv) * kD;
-      const float x1 = __bfloat162float(q[i]), x2 = __bfloat162float(q[i + kD / 2]);
-      const float sc = kLog2e * rsqrtf((float)kD);
-      qa[sb][hh][i] = (x1 * cs - x2 * sn) * sc;
-      qb[sb][hh][i] = (x1 * sn + x2 * cs) * sc;
-    }
-    __syncthreads();
-  }
-  const int64_t ld = (int64_t)lt.grp_nh[g] * kD;
-  // thread -> (head, row, 8-column chunk): nh x ws rows x 16 chunks (2 halves x 8)
-  for (int idx = threadIdx.x; idx < nh * ws * 16; idx += blockDim.x) {
-    const int hh = idx / (ws * 16), r = (idx >> 4) % ws, ch = idx & 15;
-    const int half = ch >> 3, c8 = ch & 7;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int groups = kFold ? (a.B + kPrepSeqs - 1) / kPrepSeqs : 1;
+  // lane: columns of pairs [4 ch, 4 ch + 4), i.e. 16-byte chunk c8 of a half, of ranks rl, rl + 2, ..
+  const int ch = lane & 15, half = ch >> 3, c8 = ch & 7, rl = lane >> 4;
+  const int w = (blockIdx.x - pa.app.n_blocks) * (kPrepThreads / 32) + warp;
+  if (w < groups * pa.n_units) {
+    const int u = w % pa.n_units, bs0 = w / pa.n_units * kPrepSeqs;
+    const PrepItem it = pa.item[pa.unit[u]];
+    const int ws = it.ws, r8 = (u * kUnitBytes - it.off) / kUnitBytes;  // eight-rank group of the item's heads
+    const int hh = r8 / (ws / 8), r0 = r8 % (ws / 8) * 8;
     const __nv_bfloat16* __restrict__ Bs =
-        static_cast<const __nv_bfloat16*>(a.Bk) + lt.grp_boff[g] + (it.s0 + hh) * kD + (int64_t)(it.k0 + r) * ld;
-    const int64_t doff = it.off + (hh * 2 + half) * (ws * 128) + r * 128 + ((c8 ^ (r & 7)) << 4);
+        static_cast<const __nv_bfloat16*>(a.Bk) + it.src + hh * kD + (int64_t)(r0 + rl) * it.ld;
+    uint8_t* dst = img + it.off + (hh * 2 + half) * (ws * 128) + (r0 + rl) * 128;
     if (kFold) {
-      // output columns col = 64*half + 8*c8 + t, t even/odd -> pair i = col/2 = 32*half + 4*c8 + t/2:
-      // the x-halves B[:, i] and y-halves B[:, i+64] of four pairs, one 8-byte load each
-      const int i0 = 32 * half + 4 * c8;
-      const uint2 xr = *reinterpret_cast<const uint2*>(Bs + i0);
-      const uint2 yr = *reinterpret_cast<const uint2*>(Bs + kD / 2 + i0);
-      const __nv_bfloat16* xh = reinterpret_cast<const __nv_bfloat16*>(&xr);
-      const __nv_bfloat16* yh = reinterpret_cast<const __nv_bfloat16*>(&yr);
-      float x[4], y[4];
+      // the x-halves B[:, i] and y-halves B[:, i+64] of four pairs in four ranks
+      uint2 xr[4], yr[4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        x[t] = __bfloat162float(xh[t]);
-        y[t] = __bfloat162float(yh[t]);
+      for (int k = 0; k < 4; ++k) {
+        xr[k] = *reinterpret_cast<const uint2*>(Bs + (int64_t)(2 * k) * it.ld + 4 * ch);
+        yr[k] = *reinterpret_cast<const uint2*>(Bs + (int64_t)(2 * k) * it.ld + kD / 2 + 4 * ch);
       }
-      for (int sb = 0; sb < nbs; ++sb) {
-        if (!live[sb]) continue;
-        uint4 out;
-        __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&out);
+      float q1[kPrepSeqs][4], q2[kPrepSeqs][4];
+      int len[kPrepSeqs];
+#pragma unroll
+      for (int sb = 0; sb < kPrepSeqs; ++sb) {
+        len[sb] = 0;  // no tile of an empty sequence is ever processed
+        if (bs0 + sb >= a.B) continue;
+        len[sb] = valid_len(a.seq_len, a.seq_start, bs0 + sb, a.n_rows);
+        const __nv_bfloat16* q =
+            static_cast<const __nv_bfloat16*>(a.q) + ((int64_t)(bs0 + sb) * lt.Hq + it.kv[hh]) * kD + 4 * ch;
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-          const float qa_ = qa[sb][hh][i0 + t], qb_ = qb[sb][hh][i0 + t];
-          o2[t] = __floats2bfloat162_rn(fmaf(qa_, x[t], qb_ * y[t]), fmaf(qb_, x[t], -qa_ * y[t]));
+          q1[sb][t] = __bfloat162float(q[t]);
+          q2[sb][t] = __bfloat162float(q[kD / 2 + t]);
         }
-        *reinterpret_cast<uint4*>(img + (int64_t)(bs0 + sb) * pa.seq_bytes + doff) = out;
+      }
+      const float sc = kLog2e * rsqrtf((float)kD);
+#pragma unroll
+      for (int sb = 0; sb < kPrepSeqs; ++sb) {
+        if (len[sb] <= 0) continue;
+        float qa[4], qb[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          float sn, cs;
+          rope_sincos(pa.rf.f[4 * ch + t], (uint32_t)(len[sb] - 1), sn, cs);
+          qa[t] = (q1[sb][t] * cs - q2[sb][t] * sn) * sc;
+          qb[t] = (q1[sb][t] * sn + q2[sb][t] * cs) * sc;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 x01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&xr[k].x));
+          const float2 x23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&xr[k].y));
+          const float2 y01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&yr[k].x));
+          const float2 y23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&yr[k].y));
+          const uint4 out = make_uint4(
+              pack_bf16x2(fmaf(qa[0], x01.x, qb[0] * y01.x), fmaf(qb[0], x01.x, -qa[0] * y01.x)),
+              pack_bf16x2(fmaf(qa[1], x01.y, qb[1] * y01.y), fmaf(qb[1], x01.y, -qa[1] * y01.y)),
+              pack_bf16x2(fmaf(qa[2], x23.x, qb[2] * y23.x), fmaf(qb[2], x23.x, -qa[2] * y23.x)),
+              pack_bf16x2(fmaf(qa[3], x23.y, qb[3] * y23.y), fmaf(qb[3], x23.y, -qa[3] * y23.y)));
+          *reinterpret_cast<uint4*>(dst + (int64_t)(bs0 + sb) * pa.seq_bytes + 256 * k +
+                                    ((c8 ^ (rl + 2 * k)) << 4)) = out;  // rank row (rl + 2 k) mod 8 of its atom
+        }
       }
     } else {
-      *reinterpret_cast<uint4*>(img + doff) = *reinterpret_cast<const uint4*>(Bs + 64 * half + 8 * c8);
+      uint4 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const uint4*>(Bs + (int64_t)(2 * k) * it.ld + 8 * ch);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) *reinterpret_cast<uint4*>(dst + 256 * k + ((c8 ^ (rl + 2 * k)) << 4)) = v[k];
     }
   }
 }
@@ -1129,14 +1149,13 @@ cudaError_t launch_mode(const LayerTable& lt, const DecodeArgs& a, const Maps& m
                         const PrepArgs& pa, cudaStream_t s) {
   cudaError_t e = set_smem_attr<kFold>();
   if (e != cudaSuccess) return e;
-  const int prep_rows = kFold ? (a.B + kPrepSeqs - 1) / kPrepSeqs : 1;
-  const int app_rows = (pa.app.n_blocks + pa.n_items - 1) / pa.n_items;
   const size_t app_smem = pa.app.n_blocks ? app_smem_bytes(a.B) : 0;
   if (app_smem) {
     e = cudaFuncSetAttribute(factor_prep_kernel<kFold>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem);
     if (e != cudaSuccess) return e;
   }
-  factor_prep_kernel<kFold><<<dim3(pa.n_items, prep_rows + app_rows), 256, app_smem, s>>>(
+  const int pieces = pa.n_units * (kFold ? (a.B + kPrepSeqs - 1) / kPrepSeqs : 1), per = kPrepThreads / 32;
+  factor_prep_kernel<kFold><<<pa.app.n_blocks + (pieces + per - 1) / per, kPrepThreads, app_smem, s>>>(
       lt, a, pa, static_cast<uint8_t*>(a.extra));
   e = hook_launched(a.hook, s);
   if (e != cudaSuccess) return e;
@@ -1217,15 +1236,15 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
         if (item >= kMaxItems) return false;
         const int w = gs.w[p], bytes = nh * w * 256;
         PrepItem& pi = pa.item[item];
-        pi.g = (int8_t)g;
-        pi.s0 = (int8_t)s0;
+        pi.src = (int32_t)(lt.grp_boff[g] + (int64_t)gs.k[p] * lt.grp_nh[g] * kD + s0 * kD);
+        pi.ld = (int16_t)(lt.grp_nh[g] * kD);
         for (int hh = 0; hh < nh; ++hh)
           for (int h = 0; h < lt.Hkv; ++h)
             if (lt.head_group[h] == g && lt.head_slot[h] == s0 + hh) pi.kv[hh] = (int8_t)h;
-        pi.nh = (int8_t)nh;
         pi.ws = (int8_t)w;
-        pi.k0 = gs.k[p];
         pi.off = off;
+        if ((off + bytes) / kUnitBytes > kMaxPrepUnits) return false;
+        for (int u = off / kUnitBytes; u < (off + bytes) / kUnitBytes; ++u) pa.unit[u] = (uint8_t)item;
         ta.item[item] = (uint32_t)off | ((uint32_t)(bytes >> 12) << 26);
         off += bytes;
         ++item;
@@ -1235,16 +1254,10 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
   ta.n_units = unit;
   ta.uitem[unit] = (int16_t)item;
   ta.n_items = item;
-  pa.n_items = item;
+  pa.n_units = off / kUnitBytes;
   pa.seq_bytes = off;
   ta.fimg_seq_bytes = off;
   return true;
-}
-
-// RoPE frequencies w_i = theta^(-2i/d) in fp64 (positions reach 1e5 and more,
-// so the angle t w_i needs the extra precision before its reduction mod 2 pi).
-void rope_freqs(float theta, double* om) {
-  for (int i = 0; i < kD / 2; ++i) om[i] = std::exp2(-2.0 * i / kD * std::log2((double)theta));
 }
 
 // Workspace layout of the tensor-core path (after the split partials):
@@ -1307,8 +1320,7 @@ cudaError_t launch_decode_tc(const LayerTable& lt, const DecodeArgs& a, const Tc
     pa.app.D = app->D;
     pa.app.n_blocks = (lt.Rk + lt.rv) / kAppCols;
   }
-  ta.rf = rope_freqs_of(a.theta, kD);
-  rope_freqs(a.theta, pa.om);
+  ta.rf = pa.rf = rope_freqs_of(a.theta, kD);
   const ExtraLayout xl = extra_layout(lt, a.B, a.n_rows);
   uint8_t* base = static_cast<uint8_t*>(a.extra);
   ta.n_pairs = a.n_items / 2;
