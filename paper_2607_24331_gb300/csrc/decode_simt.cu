@@ -186,12 +186,15 @@ __global__ void __launch_bounds__(kThreads, QP == 1 ? kBlocksPerSm : 1)
       buf ^= 1;
       if (t0 + kTok < t_end) load_c(t0 + kTok, buf);
       // reconstruction: k_t[e] = sum_k c_t[k] B_g[k][slot*D + e], four ranks at a
-      // time; even and odd ranks are summed apart (half the length of the rounding chain)
-      float ka[TPT][4], kb[TPT][4];
+      // time; every kChains-th rank is summed apart (shorter rounding chains)
+      constexpr int kChains = TPT == 2 ? 4 : 2;
+      float kc_[kChains][TPT][4];
 #pragma unroll
-      for (int u = 0; u < TPT; ++u)
+      for (int q = 0; q < kChains; ++q)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ka[u][j] = kb[u][j] = 0.f;
+        for (int u = 0; u < TPT; ++u)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) kc_[q][u][j] = 0.f;
 #pragma unroll 2
       for (int k = 0; k < r; k += 4) {
         float4 cv[TPT];
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, QP == 1 ? kBlocksPerSm : 1)
 #pragma unroll
           for (int u = 0; u < TPT; ++u) {
             const float w = q == 0 ? cv[u].x : (q == 1 ? cv[u].y : (q == 2 ? cv[u].z : cv[u].w));
-            float(&kk)[4] = (q & 1) ? kb[u] : ka[u];
+            float(&kk)[4] = kc_[q % kChains][u];
             kk[0] = fmaf(w, lo.x, kk[0]);
             kk[1] = fmaf(w, lo.y, kk[1]);
             kk[2] = fmaf(w, hi.x, kk[2]);
@@ -212,10 +215,13 @@ __global__ void __launch_bounds__(kThreads, QP == 1 ? kBlocksPerSm : 1)
           }
         }
       }
+      float ka[TPT][4];
 #pragma unroll
       for (int u = 0; u < TPT; ++u)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ka[u][j] += kb[u][j];
+        for (int j = 0; j < 4; ++j)
+          ka[u][j] = kChains == 4 ? (kc_[0][u][j] + kc_[1][u][j]) + (kc_[2 % kChains][u][j] + kc_[3 % kChains][u][j])
+                                  : kc_[0][u][j] + kc_[1][u][j];
       // RoPE at the token's position, then the scores (log2 units): this thread's
       // four columns, summed over the column groups
 #pragma unroll
