@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kAThreads, 1)
   const PairScan scan = pair_scan(a, sm.sc);
   const int NP = scan.total256;
   DCK_AB_TRACE(4);
-  const PSplit sp(NP, pl.P);
+  const PSplit sp(NP, pl.P, a.fine_below);
   pl.NPm = sp.NPm;
   const bool fits = scan.total128 <= aa.max_tiles;  // else the scores kernel has reported the input
   const int X0 = fits ? sp.main_begin(pl.pr, pl.P) : 0;
@@ -282,11 +282,19 @@ __global__ void __launch_bounds__(kAThreads, 1)
           }
           if (!(ok = wait_slots(sm.p_empty, kNP, p_cnt, 1, lane, abort_flag))) break;
           {
+            // the P image first: the decision below needs the maxima, a round trip later
+            // (the barrier completes only with the arrival that follows it)
+            const int sl = p_cnt % kNP;
+            if (lane == 0) bulk_load(sm.p[sl], aa.pglob + x * pbytes, pbytes, &sm.p_full[sl], pol);
             // does any head's reference max rise at this tile?  (decided here, once,
             // for the MMA thread; the epilogue warps take the same decision)
             bool need = false;
             const float m_now = have_pf ? m_pf : (lane < Hq ? aa.mglob[x * Hq + lane] : 0.f);
             if (i > 0) need = __any_sync(0xffffffffu, m_now > m_prev);
+            if (lane == 0) {
+              sm.pneed[sl] = need ? 1 : 0;
+              mbar_expect_tx(&sm.p_full[sl], pbytes);
+            }
             have_pf = true;
             if (i + 1 < seg.n) {
               m_pf = lane < Hq ? aa.mglob[seg.x(i + 1) * Hq + lane] : 0.f;
@@ -297,12 +305,6 @@ __global__ void __launch_bounds__(kAThreads, 1)
               else have_pf = false;
             }
             m_prev = m_now;
-            if (lane == 0) {
-              const int sl = p_cnt % kNP;
-              sm.pneed[sl] = need ? 1 : 0;
-              mbar_expect_tx(&sm.p_full[sl], pbytes);
-              bulk_load(sm.p[sl], aa.pglob + x * pbytes, pbytes, &sm.p_full[sl], pol);
-            }
           }
           __syncwarp();
           DCK_AB_TRACE(1);

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   }
 
   // tiles: pair tiles (tensor-core path) or kSimtTile-token tiles; items: CTA pairs or CTAs
-  const bool pairs = a.split_extra != 0;
+  const bool pairs = a.fine_below != 0;
   const int n_it = pairs ? a.n_items / 2 : a.n_items;
   // tiles per sequence (every thread a share), then an exclusive prefix by warp 0
   const int tile = pairs ? 2 * kTile : kSimtTile;
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   // Partials of sequence b: the items whose main tiles (the first NTm, split
   // evenly in whole tiles) cover b's; on the tensor-core path also the extra
   // pair tiles of b (x >= NTm), two slots (halves) per item and per extra tile.
-  const int NTm = main_tiles(NT, n_it, pairs);
+  const int NTm = main_tiles(NT, n_it, a.fine_below);
   for (int c = threadIdx.x; c <= n_it; c += kThreads) ibeg[c] = item_begin(c, NTm, n_it);
   if (threadIdx.x < nrow) {
     const int b = b0 + threadIdx.x / qpg;

@@ -50,7 +50,8 @@ struct DecodeArgs {
   int64_t n_rows;
   int32_t B;
   int32_t n_items;
-  int32_t split_extra;  // tensor-core path: the pair-tile plan of tc_common.cuh (n_items = 2 x CTA pairs)
+  int32_t fine_below;  // tensor-core path: the pair-tile plan of tc_common.cuh (n_items = 2 x CTA pairs) with this
+                       // threshold of its fine split; 0: CUDA-core path
   float theta;
   float* part_u;   // [n_slots, Hq, rv]
   float* part_ml;  // [n_slots, Hq, 2]  (running max in log2 units, sum)
@@ -190,13 +191,18 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 
 // Tiles [0, main_tiles) are split in contiguous whole-tile ranges over the
-// n_items work items; with `split_extra` (tensor-core path) and fewer than
-// kFineSplitBelow tiles per item, only n_items * floor(NT / n_items) of them,
-// the rest ("extra tiles") being shared out more finely (see tc_common.cuh).
-constexpr int kFineSplitBelow = 8;
-__host__ __device__ __forceinline__ int main_tiles(int NT, int n_items, bool split_extra) {
-  return split_extra && NT / n_items < kFineSplitBelow ? NT / n_items * n_items : NT;
+// n_items work items; with fewer than `fine_below` tiles per item, only n_items *
+// floor(NT / n_items) of them, the rest ("extra tiles") being shared out more
+// finely (see tc_common.cuh; 0 on the CUDA-core path).
+__host__ __device__ __forceinline__ int main_tiles(int NT, int n_items, int fine_below) {
+  return NT / n_items < fine_below ? NT / n_items * n_items : NT;
 }
+// An extra tile costs each of its CTAs a segment (a tile end, a partial); a whole
+// one more on some CTAs costs the call a tile's time.  32-head MHA layer, 32 ragged
+// sequences, 9.9 tiles per CTA pair: 300 us shared out, 311 not.  With several query
+// heads per KV head a segment also rotates its queries again: 8 x 32768 tokens,
+// 13.5 tiles per pair: 210 us shared out, 202 not.
+inline int fine_split_below(int qpg) { return qpg == 1 ? 32 : 8; }
 
 // The item whose tile range contains tile x (0 <= x < NT).
 __device__ __forceinline__ int item_of_tile(int x, int NT, int n_items) {

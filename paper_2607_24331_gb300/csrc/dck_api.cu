@@ -305,7 +305,7 @@ dck_status decode_call(const dck_layer_desc* desc, const void* q, const void* kc
   hook.ev = t_events;
   hook.n_ev = t_n_events;
   a.hook = &hook;
-  a.split_extra = use_tc ? 1 : 0;
+  a.fine_below = use_tc ? fine_split_below(lt.qpg) : 0;
   // the tensor-core kernels run on the pairs' SMs
   a.n_items = use_tc ? 2 * pairs : simt_items(lt, desc->dtype, batch, n_rows, sms);
   if (use_tc) e = launch_decode_tc(lt, a, app, s);

@@ -110,12 +110,6 @@ constexpr int kEpiWarps = 16;
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kThreadsTc = 32 * kCtlWarps + kEpiThreads;
 constexpr int kFreqW = kD / 2 / 4;  // RoPE pairs of a frequency quarter
-// Latent tiles prefetched toward L2 ahead of their loads: two in query-folded
-// mode; none in key mode, whose TMA loads keep enough of the latent stream in
-// flight themselves and whose prefetches only competed with it (7B GQA layer,
-// 0 / 1 / 2 / 4 tiles ahead: 298 / 301 / 306 / 315 us per step)
-template <bool kFold>
-__host__ __device__ constexpr int prefetch_ahead() { return kFold ? 2 : 0; }
 constexpr float kRescaleThr = 8.f;  // log2 units: probabilities stay <= 256
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kKCols = 256;    // TMEM columns of one key accumulator
@@ -278,7 +272,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   __shared__ PairScratch sc;
   const PairScan scan = pair_scan(a, sc);
   const int NP = scan.total256, NT128 = scan.total128;
-  const PSplit sp(NP, P);
+  const PSplit sp(NP, P, a.fine_below);
   // the per-tile stores are sized for non-overlapping sequences; more tiles
   // than that is reported as invalid input and nothing is computed
   const bool fits = NT128 <= ta.max_tiles;
@@ -319,48 +313,24 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   // Programmatic dependent launch: every thread lets the absorption kernel
   // launch only after it has seen the preparation kernel complete, so that
   // the absorption's value loads ahead of its own grid-dependency wait find
-  // the rows a decode step appends.  The latent producer first moves its
-  // first tiles toward L2.
-  if (warp != 0) {
-    griddep_wait();
-    griddep_launch();
-  }
+  // the rows a decode step appends.
+  griddep_wait();
+  griddep_launch();
 
   if (warp == 0) {
     // ---- latent pieces (this CTA's 128 rows of each), issued as soon as their
-    // slots are free ---------------------------------------------------------
+    // slots are free.  No L2 prefetch runs ahead of them: two tiles ahead of every
+    // CTA, it queued in HBM before the first tile's loads and cost 3 to 4 % of the
+    // 32-head layer's steps ------------------------------------------------------
     if (has_work) {
       const uint64_t pol = policy_evict_first();
       const bool el = elect_one();
       int slot = 0, fills = 0;  // latent ring: next slot, times round
       bool ok = true;
-      // L2 prefetch of this half's latent rows, prefetch_ahead() tiles ahead of the
-      // loads (across segment boundaries): the TMA loads then find them in L2
-      PairWalker pwalk = walker(0);
-      PSegment pseg = {};
-      int pph = 0, pti = 0;
-      auto prefetch_next = [&]() {
-        if (lane != 0) return;
-        while (pti >= pseg.ntiles) {
-          pti = 0;
-          if (pph >= 2) return;
-          if (!pwalk.next(a, pseg)) {
-            pseg.ntiles = 0;
-            if (++pph < 2) pwalk = walker(pph);
-          }
-        }
-        const int64_t r0 = pseg.row0 + pseg.t0(pti++, hr);
-        const int64_t nr = a.n_rows - r0 < kTile ? a.n_rows - r0 : (int64_t)kTile;
-        if (nr > 0) prefetch_l2(static_cast<const __nv_bfloat16*>(a.kc) + r0 * lt.Rk, (uint32_t)(nr * lt.Rk * 2));
-      };
-      for (int q = 0; q < prefetch_ahead<kFold>(); ++q) prefetch_next();
-      griddep_wait();  // the preparation launch may append the step's own latents
-      griddep_launch();
       for (int ph = 0; ph < 2 && ok; ++ph)
         for (PairWalker walk = walker(ph); ok && walk.next(a, seg);) {
           for (int i = 0; i < seg.ntiles && ok; ++i) {
             const int64_t yrow = seg.row0 + seg.t0(i, hr);
-            prefetch_next();
             int ua, ub;
             units_of(ph, seg.X0 + i, ua, ub);
             for (int g = 0; g < lt.G && ok; ++g) {
@@ -383,9 +353,6 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
           }
         }
       if (!ok && lane == 0) stop_peer();
-    } else {
-      griddep_wait();
-      griddep_launch();
     }
   } else if (warp == 2) {
     // ---- factor items: this CTA's head of each (or its half of a lone head's),

@@ -67,7 +67,7 @@ __device__ __forceinline__ bool wait_slots(uint64_t* empty, int depth, int cnt, 
 // the rest to its odd CTA (half 1).  The flattened pair-tile list (sequences in
 // order) is split over the pairs: pair p takes the contiguous range
 // [floor(p NPm / P), floor((p+1) NPm / P)) of the first NPm tiles; with fewer
-// than kFineSplitBelow tiles per pair the R = NP - NPm left over are shared
+// than fine_split_below() tiles per pair the R = NP - NPm left over are shared
 // out by units (groups of heads) instead, pair p taking units
 // [floor(p R U / P), floor((p+1) R U / P)) of the flattened (extra tile, unit)
 // list.  The absorption kernel's CTA c = 2p + h follows half h of pair p's
@@ -105,7 +105,8 @@ __host__ __device__ inline int64_t pair_slot_count(int P, int B, int64_t n_rows)
 // Split of NP pair tiles over P pairs (see above).
 struct PSplit {
   int NP, NPm, R;
-  __host__ __device__ PSplit(int np, int P) : NP(np), NPm(np / P < kFineSplitBelow ? np / P * P : np), R(np - NPm) {}
+  __host__ __device__ PSplit(int np, int P, int fine_below)
+      : NP(np), NPm(main_tiles(np, P, fine_below)), R(np - NPm) {}
   // floor(p NPm / P): the tiles of caches of fewer than 2^31 rows times the pairs of a GPU stay below 2^32
   __host__ __device__ int main_begin(int p, int P) const {
     return (int)((uint32_t)p * (uint32_t)NPm / (uint32_t)P);
