@@ -87,13 +87,14 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   extern __shared__ __align__(16) uint8_t smem_c[];
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
+  const int lsplit = split == kMaxSplit ? 3 : 2;  // split = 2^lsplit
   const int B = a.B;
   const int qpg = lt.qpg, rv = lt.rv, Hq = lt.Hq;
-  const int h = blockIdx.x / split;
+  const int h = blockIdx.x >> lsplit;
   const int b0 = blockIdx.y * bchunk;
   const int nb = min(bchunk, B - b0);
   const int nrow = nb * qpg;
-  const int rr = rv / split;            // rows of u / B_v owned by this CTA (a multiple of 4)
+  const int rr = rv >> lsplit;            // rows of u / B_v owned by this CTA (a multiple of 4)
   const int r0 = rank * rr;
   DCK_CB_TRACE(99);
 
@@ -179,21 +180,22 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   asm volatile("griddepcontrol.wait;" ::: "memory");
   DCK_CB_TRACE(2);
 
-  // (1) one warp per row: each live partial's slot, reference max m (log2
+  // (1) sixteen lanes per row, all rows at once: each live partial's slot, reference max m (log2
   // units) and sum l, their loads all in flight together (a lane per
   // partial); then M = max m, the weights 2^(m - M) and 1/l; (2) this CTA's
   // rows of u as the weighted sum, all of a row's loads independent.
   {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nps = pairs ? 2 : 1;  // slots per item or extra tile
-    for (int i = warp; i < nrow; i += kThreads / 32) {
-      const int b = b0 + i / qpg, j = h * qpg + i % qpg;
-      const int c0 = rc[4 * i], nm = rc[4 * i + 1], e0 = rc[4 * i + 2];
-      const int ns = nps * (nm + rc[4 * i + 3]);
-      const int n128 = rn128[i];
+    const int l16 = threadIdx.x & 15;
+    const int ps2 = pairs ? 1 : 0;  // log2 of the slots per item or extra tile
+    for (int i = threadIdx.x >> 4; i < kMaxRows; i += kThreads / 16) {  // (whole warps: the shuffles below)
+      const bool on = i < nrow;
+      const int b = on ? b0 + i / qpg : 0, j = on ? h * qpg + i % qpg : 0;
+      const int c0 = on ? rc[4 * i] : 0, nm = on ? rc[4 * i + 1] : 0, e0 = on ? rc[4 * i + 2] : 0;
+      const int ns = on ? (nm + rc[4 * i + 3]) << ps2 : 0;
+      const int n128 = on ? rn128[i] : 0;
       float M = -INFINITY;
-      for (int q = lane; q < ns; q += 32) {
-        const int k = q / nps, hh = q % nps;
+      for (int q = l16; q < ns; q += 16) {
+        const int k = q >> ps2, hh = q & ((1 << ps2) - 1);
         bool live;
         int64_t slot;
         if (k < nm) {  // item c0 + k
@@ -223,16 +225,16 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
         M = fmaxf(M, m);
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+      for (int o = 8; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
       float l = 0.f;
-      for (int q = lane; q < ns; q += 32) {  // entries this lane wrote itself
+      for (int q = l16; q < ns; q += 16) {  // entries this lane wrote itself
         const float wq = M == -INFINITY ? 0.f : exp2f(pw[(size_t)i * cap + q] - M);  // 0 for slots not live
         pw[(size_t)i * cap + q] = wq;
         l = fmaf(wq, pl[(size_t)i * cap + q], l);
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-      if (lane == 0) {
+      for (int o = 8; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (on && l16 == 0) {
         sinv[i] = l > 0.f ? 1.f / l : 0.f;
         pn[i] = ns;
       }
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   cp_async_wait_all();
   __syncthreads();
   DCK_CB_TRACE(5);
-  const int share = kMaxRows * D / split;
+  const int share = kMaxRows * D >> lsplit;
   if constexpr (std::is_same<T, __nv_bfloat16>::value && D == 128) {
     // partial o over this CTA's rows of B_v on the tensor cores: o[16 x 128] =
     // u[16 x rr] B_v[rr x 128], mma m16n8k8 tf32 (B_v's bf16 converts exactly;
@@ -309,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
         const int i = gid + 8 * (q >> 1), col = 16 * warp + 8 * nt + 2 * tig + (q & 1);
         if (i < nrow) {
           const int e = i * D + col;
-          cluster.map_shared_rank(so, e % split)[rank * share + e / split] = acc[nt][q];
+          cluster.map_shared_rank(so, e & (split - 1))[rank * share + (e >> lsplit)] = acc[nt][q];
         }
       }
   } else {
@@ -350,7 +352,7 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
         const int e = i * D + 2 * cp + t;
-        cluster.map_shared_rank(so, e % split)[rank * share + e / split] = acc[q][t];
+        cluster.map_shared_rank(so, e & (split - 1))[rank * share + (e >> lsplit)] = acc[q][t];
       }
   }
   }
