@@ -51,7 +51,7 @@ constexpr int kMaxGroupsP = 16;
 // epilogue of one tile overlaps the next tile's MMAs.  Key tiles are rotated in
 // the epilogue (a thread holds one row, both halves of every frequency pair).
 // Pair p takes tiles p, p + P, ... of the list (values of every row tile, then
-// keys: the costliest tiles first).  Four more warps of each CTA rotate and
+// keys: the costliest tiles first).  Six more warps of each CTA rotate and
 // scale the queries into `out`, from where the attention kernel loads them by
 // TMA before it overwrites them with the results: the tensor-bound GEMM hides
 // that pass over q.
@@ -61,9 +61,14 @@ constexpr int kMaxGroupsP = 16;
 // query row).  Whole prefill calls, before and after: 32-head MHA prompt 2 x 4096
 // 1193 -> 738 us, GQA prompt 8192 1228 -> 1041 us, four 300-512 token chunks in a
 // pooled GQA cache 436 -> 268 us, eight MHA prompts of 44-214 tokens 139 -> 75 us.
+// Then with deep loads for the queries, two epilogue warps per lane quadrant and
+// MMAs issued by a uniform warp, the launches alone (cold): MHA prompt 101 + 40 ->
+// 63 + 34 us, GQA prompt 81 + 21 -> 33 + 18 us.
 // ---------------------------------------------------------------------------
 
-constexpr int kRThreads = 320;   // warp 0 TMA, warp 1 MMA/TMEM, warps 2-5 epilogue, warps 6-9 queries
+constexpr int kREpiWarps = 8;    // two per TMEM lane quadrant
+constexpr int kRQWarps = 6;      // queries
+constexpr int kRThreads = 32 * (2 + kREpiWarps + kRQWarps);  // warp 0 TMA, warp 1 MMA/TMEM, epilogue, queries
 constexpr int kRStages = 6;
 constexpr int kRBK = 64;
 constexpr int kRABytes = kTile * kRBK * 2;   // 16 KB: this CTA's 128 latent rows x 64 of K
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
   uint64_t* acc_empty = acc_full + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  int* scan = reinterpret_cast<int*>(smem);            // [2][kRThreads], before the first copy into the ring
+  int* scan = reinterpret_cast<int*>(smem);            // [2][warps], before the first copy into the ring
   int* rpre = reinterpret_cast<int*>(tmem_slot + 2);   // [B + 1] row tiles before sequence b
   int* qpre = rpre + ra.B + 1;                         // [B + 1] queries before sequence b
 
@@ -144,11 +149,12 @@ __global__ void __launch_bounds__(kRThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 8);  // even CTA: the four epilogue warps of both CTAs
+      mbar_init(&acc_empty[b], 2 * kREpiWarps);  // even CTA: the epilogue warps of both CTAs
     }
     *abort_flag = 0;
     fence_mbar_init();
   }
+  griddep_launch();
   if (warp == 1) {
     tmem_alloc_pair(tmem_slot, 512);
     tmem_relinquish_pair();
@@ -162,17 +168,30 @@ __global__ void __launch_bounds__(kRThreads, 1)
       nr += (L + kRRows - 1) / kRRows;
       nq += L ? ra.q_len[b] : 0;
     }
-    scan[tid] = nr;
-    scan[kRThreads + tid] = nq;
-    __syncthreads();
-    for (int off = 1; off < kRThreads; off <<= 1) {
-      const int v = tid >= off ? scan[tid - off] : 0, w = tid >= off ? scan[kRThreads + tid - off] : 0;
-      __syncthreads();
-      scan[tid] += v;
-      scan[kRThreads + tid] += w;
-      __syncthreads();
+    int ir = nr, iq = nq;  // inclusive over the warp, then the totals of the warps before
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, ir, o), w = __shfl_up_sync(0xffffffffu, iq, o);
+      if (lane >= o) {
+        ir += v;
+        iq += w;
+      }
     }
-    int r = scan[tid] - nr, q = scan[kRThreads + tid] - nq;
+    if (lane == 31) {
+      scan[warp] = ir;
+      scan[kRThreads / 32 + warp] = iq;
+    }
+    __syncthreads();
+    int r = ir - nr, q = iq - nq, tr = 0, tq = 0;
+    for (int w = 0; w < kRThreads / 32; ++w) {
+      const int vr = scan[w], vq = scan[kRThreads / 32 + w];
+      if (w < warp) {
+        r += vr;
+        q += vq;
+      }
+      tr += vr;
+      tq += vq;
+    }
     for (int b = b0; b < b0 + per && b < ra.B; ++b) {
       const int L = prefill_len(ra.seq_len, ra.seq_start, ra.q_len, b, ra.n_rows, ra.qmax, ra.max_len);
       rpre[b] = r;
@@ -181,8 +200,8 @@ __global__ void __launch_bounds__(kRThreads, 1)
       q += L ? ra.q_len[b] : 0;
     }
     if (tid == 0) {
-      rpre[ra.B] = scan[kRThreads - 1];
-      qpre[ra.B] = scan[2 * kRThreads - 1];
+      rpre[ra.B] = tr;
+      qpre[ra.B] = tq;
     }
   }
   tc_fence_before();
@@ -205,65 +224,78 @@ __global__ void __launch_bounds__(kRThreads, 1)
 
   if (warp == 0) {
     // ---- TMA producer (both CTAs): this CTA's latent rows and its half of the factor columns
-    if (lane == 0) {
-      const uint64_t pol = policy_evict_last();
-      int64_t it = 0;
-      bool ok = true;
-      for (int64_t t = pair; t < n_tiles && ok; t += P) {
-        int rt;
-        const RCol& c = tile_at(t, rt);
-        const int b = seq_of_tile(rpre, ra.B, rt);
-        const int32_t y = (int32_t)(ra.seq_start[b] + (int64_t)(rt - rpre[b]) * kRRows + hr * kTile);
-        const CUtensorMap* am = c.g >= 0 ? &maps.ka[c.g] : &maps.va;
-        const CUtensorMap* bm = c.g >= 0 ? &maps.kb[c.g] : &maps.vb;
-        const int half = c.w / 2, nbx = half / 64;
-        for (int k0 = 0; k0 < c.k; k0 += kRBK, ++it) {
-          const int s = (int)(it % kRStages);
-          if (it >= kRStages && !(ok = mbar_wait(&empty[s], (uint32_t)(((it / kRStages) - 1) & 1), abort_flag))) break;
-          uint8_t* as = smem + s * kRStageBytes;
+    const bool el = elect_one();
+    const uint64_t pol = policy_evict_last();
+    int st = 0, fills = 0;  // next stage, times round
+    bool ok = true;
+    for (int64_t t = pair; t < n_tiles && ok; t += P) {
+      int rt;
+      const RCol& c = tile_at(t, rt);
+      const int b = seq_of_tile(rpre, ra.B, rt);
+      const int32_t y = (int32_t)(ra.seq_start[b] + (int64_t)(rt - rpre[b]) * kRRows + hr * kTile);
+      const CUtensorMap* am = c.g >= 0 ? &maps.ka[c.g] : &maps.va;
+      const CUtensorMap* bm = c.g >= 0 ? &maps.kb[c.g] : &maps.vb;
+      const int half = c.w / 2, ck = c.k, x0 = c.n0 + hr * half;
+      for (int k0 = 0; k0 < ck; k0 += kRBK) {
+        if (fills && !(ok = wwait(&empty[st], (uint32_t)((fills - 1) & 1), abort_flag))) break;
+        if (el) {
+          uint8_t* as = smem + st * kRStageBytes;
           uint8_t* bs = as + kRABytes;
-          if (leader) mbar_expect_tx(&full[s], 2u * (uint32_t)(kRABytes + nbx * kRBK * 64 * 2));
-          tma_load_2d_pair(as, am, lead(&full[s]), k0, y, pol);
-          for (int bx = 0; bx < nbx; ++bx)
-            tma_load_2d_pair(bs + bx * (kRBK * 64 * 2), bm, lead(&full[s]), c.n0 + hr * half + 64 * bx, k0, pol);
+          const uint32_t bar = lead(&full[st]);
+          if (leader) mbar_expect_tx(&full[st], 2u * (uint32_t)(kRABytes + half * kRBK * 2));
+          tma_load_2d_pair(as, am, bar, k0, y, pol);
+          tma_load_2d_pair(bs, bm, bar, x0, k0, pol);
+          if (half > 64) tma_load_2d_pair(bs + kRBK * 64 * 2, bm, bar, x0 + 64, k0, pol);
+        }
+        if (++st == kRStages) {
+          st = 0;
+          ++fills;
         }
       }
-      if (!ok) stop_peer();
     }
+    if (!ok && lane == 0) stop_peer();
   } else if (warp == 1) {
-    // ---- pair MMAs (even CTA, one thread) -------------------------------------
-    if (leader && lane == 0) {
-      int64_t it = 0;
+    // ---- pair MMAs (even CTA): the warp runs the schedule, one lane issues ----
+    if (leader) {
+      const bool el = elect_one();
+      const uint32_t s0 = smem_u32(smem);
+      const uint64_t da = sdesc(s0, 16, 1024, kSw128), db = sdesc(s0 + kRABytes, kRBK * 64 * 2, 1024, kSw128);
+      int st = 0;
+      uint32_t sph = 0;
       bool ok = true;
       int lt = 0;  // tiles of this pair so far
       for (int64_t t = pair; t < n_tiles && ok; t += P, ++lt) {
         int rt;
         const RCol& c = tile_at(t, rt);
-        const int buf = lt & 1;
-        if (lt >= 2 && !(ok = mbar_wait(&acc_empty[buf], (uint32_t)(((lt >> 1) - 1) & 1), abort_flag))) break;
-        tc_fence_after();
-        const uint32_t idesc = idesc_bf16(kRRows, c.w, false, true);
+        const int buf = lt & 1, ck = c.k;
+        if (lt >= 2 && !(ok = wwait(&acc_empty[buf], (uint32_t)(((lt >> 1) - 1) & 1), abort_flag))) break;
+        const uint32_t idesc = c.w == 256 ? idesc_bf16(kRRows, 256, false, true) : idesc_bf16(kRRows, 128, false, true);
         const uint32_t d = tmem + buf * 256;
-        for (int k0 = 0; k0 < c.k; k0 += kRBK, ++it) {
-          const int s = (int)(it % kRStages);
-          if (!(ok = mbar_wait(&full[s], (uint32_t)((it / kRStages) & 1), abort_flag))) break;
+        for (int k0 = 0; k0 < ck; k0 += kRBK) {
+          if (!(ok = wwait(&full[st], sph, abort_flag))) break;
           tc_fence_after();
-          const uint32_t xa = smem_u32(smem + s * kRStageBytes);
-          const uint32_t ba = xa + kRABytes;
-          const int nk = min(kRBK, c.k - k0) / 16;
-          for (int k = 0; k < nk; ++k)
-            umma_f16_pair(d, sdesc(xa + k * 32, 16, 1024, kSw128), sdesc(ba + k * 2048, kRBK * 64 * 2, 1024, kSw128),
-                          idesc, (k0 > 0 || k > 0) ? 1u : 0u);
-          umma_commit_pair(&empty[s]);  // the stage's slots in both CTAs, once these MMAs are done
+          const uint64_t o = (uint64_t)(st * (kRStageBytes >> 4));
+          if (el) {
+#pragma unroll
+            for (int k = 0; k < kRBK / 16; ++k)
+              if (k0 + 16 * k < ck)
+                umma_f16_pair(d, da + o + 2 * k, db + o + 128 * k, idesc, (k0 > 0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(&empty[st]);  // the stage's slots in both CTAs, once these MMAs are done
+          }
+          if (++st == kRStages) {
+            st = 0;
+            sph ^= 1;
+          }
         }
-        if (ok) umma_commit_pair(&acc_full[buf]);
+        if (ok && el) umma_commit_pair(&acc_full[buf]);
       }
-      if (!ok) stop_peer();
+      if (!ok && lane == 0) stop_peer();
     }
     __syncwarp();
-  } else if (warp < 6) {
-    // ---- epilogue (warps 2-5, both CTAs): this CTA's 128 rows of each tile -----
-    const int quad = warp & 3;
+  } else if (warp < 2 + kREpiWarps) {
+    // ---- epilogue (both CTAs): this CTA's 128 rows of each tile, half of the
+    // frequency pairs per warp --------------------------------------------------
+    const int quad = warp & 3, c_lo = (warp - 2) / 4 * (kPD / 4);
     const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
     int lt = 0;
     bool ok = true;
@@ -283,7 +315,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
       const uint32_t acc = tmem + lane_base + buf * 256;
       // frequency pairs (i, i + 64): columns [cc, cc + 16) with [64 + cc, 64 + cc + 16)
 #pragma unroll 1
-      for (int cc = 0; cc < kPD / 2; cc += 16) {
+      for (int cc = c_lo; cc < c_lo + kPD / 4; cc += 16) {
         float sn[16], cs[16];
         if (key) {
 #pragma unroll
@@ -327,39 +359,57 @@ __global__ void __launch_bounds__(kRThreads, 1)
     }
     if (!ok && lane == 0) stop_peer();
   } else if (ra.q) {
-    // ---- queries (warps 6-9): one warp per (sequence, new token); lane = (one of
-    // four heads at a time, frequency pairs [8 c, 8 c + 8)) ----------------------
-    const int nw = 4 * gridDim.x, nq = qpre[ra.B];
+    // ---- queries: one warp per (sequence, new token); lane = (one of four heads
+    // at a time, frequency pairs [8 c, 8 c + 8)).  Bound by the pass over q; the
+    // loads of kQAhead rounds are issued before the first is used (with four
+    // rounds on four warps the pass took longer than the products: 81 us of the
+    // 8-KV-head prompt of 8192 for 134 MB) ---------------------------------------
+    constexpr int kQAhead = 8;
+    const int nw = kRQWarps * gridDim.x, nq = qpre[ra.B];
     const int c8 = lane & 7, hs = lane >> 3;
-    for (int u = 4 * blockIdx.x + warp - 6; u < nq; u += nw) {
+    for (int u = kRQWarps * blockIdx.x + warp - 2 - kREpiWarps; u < nq; u += nw) {
       const int b = seq_of_tile(qpre, ra.B, u), qi = u - qpre[b];
       const uint32_t pos = (uint32_t)(ra.seq_len[b] - ra.q_len[b] + qi);
-      float sn[8], cs[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        rope_sincos(ra.rf.f[8 * c8 + i], pos, sn[i], cs[i]);
-        sn[i] *= ra.qscale;
-        cs[i] *= ra.qscale;
-      }
       const int64_t off = ((int64_t)b * ra.qmax + qi) * ra.Hq * kPD + 8 * c8;
-#pragma unroll 4
-      for (int h = hs; h < ra.Hq; h += 4) {
-        const __nv_bfloat16* src = ra.q + off + h * kPD;
-        const uint4 xv = *reinterpret_cast<const uint4*>(src), yv = *reinterpret_cast<const uint4*>(src + kPD / 2);
-        const uint32_t xs[4] = {xv.x, xv.y, xv.z, xv.w}, ys[4] = {yv.x, yv.y, yv.z, yv.w};
-        uint32_t xo[4], yo[4];
+      float sn[8], cs[8];
+      for (int h0 = hs; h0 < ra.Hq; h0 += 4 * kQAhead) {
+        uint4 xv[kQAhead], yv[kQAhead];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 x = unpack2(xs[i]), y = unpack2(ys[i]);
-          xo[i] = pack2(x.x * cs[2 * i] - y.x * sn[2 * i], x.y * cs[2 * i + 1] - y.y * sn[2 * i + 1]);
-          yo[i] = pack2(x.x * sn[2 * i] + y.x * cs[2 * i], x.y * sn[2 * i + 1] + y.y * cs[2 * i + 1]);
+        for (int r = 0; r < kQAhead; ++r)
+          if (h0 + 4 * r < ra.Hq) {
+            const __nv_bfloat16* src = ra.q + off + (h0 + 4 * r) * kPD;
+            xv[r] = *reinterpret_cast<const uint4*>(src);
+            yv[r] = *reinterpret_cast<const uint4*>(src + kPD / 2);
+          }
+        if (h0 == hs) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            rope_sincos(ra.rf.f[8 * c8 + i], pos, sn[i], cs[i]);
+            sn[i] *= ra.qscale;
+            cs[i] *= ra.qscale;
+          }
         }
-        __nv_bfloat16* dst = ra.qr + off + h * kPD;
-        *reinterpret_cast<uint4*>(dst) = make_uint4(xo[0], xo[1], xo[2], xo[3]);
-        *reinterpret_cast<uint4*>(dst + kPD / 2) = make_uint4(yo[0], yo[1], yo[2], yo[3]);
+#pragma unroll
+        for (int r = 0; r < kQAhead; ++r)
+          if (h0 + 4 * r < ra.Hq) {
+            const uint32_t xs[4] = {xv[r].x, xv[r].y, xv[r].z, xv[r].w}, ys[4] = {yv[r].x, yv[r].y, yv[r].z, yv[r].w};
+            uint32_t xo[4], yo[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float2 x = unpack2(xs[i]), y = unpack2(ys[i]);
+              xo[i] = pack2(x.x * cs[2 * i] - y.x * sn[2 * i], x.y * cs[2 * i + 1] - y.y * sn[2 * i + 1]);
+              yo[i] = pack2(x.x * sn[2 * i] + y.x * cs[2 * i], x.y * sn[2 * i + 1] + y.y * cs[2 * i + 1]);
+            }
+            __nv_bfloat16* dst = ra.qr + off + (h0 + 4 * r) * kPD;
+            *reinterpret_cast<uint4*>(dst) = make_uint4(xo[0], xo[1], xo[2], xo[3]);
+            *reinterpret_cast<uint4*>(dst + kPD / 2) = make_uint4(yo[0], yo[1], yo[2], yo[3]);
+          }
       }
     }
   }
+  // The keys' launch may start while the values' ends (it reads nothing of it); it
+  // is complete only after it, and so are both for the attention that follows.
+  griddep_wait();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
