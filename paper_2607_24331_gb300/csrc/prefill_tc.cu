@@ -461,19 +461,21 @@ int recon_pairs_of_device() {
   return cache[dev];
 }
 
-cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, cudaStream_t s) {
+cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, bool early, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
   cfg.blockDim = dim3(kRThreads);
   cfg.dynamicSmemBytes = recon_smem(ra.B);
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 2 : 1;  // early: only after this call's own first launch
   return cudaLaunchKernelEx(&cfg, recon_kernel, rm, ra);
 }
 
@@ -653,6 +655,7 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  griddep_wait();  // rotated queries, keys and values come from the launches before
   const uint32_t tmem = sm.tmem_base;
   PItems list;
   PItem it;
@@ -1070,7 +1073,7 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
     ra.q = l == 0 ? static_cast<const __nv_bfloat16*>(q) : nullptr;
     std::copy(val, val + ra.n_val, ra.col);
     std::copy(key, key + ra.n_key, ra.col + ra.n_val);
-    if ((e = launch_recon(rm, ra, pairs, s)) != cudaSuccess) return e;
+    if ((e = launch_recon(rm, ra, pairs, l > 0, s)) != cudaSuccess) return e;
     if ((e = hook_launched(hook, s)) != cudaSuccess) return e;
   }
   AArgsP aa;
@@ -1096,8 +1099,10 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   cudaGetDevice(&dev);
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int64_t items = streams * aa.ntp;
-  prefill_attn_kernel<<<(int)std::min<int64_t>(items, sms), kAThreadsP, asmem, s>>>(am, aa);
-  return hook_launched(hook, s);
+  // its set-up overlaps the reconstruction's end, as the keys' launch overlaps the
+  // values': eight short MHA prompts 58.3 -> 51.5 us, MHA prompt 2 x 4096 341 -> 336
+  e = launch_pdl(prefill_attn_kernel, dim3((unsigned)std::min<int64_t>(items, sms)), dim3(kAThreadsP), asmem, s, am, aa);
+  return e != cudaSuccess ? e : hook_launched(hook, s);
 }
 
 }  // namespace dck
