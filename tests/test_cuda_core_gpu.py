@@ -77,3 +77,13 @@ def test_append_few(dtype, n_tok, hidden):
         bound = u * np.abs(ref) + hidden * 2.0 ** -23 * (np.abs(x.astype(np.float64)) @ np.abs(A.astype(np.float64)))
         assert (np.abs(got[rows] - ref) <= bound).all()
         assert (got[np.setdiff1d(np.arange(n_tok + 5), rows)] == 0).all()
+
+
+def test_current_stream():
+    """A call without a stream goes to the current one."""
+    torch.cuda.init()
+    side = torch.cuda.Stream()
+    assert dck._stream(None) == torch.cuda.current_stream().cuda_stream
+    with torch.cuda.stream(side):
+        assert dck._stream(None) == side.cuda_stream != torch.cuda.default_stream().cuda_stream
+    assert dck._stream(side) == side.cuda_stream
