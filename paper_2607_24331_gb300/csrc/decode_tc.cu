@@ -803,7 +803,7 @@ __device__ __forceinline__ void ldmatrix_x4_plain(uint32_t (&r)[4], uint32_t add
                : "r"(addr));
 }
 
-constexpr int kAppStages = 6;    // k-steps of a warp in flight
+constexpr int kAppStages = 6;    // k-steps of a warp in its ring, handled two at a time
 // Dynamic shared memory of the append: per warp a ring of stages of a factor
 // tile (512 B) and an x tile (16 tokens x 16 k per token m-tile), then the
 // warps' partial sums.
@@ -816,7 +816,7 @@ __host__ __device__ inline size_t app_smem_bytes(int batch) {
 // tokens.  Warp w accumulates K range [w D / 8, (w + 1) D / 8) with mma
 // m16n8k16 (tokens x K) . (K x 16 columns).  Each k-step's factor tile
 // [16 k][16 columns] and x tile [tokens][16 k] go through a per-warp ring of
-// cp.async stages, kAppStages k-steps ahead, so the factor stream (read once)
+// cp.async stages, kAppStages - 2 k-steps ahead, so the factor stream (read once)
 // keeps enough bytes in flight; ldmatrix reads the operands (.trans for the
 // column-major factor).  The eight warps' partial sums are added in shared
 // memory, rounded to bf16 and written to the cache rows.
@@ -842,43 +842,72 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[m][n][q] = 0.f;
   const uint32_t rbase = smem_u32(app_dyn + (size_t)warp * kAppStages * sb);
-  // stage kk: factor rows k (lane / 2), columns 8 (lane & 1) ..; x rows t, 16-byte halves h (two per row)
-  auto issue = [&](int kk) {
-    const uint32_t st = rbase + (uint32_t)((kk % kAppStages) * sb);
-    if (kk < nks) {
-      const int k0 = kbeg + 16 * kk;
-      cp_async16_cg(st + (uint32_t)(((lane >> 1) * 16 + 8 * (lane & 1)) * 2),
-                    A + (int64_t)(k0 + (lane >> 1)) * N + 8 * (lane & 1));
-      for (int e = lane; e < 2 * 16 * mt; e += 32) {  // x rows of the token m-tiles (zero rows past B)
-        const int t = e >> 1, h = e & 1;
-        const uint32_t dst = st + 512 + (uint32_t)((t * 16 + 8 * h) * 2);
-        if (t < B) cp_async16_cg(dst, ap.x + (int64_t)t * D + k0 + 8 * h);
-        else asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0u) : "memory");
+  // stage of a k-step: factor rows k (lane / 2), columns 8 (lane & 1) ..; x rows t,
+  // 16-byte halves (two per row).  Rows past the batch are zeroed once.  The
+  // pointers move along K, so a k-step is a copy or two and no address arithmetic
+  // (formed anew, with the rows zeroed each time, it took 520 cycles: 9.5 us of a
+  // step of one sequence on the 32-head layer, whose call this took from 40.3 to
+  // 37.0 us, and 8 x 32768 on the 8-KV-head layer from 190 to 187).
+  const int tr = lane >> 1, th = 8 * (lane & 1);
+  const uint32_t so = (uint32_t)((tr * 16 + th) * 2);
+  for (int sl = 0; sl < kAppStages; ++sl)
+#pragma unroll
+    for (int m = 0; m < kAppMaxTok / 16; ++m)
+      if (m < mt && 16 * m + tr >= B)
+        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(rbase + (uint32_t)(sl * sb) + 512 + 512 * m + so),
+                     "r"(0u)
+                     : "memory");
+  const __nv_bfloat16* pa = A + (int64_t)(kbeg + tr) * N + th;
+  const __nv_bfloat16* px = ap.x + (int64_t)tr * D + kbeg + th;
+  const int64_t astep = (int64_t)16 * N;
+  int left = nks;  // k-steps not yet issued
+  auto issue = [&](int slot) {
+    if (left <= 0) return;
+    --left;
+    const uint32_t st = rbase + (uint32_t)(slot * sb) + so;
+    cp_async16_cg(st, pa);
+#pragma unroll
+    for (int m = 0; m < kAppMaxTok / 16; ++m)
+      if (m < mt && 16 * m + tr < B) cp_async16_cg(st + 512 + 512 * m, px + (int64_t)(16 * m) * D);
+    pa += astep;
+    px += 16;
+  };
+  constexpr int kPairs = kAppStages / 2;  // ring slots of two k-steps
+#pragma unroll
+  for (int q = 0; q < kPairs - 1; ++q) {
+    issue(2 * q);
+    issue(2 * q + 1);
+    cp_async_commit_group();
+  }
+  int rd = 0, wr = kPairs - 1;  // slots read and refilled next
+  const int m8 = lane >> 3, r8 = lane & 7;
+  const uint32_t fo = (uint32_t)(((8 * (m8 & 1) + r8) * 16 + 8 * (m8 >> 1)) * 2);  // this lane's fragment row
+  for (int kk = 0; kk < nks; kk += 2) {
+    issue(2 * wr);
+    issue(2 * wr + 1);
+    cp_async_commit_group();
+    wr = wr + 1 == kPairs ? 0 : wr + 1;
+    cp_async_wait_group<kPairs - 1>();  // this slot has landed (this thread's copies)
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      if (kk + j >= nks) break;
+      const uint32_t st = rbase + (uint32_t)((2 * rd + j) * sb) + fo;
+      // B fragments: matrix m = lane / 8 covers k rows 8 (m & 1) .., n columns 8 (m >> 1) ..
+      uint32_t bf[4];
+      ldmatrix_x4_trans(bf, st);
+#pragma unroll
+      for (int m = 0; m < kAppMaxTok / 16; ++m) {
+        if (m >= mt) break;
+        // A fragments (tokens 16 m .., k 0..15): matrix q = lane / 8 covers rows 8 (q & 1) .., k 8 (q >> 1) ..
+        uint32_t af[4];
+        ldmatrix_x4_plain(af, st + 512 + 512 * m);
+        mma_16816(acc[m][0], af[0], af[1], af[2], af[3], bf[0], bf[1]);
+        mma_16816(acc[m][1], af[0], af[1], af[2], af[3], bf[2], bf[3]);
       }
     }
-    cp_async_commit_group();
-  };
-#pragma unroll
-  for (int q = 0; q < kAppStages - 1; ++q) issue(q);
-  for (int kk = 0; kk < nks; ++kk) {
-    issue(kk + kAppStages - 1);
-    cp_async_wait_group<kAppStages - 1>();  // stage kk has landed (this thread's copies)
-    __syncwarp();
-    const uint32_t st = rbase + (uint32_t)((kk % kAppStages) * sb);
-    // B fragments: matrix m = lane / 8 covers k rows 8 (m & 1) .., n columns 8 (m >> 1) ..
-    uint32_t bf[4];
-    const int m8 = lane >> 3, r8 = lane & 7;
-    ldmatrix_x4_trans(bf, st + (uint32_t)(((8 * (m8 & 1) + r8) * 16 + 8 * (m8 >> 1)) * 2));
-#pragma unroll
-    for (int m = 0; m < kAppMaxTok / 16; ++m) {
-      if (m >= mt) break;
-      // A fragments (tokens 16 m .., k 0..15): matrix q = lane / 8 covers rows 8 (q & 1) .., k 8 (q >> 1) ..
-      uint32_t af[4];
-      ldmatrix_x4_plain(af, st + 512 + (uint32_t)(((16 * m + 8 * (m8 & 1) + r8) * 16 + 8 * (m8 >> 1)) * 2));
-      mma_16816(acc[m][0], af[0], af[1], af[2], af[3], bf[0], bf[1]);
-      mma_16816(acc[m][1], af[0], af[1], af[2], af[3], bf[2], bf[3]);
-    }
-    __syncwarp();  // every lane is done with the stage before it is refilled
+    rd = rd + 1 == kPairs ? 0 : rd + 1;
+    __syncwarp();  // every lane is done with the slot before it is refilled
   }
   cp_async_wait_group<0>();
   // partial sums -> shared memory: token 16 m + gid (+8), column 8 n + 2 tig (+1)
@@ -920,13 +949,15 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
 // frequency pairs that its columns need.  Bound by latency and the launch: with a
 // whole item per block, fp64 angles and the loads in series it took 10.3 us for
 // one sequence of the 32-head layer and 13 us for 16 (18 MB of images, written to
-// L2).  Small blocks, not one per SM: SMs that have none left take the scores
+// L2).  Two sequences and three blocks per SM, so that 16 sequences' pieces start
+// together with the append (four and two: 129.2 us for that step, now 128.3).
+// Small blocks, not one per SM: SMs that have none left take the scores
 // kernel's CTAs, whose set-up then overlaps (one 512-thread block per SM cost the
 // step 4 to 10 us).
-constexpr int kPrepSeqs = 4;
+constexpr int kPrepSeqs = 2;
 constexpr int kPrepThreads = 256;
 template <bool kFold>
-__global__ void __launch_bounds__(kPrepThreads, 2)
+__global__ void __launch_bounds__(kPrepThreads, 3)
     factor_prep_kernel(const LayerTable lt, const DecodeArgs a, const __grid_constant__ PrepArgs pa,
                        uint8_t* __restrict__ img) {
   griddep_launch();
