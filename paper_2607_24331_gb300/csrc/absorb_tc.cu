@@ -20,12 +20,14 @@
 // lane per r_v row of a chunk.
 //
 // Warps: 0 producer (P images by bulk copy, value chunks by TMA), 1 and 6 MMA
-// issuers (lane 0 of each; M = 128 r_v rows, N = Hq_pad, K = 16 tokens; 8 per
-// chunk and tile), each taking half
-// of a tile's r_v chunks from its own ring of value slots (a single thread's
-// MMA issue, commits and barrier tests took longer than the values took to
-// arrive); warp 1 owns TMEM.  2-5 epilogue (one TMEM lane quadrant each:
-// rescales and the U readout).
+// issuers (M = 128 r_v rows, N = Hq_pad, K = 16 tokens; 8 per chunk and tile), each
+// taking half of a tile's r_v chunks from its own ring of value slots (a single
+// warp's issue, commits and barrier tests took longer than the values took to
+// arrive); warp 1 owns TMEM.  2-5 epilogue (one TMEM lane quadrant each: rescales
+// and the U readout).  Where a sequence ends inside a tile, the issuing warp clears
+// the chunk's rows past it: by one lane, as the issuing once was, that was up to
+// 2032 stores a chunk (steps of the 32-head layer, one lane / the warp: 32 ragged
+// sequences 271 / 250 us, 8 x 777 tokens 54 / 46, 1 x 777 37 / 33).
 // Every wait is bounded; on expiry the CTA records kErrTimeout and releases
 // TMEM after the work in flight has landed.
 #include <algorithm>
@@ -320,36 +322,41 @@ __global__ void __launch_bounds__(kAThreads, 1)
       }
     }
   } else if (warp == 1 || warp == 6) {
-    // ---- MMA issuers: lane 0 of warp 1 takes chunks [ca, cm) of every tile,
-    // lane 0 of warp 6 chunks [cm, cb), each from its own value ring; both wait
-    // for every P slot and every hand-off with the epilogue, and both release --
-    if (lane == 0 && has_work) {
+    // ---- MMA issuers: warp 1 takes chunks [ca, cm) of every tile, warp 6 chunks
+    // [cm, cb), each from its own value ring; both wait for every P slot and every
+    // hand-off with the epilogue, and both release.  The whole warp runs the schedule
+    // and an elected lane issues, with descriptors as a base plus a slot and a
+    // constant per k-step ------------------------------------------------------
+    if (has_work) {
+      const bool el = elect_one();
       const int t = warp == 1 ? 0 : 1;
       const uint32_t idesc_v = idesc_bf16(128, hq_pad, true, false);
+      const uint64_t dv = sdesc(smem_u32(sm.v[0]), kVSlot / 2, 1024, kSw128);
+      const uint64_t dp = sdesc(smem_u32(sm.p[0]), 16, 1024, kSw128);
+      const uint64_t patom = (uint64_t)(hq_pad * 128 >> 4);  // 64 tokens of P
       int vs = 0, vph = 0, p_cnt = 0, rc = 0, sgc = 0;
       bool ok = true;
       for (AWalk walk = walk0; ok && walk.next(a, pl, seg);) {
+        const uint32_t ubuf = tmem + (sgc % nub) * ucols;
         for (int i = 0; i < seg.n && ok; ++i) {
           const int psl = p_cnt % kNP;
-          if (!(ok = mbar_wait(&sm.p_full[psl], (p_cnt / kNP) & 1, abort_flag))) break;
+          if (!(ok = wwait(&sm.p_full[psl], (p_cnt / kNP) & 1, abort_flag))) break;
           if (i > 0) {
             // some head's reference max rises at this tile: the epilogue rescales U
             // once the earlier tiles' MMAs are done (drain) and releases this tile
             // (tile_ok)
             if (sm.pneed[psl]) {
-              umma_commit(&sm.drain);
-              if (!(ok = mbar_wait(&sm.tile_ok, rc & 1, abort_flag))) break;
+              if (el) umma_commit(&sm.drain);
+              if (!(ok = wwait(&sm.tile_ok, rc & 1, abort_flag))) break;
               tc_fence_after();
-              DCK_AB_TRACE(10);
               ++rc;
             }
           } else if (sgc >= nub) {  // the epilogue has read out this buffer's previous segment
-            if (!(ok = mbar_wait(&sm.u_free[sgc % nub], (sgc / nub - 1) & 1, abort_flag))) break;
+            if (!(ok = wwait(&sm.u_free[sgc % nub], (sgc / nub - 1) & 1, abort_flag))) break;
             tc_fence_after();
           }
-          DCK_AB_TRACE(11);
           const int nvalid = seg.nvalid(i);
-          const uint32_t pbase = smem_u32(sm.p[psl]);
+          const uint64_t pd = dp + (uint64_t)(psl * (kPSlot >> 4));
           // chunks in pairs: the K = 16 MMAs of one chunk form a dependent chain on
           // its accumulator (about 120 cycles each at N = Hq_pad), so two chunks'
           // chains are interleaved
@@ -358,44 +365,54 @@ __global__ void __launch_bounds__(kAThreads, 1)
           const int c0 = t ? cm : ca, c1 = t ? cb : cm;
           for (int c = c0; c < c1 && ok; c += 2) {
             const int nc = min(2, c1 - c);
-            uint32_t vb[2] = {0u, 0u};
             int sl[2] = {0, 0};
-            for (int q = 0; q < nc && ok; ++q) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              if (q == nc) break;
               sl[q] = t * kNVr + vs;
-              if (!(ok = mbar_wait(&sm.v_full[sl[q]], vph, abort_flag))) break;
+              if (!(ok = wwait(&sm.v_full[sl[q]], vph, abort_flag))) break;
               if (++vs == kNVr) {
                 vs = 0;
                 vph ^= 1;
               }
               if (nvalid < kTile) {  // rows past the sequence end: exact zeros
-                for (int r = nvalid; r < kTile; ++r)
-#pragma unroll
-                  for (int w = 0; w < 8; ++w) {
-                    reinterpret_cast<uint4*>(sm.v[sl[q]] + r * 128)[w] = make_uint4(0, 0, 0, 0);
-                    reinterpret_cast<uint4*>(sm.v[sl[q]] + kVSlot / 2 + r * 128)[w] = make_uint4(0, 0, 0, 0);
-                  }
+                uint8_t* v = sm.v[sl[q]];
+                for (int e = lane; e < (kTile - nvalid) * 16; e += 32)
+                  *reinterpret_cast<uint4*>(v + ((e >> 3) & 1) * (kVSlot / 2) + (nvalid + (e >> 4)) * 128 +
+                                            (e & 7) * 16) = make_uint4(0, 0, 0, 0);
                 fence_proxy_async_smem();
+                __syncwarp();
               }
-              vb[q] = smem_u32(sm.v[sl[q]]);
             }
             if (!ok) break;
+            tc_fence_after();
+            if (el) {
+              const uint64_t v0 = dv + (uint64_t)(sl[0] * (kVSlot >> 4)), v1 = dv + (uint64_t)(sl[1] * (kVSlot >> 4));
+              const uint32_t u0 = ubuf + c * hq_pad, u1 = u0 + hq_pad;
+              if (nc == 2) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const uint64_t bd = sdesc(pbase + (k >> 2) * (hq_pad * 128) + (k & 3) * 32, 16, 1024, kSw128);
-              for (int q = 0; q < nc; ++q)
-                umma_f16(tmem + (sgc % nub) * ucols + (c + q) * hq_pad, sdesc(vb[q] + k * 2048, kVSlot / 2, 1024, kSw128), bd, idesc_v,
-                         (i == 0 && k == 0) ? 0u : 1u);
+                for (int k = 0; k < 8; ++k) {
+                  const uint64_t bd = pd + (k >> 2) * patom + 2 * (k & 3);
+                  const uint32_t acc = i == 0 && k == 0 ? 0u : 1u;
+                  umma_f16(u0, v0 + 128 * k, bd, idesc_v, acc);
+                  umma_f16(u1, v1 + 128 * k, bd, idesc_v, acc);
+                }
+                umma_commit(&sm.v_empty[sl[0]]);
+                umma_commit(&sm.v_empty[sl[1]]);
+              } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                  umma_f16(u0, v0 + 128 * k, pd + (k >> 2) * patom + 2 * (k & 3), idesc_v, i == 0 && k == 0 ? 0u : 1u);
+                umma_commit(&sm.v_empty[sl[0]]);
+              }
             }
-            for (int q = 0; q < nc; ++q) umma_commit(&sm.v_empty[sl[q]]);
-            DCK_AB_TRACE(12);
           }
           if (!ok) break;
-          umma_commit(&sm.p_empty[psl]);
+          if (el) umma_commit(&sm.p_empty[psl]);
           ++p_cnt;
         }
         if (!ok) break;
-        umma_commit(&sm.u_ready[sgc % nub]);
-        DCK_AB_TRACE(13);
+        if (el) umma_commit(&sm.u_ready[sgc % nub]);
         ++sgc;
       }
     }
