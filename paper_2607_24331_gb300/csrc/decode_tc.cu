@@ -805,11 +805,12 @@ __device__ __forceinline__ void ldmatrix_x4_plain(uint32_t (&r)[4], uint32_t add
 
 constexpr int kAppStages = 6;    // k-steps of a warp in its ring, handled two at a time
 // Dynamic shared memory of the append: per warp a ring of stages of a factor
-// tile (512 B) and an x tile (16 tokens x 16 k per token m-tile), then the
-// warps' partial sums.
+// tile (512 B) and an x tile (16 tokens x 16 k per token m-tile); the warps'
+// partial sums follow in the same place.  Every block of the launch carries it, and
+// the factor pieces want three blocks per SM.
 __host__ __device__ inline int app_stage_bytes(int batch) { return 512 + ((batch + 15) / 16) * 512; }
-__host__ __device__ inline size_t app_smem_bytes(int batch) {
-  return (size_t)kAppWarps * kAppStages * app_stage_bytes(batch) + (size_t)kAppWarps * batch * kAppCols * 4;
+inline size_t app_smem_bytes(int batch) {
+  return std::max((size_t)kAppWarps * kAppStages * app_stage_bytes(batch), (size_t)kAppWarps * batch * kAppCols * 4);
 }
 
 // One GEMV block: output columns [c0, c0 + 16) of [A_k | A_v] for B <= 64
@@ -824,7 +825,7 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
                                                   int blk) {
   extern __shared__ __align__(128) uint8_t app_dyn[];
   const int sb = app_stage_bytes(a.B);
-  float* red = reinterpret_cast<float*>(app_dyn + (size_t)kAppWarps * kAppStages * sb);  // [warp][B * 16]
+  float* red = reinterpret_cast<float*>(app_dyn);  // [warp][B * 16], after the ring's last use
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gid = lane >> 2, tig = lane & 3;
   const int c0 = blk * kAppCols;
@@ -910,6 +911,7 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
     __syncwarp();  // every lane is done with the slot before it is refilled
   }
   cp_async_wait_group<0>();
+  __syncthreads();  // every warp is done with its ring
   // partial sums -> shared memory: token 16 m + gid (+8), column 8 n + 2 tig (+1)
 #pragma unroll
   for (int m = 0; m < kAppMaxTok / 16; ++m)
