@@ -66,8 +66,9 @@
 // score MMA's operand layout, which the 16x256b TMEM load gives directly.  The
 // rings hand out single pieces and items: with whole units, a second unit of
 // three items did not fit and its load came after the first one's MMAs.
-// Whole calls, before / now: 32-head MHA 16 x 4096 169.5 / 147.6 us, 32 ragged
-// 367 / 321; GQA 8 x 32768 251 / 228, 2 x 131072 286 / 222.
+// Whole calls before / with these: 32-head MHA 16 x 4096 169.5 / 147.6 us, 32 ragged
+// 367 / 321; GQA 8 x 32768 251 / 228, 2 x 131072 286 / 222 (with the changes of the
+// other kernels and shared-space addressing since: 129, 251, 191, 189).
 // Every wait is bounded (about 2 s); on expiry the CTA stops issuing work,
 // tells its peer to stop, records kErrTimeout, waits for work in flight and
 // still releases TMEM.

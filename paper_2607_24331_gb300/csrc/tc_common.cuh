@@ -34,11 +34,6 @@ __device__ __forceinline__ void bulk_store_wait_read() { asm volatile("cp.async.
 // ... and their writes are complete.
 __device__ __forceinline__ void bulk_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// Moves [src, src + bytes) toward L2 ahead of its TMA loads (16-byte multiples).
-__device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
 // Bounded wait whose outcome is the same in every lane of the warp.
 __device__ __forceinline__ bool wwait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   const bool r = mbar_wait(bar, parity, abort_flag);
