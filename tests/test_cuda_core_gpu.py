@@ -59,11 +59,12 @@ def test_step_fp32(lens):
     _step(S.workload(0).layer, lens, seed=6)
 
 
-@pytest.mark.parametrize("hidden", [1, 127, 130, 512, 1100])
-@pytest.mark.parametrize("n_tok", [1, 8, 9, 512, 513])
+@pytest.mark.parametrize("hidden", [1, 8, 127, 128, 130, 200, 512, 1100])
+@pytest.mark.parametrize("n_tok", [1, 8, 9, 129, 256, 512, 513])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_append_few(dtype, n_tok, hidden):
-    # (a bf16 layer whose rank sums the tensor-core append does not take goes the same way)
+    # (bf16 layers whose hidden width is a multiple of 8 take the tensor-core cluster: here with output widths
+    # below its 64 columns and with fewer 64-wide K blocks than CTAs; the other bf16 layers go the fp32 way)
     spec = _layer(2, ((1,), (0,)), (16, 32), 16, 64, dtype, hidden)
     x, A_k, A_v = S.make_append_inputs(spec, n_tok, seed=hidden)
     rows = np.random.default_rng(n_tok).choice(n_tok + 5, size=n_tok, replace=False)
