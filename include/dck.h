@@ -299,6 +299,20 @@ int32_t dck_last_launch_count(void);
 dck_status dck_selftest_bounded_wait(int64_t limit_cycles, void* stream);
 
 /*
+ * Self-test of an append whose operands do not arrive: dck_latent_append's
+ * tensor-core kernel for these arguments, with the load of its last block of x
+ * and factors left out, so that its wait for them gives up after
+ * `limit_cycles` SM clock cycles (1000 .. 4e9).  The kernel stops, writes no
+ * row of an output tile that is not whole (here: none at all) and records the
+ * timeout; the context stays usable.  DCK_ERR_UNSUPPORTED where the append
+ * takes another kernel: fp32, or more than 256 tokens with R_k and r_v
+ * multiples of 64.
+ */
+dck_status dck_selftest_append_timeout(const dck_layer_desc* desc, const void* x, int32_t n_tok, const void* A_k,
+                                       const void* A_v, const int64_t* d_rows, void* kcache, void* vcache,
+                                       int64_t n_rows, int64_t limit_cycles, void* stream);
+
+/*
  * Seeded synthetic input (not part of the method): fills n elements of `dst`
  * with the counter-based Gaussian stream `key` starting at element `start`:
  * SplitMix64 draws 2i and 2i+1, the sum of their eight 16-bit fields s,

@@ -40,6 +40,7 @@ struct AppendParams {
   __nv_bfloat16* vc;
   int64_t n_rows;
   int* err;
+  long long limit;  // kWithhold kernels: SM cycles after which the waits for operands give up
 };
 
 __device__ __forceinline__ void tile_of(const AppendParams& p, int t, bool& is_k, int& n0, int& nt) {
@@ -49,6 +50,8 @@ __device__ __forceinline__ void tile_of(const AppendParams& p, int t, bool& is_k
   nt = min(kMaxBN, N - n0);
 }
 
+// kWithhold: the self-test of the waits, whose last K block is never loaded.
+template <bool kWithhold>
 __global__ void __launch_bounds__(kThreads, 1)
     append_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_ak,
                      const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
@@ -95,7 +98,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tm_x);
     tma_prefetch_desc(tmb);
-    for (int kb = kb0; kb < kb1; ++kb) {
+    for (int kb = kb0; kb < kb1 - (kWithhold ? 1 : 0); ++kb) {
       const int i = kb - kb0, s = i % nst;
       if (i >= nst && !mbar_wait(&empty[s], ((i / nst) - 1) & 1, abort_flag)) break;
       uint8_t* a = smem + s * kStageBytes;
@@ -106,9 +109,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1 && lane == 0) {
     const uint32_t idesc = idesc_bf16(kBM, nt, false, true);
+    bool ok = true;
     for (int kb = kb0; kb < kb1; ++kb) {
       const int i = kb - kb0, s = i % nst;
-      if (!mbar_wait(&full[s], (i / nst) & 1, abort_flag)) break;
+      if (!(ok = mbar_wait(&full[s], (i / nst) & 1, abort_flag, kWithhold ? p.limit : kWaitCycles))) break;
       tc_fence_after();
       const uint32_t a = smem_u32(smem + s * kStageBytes);
       const uint32_t b = a + kABytes;
@@ -120,11 +124,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       umma_commit(&empty[s]);
     }
-    umma_commit(acc_bar);
+    if (ok) umma_commit(acc_bar);  // (a sum that is not whole is never announced)
   } else if (warp >= 2) {
     const int quad = warp & 3;
     const int m = m0 + quad * 32 + lane;
-    const bool ok = mbar_wait(acc_bar, 0, abort_flag);
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_bar, 0, abort_flag));
     tc_fence_after();
     int64_t row = -1;
     if (ok && m < p.n_tok) {
@@ -153,11 +157,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if (*abort_flag) {
+    drain_in_flight();
+    if (threadIdx.x == 0) atomicOr(p.err, kErrTimeout);
+  }
+  __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 256);
   }
-  if (threadIdx.x == 0 && *abort_flag) atomicOr(p.err, kErrTimeout);
 }
 
 // ---------------------------------------------------------------------------
@@ -184,6 +192,7 @@ static_assert(kFN == 16 * kFSplit, "a rank owns one 16-column slice");
 // pushes of a warp (one row per lane) spread over the banks.
 __device__ __forceinline__ int few_chunk(int r, int q) { return (r * 4 + (q ^ ((r >> 1) & 3))) * 16; }
 
+template <bool kWithhold>
 __global__ void __launch_bounds__(kThreads, 1)
     append_few_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_ak,
                       const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
@@ -224,12 +233,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_launch_dependents();
   const uint32_t tmem = *tmem_slot;
   const CUtensorMap* tmb = is_k ? &tm_ak : &tm_av;
+  // a wait that gave up stops the whole cluster: no rank adds sums that are not whole
+  auto stop_cluster = [&]() {
+    for (uint32_t c = 0; c < kFSplit; ++c) st_cluster_u32(mapa_shared(smem_u32((const void*)abort_flag), c), 1u);
+  };
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int kb = kb0; kb < kb1; ++kb) {
+      const int kbe = kb1 - (kWithhold && rank == kFSplit - 1 ? 1 : 0);
+      for (int kb = kb0; kb < kbe; ++kb) {
         const int i = kb - kb0, s = i % kFStages;
-        if (i >= kFStages && !mbar_wait(&empty[s], ((i / kFStages) - 1) & 1, abort_flag)) break;
+        if (i >= kFStages && !mbar_wait(&empty[s], ((i / kFStages) - 1) & 1, abort_flag)) {
+          stop_cluster();
+          break;
+        }
         uint8_t* a = smem + s * kFStageBytes;
         mbar_expect_tx(&full[s], kFStageBytes);
         tma_load_2d(a + kABytes, tmb, &full[s], n0, kb * kBK);
@@ -243,7 +260,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (int i = 0; i < kb1 - kb0; ++i) {
       const int s = i % kFStages;
-      ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (i / kFStages) & 1, abort_flag));
+      ok = __all_sync(0xffffffffu, mbar_wait(&full[s], (i / kFStages) & 1, abort_flag,
+                                             kWithhold ? p.limit : kWaitCycles));
       if (!ok) break;
       tc_fence_after();
       const uint64_t o = (uint64_t)(s * (kFStageBytes >> 4));
@@ -254,7 +272,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         umma_commit(&empty[s]);
       }
     }
-    if (el) umma_commit(acc_bar);
+    if (ok && el) umma_commit(acc_bar);
+    if (!ok && lane == 0) stop_cluster();
   } else {
     const int quad = warp & 3, r = quad * 32 + lane;
     const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_bar, 0, abort_flag));
@@ -279,15 +298,23 @@ __global__ void __launch_bounds__(kThreads, 1)
                          : "memory");
         }
       }
+    } else if (lane == 0) {
+      stop_cluster();
     }
   }
   tc_fence_before();
   __syncwarp();
-  cluster_sync();  // every partial sum of this rank's slice has arrived
+  cluster_sync();  // every partial sum of this rank's slice has arrived, or the flag is set in every rank
+  const bool stopped = *abort_flag != 0;
+  if (stopped) {
+    drain_in_flight();
+    if (threadIdx.x == 0) atomicOr(p.err, kErrTimeout);
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kFN);
   }
+  if (stopped) return;
   const int col = n0 + 16 * rank;
   __nv_bfloat16* dst = is_k ? p.kc : p.vc;
   for (int i = threadIdx.x; i < kBM * 4; i += kThreads) {
@@ -310,7 +337,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     *reinterpret_cast<__nv_bfloat162*>(&o.y) = __floats2bfloat162_rn(v.z, v.w);
     *reinterpret_cast<uint2*>(dst + row * N + col + 4 * q) = o;
   }
-  if (threadIdx.x == 0 && *abort_flag) atomicOr(p.err, kErrTimeout);
 }
 
 // ---------------------------------------------------------------------------
@@ -599,10 +625,12 @@ size_t tc_append_workspace(int n_tok, int Rk, int rv) {
   return n_tok <= kSplitMaxTok ? align_up((size_t)kMaxSplit * n_tok * (Rk + rv) * sizeof(float), 256) : 0;
 }
 
+// withhold_limit > 0: the self-test of the waits (see kWithhold), with that limit.
 cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
                              const int64_t* rows, void* kc, void* vc, int64_t n_rows, int* err, cudaStream_t s,
-                             int* n_launches) {
+                             int* n_launches, long long withhold_limit) {
   *n_launches = 1;
+  const bool withhold = withhold_limit > 0;
   AppendParams p;
   p.n_tok = n_tok;
   p.D = D;
@@ -615,6 +643,7 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
   p.vc = static_cast<__nv_bfloat16*>(vc);
   p.n_rows = n_rows;
   p.err = err;
+  p.limit = withhold_limit;
   CUtensorMap tx, tk, tv;
   if (!make_tmap_2d_bf16(&tx, x, D, n_tok, (uint64_t)D * 2, kBK, kBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_tmap_2d_bf16(&tk, A_k, Rk, D, (uint64_t)Rk * 2, 64, kBK, CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -626,6 +655,7 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
     cudaError_t e = cudaFuncSetAttribute(append_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem);
     if (e != cudaSuccess) return e;
     const int pairs = append_pairs_of_device(psmem);
+    if (withhold) return cudaErrorNotSupported;
     if (pairs > 0) {
       const int64_t n_mt = (n_tok + kPRows - 1) / kPRows;
       const int64_t tiles = n_mt * (pt_count(Rk) + pt_count(rv));
@@ -650,7 +680,8 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
   if (n_tok <= kSplitMaxTok) {
     p.nt_k = (Rk + kFN - 1) / kFN;
     const size_t fsmem = (size_t)kFStages * kFStageBytes + kFRecvBytes + 1024 + 256;
-    cudaError_t e = cudaFuncSetAttribute(append_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
+    auto k = withhold ? append_few_kernel<true> : append_few_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(kFSplit * (p.nt_k + (rv + kFN - 1) / kFN), (n_tok + kBM - 1) / kBM);
@@ -666,13 +697,14 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, append_few_kernel, tx, tk, tv, p);
+    return cudaLaunchKernelEx(&cfg, k, tx, tk, tv, p);
   }
   const int ntiles = p.nt_k + (rv + kMaxBN - 1) / kMaxBN;
   const size_t smem = (size_t)kStages * kStageBytes + 1024 + 256;
-  cudaError_t e = cudaFuncSetAttribute(append_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto k = withhold ? append_tc_kernel<true> : append_tc_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(append_tc_kernel, dim3(ntiles, (n_tok + kBM - 1) / kBM), dim3(kThreads), smem, s, tx, tk, tv, p);
+  return launch_pdl(k, dim3(ntiles, (n_tok + kBM - 1) / kBM), dim3(kThreads), smem, s, tx, tk, tv, p);
 }
 
 }  // namespace dck

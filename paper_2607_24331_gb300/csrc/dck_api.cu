@@ -29,7 +29,7 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
 cudaError_t launch_bounded_wait_selftest(long long limit_cycles, int* err, cudaStream_t s);
 cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
                              const int64_t* rows, void* kc, void* vc, int64_t n_rows, int* err, cudaStream_t s,
-                             int* n_launches);
+                             int* n_launches, long long withhold_limit);
 }  // namespace dck
 
 using namespace dck;
@@ -408,7 +408,7 @@ dck_status dck_latent_append(const dck_layer_desc* desc, const void* x, int32_t 
     const size_t need = tc_append_workspace(n_tok, lt.Rk, lt.rv);
     if (need && (!workspace || ws_bytes < need || !aligned(workspace, 256))) return DCK_ERR_WORKSPACE;
     e = launch_append_tc(x, n_tok, desc->hidden, A_k, A_v, lt.Rk, lt.rv, d_rows, kcache, vcache, n_rows, err, s,
-                         &launches);
+                         &launches, 0);
   } else {
     e = launch_append_simt(x, n_tok, desc->hidden, A_k, A_v, lt.Rk, lt.rv, d_rows, kcache, vcache, n_rows,
                            desc->dtype, err, s);
@@ -438,6 +438,26 @@ dck_status dck_selftest_bounded_wait(int64_t limit_cycles, void* stream) {
   return launch_bounded_wait_selftest((long long)limit_cycles, err, static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? DCK_OK
              : DCK_ERR_CUDA;
+}
+
+dck_status dck_selftest_append_timeout(const dck_layer_desc* desc, const void* x, int32_t n_tok, const void* A_k,
+                                       const void* A_v, const int64_t* d_rows, void* kcache, void* vcache,
+                                       int64_t n_rows, int64_t limit_cycles, void* stream) {
+  dck_status st = check_desc(desc);
+  if (st != DCK_OK) return st;
+  if (n_tok < 1 || n_rows < 0 || limit_cycles < 1000 || limit_cycles > 4000000000LL) return DCK_ERR_INVALID;
+  if (!x || !A_k || !A_v || !d_rows || !kcache || !vcache) return DCK_ERR_INVALID;
+  if (!aligned(x, 16) || !aligned(A_k, 16) || !aligned(A_v, 16) || !aligned(kcache, 16) || !aligned(vcache, 16))
+    return DCK_ERR_INVALID;
+  const LayerTable lt = make_table(desc);
+  if (!tc_append_supports(desc->hidden, lt.Rk, lt.rv, desc->dtype)) return DCK_ERR_UNSUPPORTED;
+  int* err = nullptr;
+  if (!device_state(&err, nullptr)) return DCK_ERR_CUDA;
+  int launches = 0;
+  const cudaError_t e = launch_append_tc(x, n_tok, desc->hidden, A_k, A_v, lt.Rk, lt.rv, d_rows, kcache, vcache,
+                                         n_rows, err, static_cast<cudaStream_t>(stream), &launches, limit_cycles);
+  if (e == cudaErrorNotSupported) return DCK_ERR_UNSUPPORTED;
+  return e == cudaSuccess ? DCK_OK : DCK_ERR_CUDA;
 }
 
 dck_status dck_synth_gaussian(void* dst, int64_t n, uint64_t key, int64_t start, float scale, int32_t dtype,

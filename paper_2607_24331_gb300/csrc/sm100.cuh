@@ -56,13 +56,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+constexpr long long kWaitCycles = 4000000000ll;  // limit of a wait, about 2 s at the GB300's clocks
+
 // Wait for phase `parity` of `bar` to complete, for at most `limit_cycles` SM
-// clock cycles (about 2 s at the GB300's clocks).  On expiry sets *abort
+// clock cycles.  On expiry sets *abort
 // (shared, visible to the CTA) and returns false; a CTA that sees *abort set
 // stops issuing work.  The budget is kept with the SM-local clock: reading the
 // global timer costs a long round trip, which would sit on every hand-off.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                          long long limit_cycles = 4000000000ll) {
+                                          long long limit_cycles = kWaitCycles) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long c0 = clock64();
   while (true) {
@@ -73,6 +75,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
       *abort = 1;
       return false;
     }
+  }
+}
+
+// After a wait that gave up: about 2 ms, in which copies and MMAs already in
+// flight land, before shared and tensor memory are released.
+__device__ __forceinline__ void drain_in_flight() {
+  const long long c0 = clock64();
+  while (clock64() - c0 < 4000000ll) {
   }
 }
 

@@ -28,7 +28,7 @@ EXPORTED = (
     "dck_status_string", "dck_validate_desc", "dck_latent_append_workspace_size", "dck_latent_append",
     "dck_decode_workspace_size", "dck_decode_attention", "dck_last_device_error", "dck_set_decode_kernel",
     "dck_last_launch_count", "dck_synth_gaussian", "dck_set_timing_events", "dck_decode_attention_noalloc",
-    "dck_selftest_bounded_wait", "dck_decode_step", "dck_decode_step_workspace_size",
+    "dck_selftest_bounded_wait", "dck_selftest_append_timeout", "dck_decode_step", "dck_decode_step_workspace_size",
     "dck_prefill_workspace_size", "dck_prefill_attention",
 )
 
@@ -100,6 +100,8 @@ def lib() -> ctypes.CDLL:
     L.dck_set_timing_events.argtypes = [P, I32]
     L.dck_selftest_bounded_wait.restype = I32
     L.dck_selftest_bounded_wait.argtypes = [I64, P]
+    L.dck_selftest_append_timeout.restype = I32
+    L.dck_selftest_append_timeout.argtypes = [D, P, I32, P, P, P, P, P, I64, I64, P]
     L.dck_synth_gaussian.restype = I32
     L.dck_synth_gaussian.argtypes = [P, I64, U64, I64, F32, I32, P]
     _lib = L
@@ -248,6 +250,15 @@ def dck_selftest_bounded_wait(limit_cycles: int, stream=None) -> int:
     """One kernel whose bounded wait on a barrier nothing arrives at gives up after
     ``limit_cycles`` SM cycles; the timeout shows in the next dck_last_device_error."""
     return lib().dck_selftest_bounded_wait(int(limit_cycles), _stream(stream))
+
+
+def dck_selftest_append_timeout(layer: Layer, x, n_tok: int, A_k, A_v, rows, kcache, vcache, n_rows: int,
+                                limit_cycles: int, stream=None) -> int:
+    """A tensor-core append whose last operand block is never loaded: its wait gives up
+    after ``limit_cycles`` SM cycles, no row is written, the timeout is reported."""
+    return lib().dck_selftest_append_timeout(layer.ref, _ptr(x), int(n_tok), _ptr(A_k), _ptr(A_v), _ptr(rows),
+                                             _ptr(kcache), _ptr(vcache), int(n_rows), int(limit_cycles),
+                                             _stream(stream))
 
 
 def check(status: int, what: str) -> None:

@@ -74,6 +74,12 @@ def test_selftest_rejects_limits_out_of_range_without_launching():
     # checked on the host before any CUDA call (stream handle 0 is never used)
     assert dck.dck_selftest_bounded_wait(10, 0) == dck.DCK_ERR_INVALID
     assert dck.dck_selftest_bounded_wait(5_000_000_000, 0) == dck.DCK_ERR_INVALID
+    p, L = 1 << 20, dck.Layer.from_spec(S.workload(1).layer)  # aligned, never dereferenced
+
+    def append(L=L, x=p, n_tok=4, limit=2000):
+        return dck.dck_selftest_append_timeout(L, x, n_tok, p, p, p, p, p, 100, limit, 0)
+    assert append(limit=10) == append(n_tok=0) == append(x=None) == append(x=p + 2) == dck.DCK_ERR_INVALID
+    assert append(L=dck.Layer.from_spec(S.workload(0).layer)) == dck.DCK_ERR_UNSUPPORTED
 
 
 def test_decode_entry_points_check_arguments_before_any_cuda_call():
