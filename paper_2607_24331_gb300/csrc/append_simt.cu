@@ -134,16 +134,25 @@ __global__ void __launch_bounds__(256) append_few_kernel(const T* __restrict__ x
   (is_k ? kc : vc)[row * N + col + c] = from_f32<T>(v);
 }
 
-// The tile kernel's time is set by its D / 16 steps in series; the other's grows with
-// every eight tokens, for which the factors are read again from L2.  fp32 layer,
-// D = 512, tile kernel / this one: 16 tokens 103 / 16 us, 64 130 / 19, 256 119 / 41,
-// 512 115 / 72, 1024 119 / 129.
+// Whether a call is one of few tokens.  The tile kernel's time is set by its D / 16
+// steps in series (about 8 + 0.22 D us while its tiles fit the SMs); this one's by its
+// multiply-adds, for every eight tokens of which the factors are read again from L2, and
+// by its blocks (about 9 + 0.49 n_tok (R_k + r_v) (D + 225) / 10^6 us): equal where
+// n_tok (R_k + r_v) (D + 225) = 4.5 10^5 D.  fp32, us, tile kernel / this one, by
+// n_tok (R_k + r_v) in thousands, ! where the rule takes the tile kernel:
+//   D = 64:   66 19 / 19    78 21 / 21    131 21 / 27!   262 22 / 46!   2097 27 / 314!
+//   D = 512:  66 105 / 33   156 113 / 70  262 124 / 103  393 122 / 148! 2097 138 / 758!
+//   D = 2048: 66 398 / 99   156 461 / 232 262 476 / 324  393 474 / 482! 2097 523 / 2443!
+// (Not beyond 512 tokens, where neither was measured on narrow layers.)
 constexpr int kFewTokens = 512;
+inline bool few_tokens(int n_tok, int D, int width) {
+  return n_tok <= kFewTokens && (int64_t)n_tok * width * (D + 256) <= (int64_t)400000 * D;
+}
 
 template <typename T>
 cudaError_t launch_t(const void* x, int n_tok, int D, const void* A_k, const void* A_v, int Rk, int rv,
                      const int64_t* rows, void* kc, void* vc, int64_t n_rows, int* err, cudaStream_t s) {
-  if (n_tok <= kFewTokens)
+  if (few_tokens(n_tok, D, Rk + rv))
     append_few_kernel<T><<<dim3((Rk + rv) / kVCols, (n_tok + kVTok - 1) / kVTok), 256, 0, s>>>(
         (const T*)x, n_tok, D, (const T*)A_k, (const T*)A_v, Rk, rv, rows, (T*)kc, (T*)vc, n_rows, err);
   else

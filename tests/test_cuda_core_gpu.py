@@ -80,6 +80,50 @@ def test_append_few(dtype, n_tok, hidden):
         assert (got[np.setdiff1d(np.arange(n_tok + 5), rows)] == 0).all()
 
 
+def _wide(dtype, hidden, width):
+    return S.LayerSpec(hidden, 2, 2, 64, ((1,), (0,)), (width // 4, width // 4), width // 2, dtype, 1e4)
+
+
+@pytest.mark.parametrize("dtype,hidden", [("f32", 200), ("bf16", 196)])
+@pytest.mark.parametrize("width,side", [(2048, 0), (2048, 1), (512, 0), (512, 1)])
+def test_append_few_or_tiles(dtype, hidden, width, side):
+    """Either side of the line between the few-token and the tile kernel: n_tok (R_k + r_v) (D + 256) = 400000 D."""
+    n_tok = 400000 * hidden // ((hidden + 256) * width) + side
+    spec = _wide(dtype, hidden, width)
+    x, A_k, A_v = S.make_append_inputs(spec, n_tok, seed=width)
+    rows = np.random.default_rng(n_tok).choice(n_tok + 5, size=n_tok, replace=False)
+    buf = device.AppendBuffers(spec, n_tok, n_tok + 5).load_host(x, A_k, A_v, rows)
+    dck.check(buf.run(), "dck_latent_append")
+    torch.cuda.synchronize()
+    assert dck.dck_last_device_error() == dck.DCK_OK
+    u = 2.0 ** -8 if dtype == "bf16" else 2.0 ** -23
+    for got, ref, A in zip((buf.kcache, buf.vcache), oracle.latent_append(x, A_k, A_v), (A_k, A_v)):
+        got = got.float().cpu().numpy().astype(np.float64)
+        bound = u * np.abs(ref) + hidden * 2.0 ** -23 * (np.abs(x.astype(np.float64)) @ np.abs(A.astype(np.float64)))
+        assert (np.abs(got[rows] - ref) <= bound).all()
+
+
+@pytest.mark.parametrize("hidden,width", [(512, 4096), (64, 4096), (512, 1024)])
+def test_wide_append_takes_no_longer_than_one_token_more(hidden, width):
+    """512 tokens against 513 (the tile kernel): 5.5, 11 and 1.5 times as long while every call of up to 512 tokens
+    went to the few-token kernel."""
+    spec = _wide("f32", hidden, width)
+    us = {}
+    for n_tok in (512, 513):
+        x, A_k, A_v = S.make_append_inputs(spec, n_tok)
+        buf = device.AppendBuffers(spec, n_tok, n_tok).load_host(x, A_k, A_v, np.arange(n_tok))
+        times = []
+        for _ in range(15):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            dck.check(buf.run(), "dck_latent_append")
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1))
+        us[n_tok] = sorted(times)[7]
+    assert us[512] <= 1.3 * us[513], us
+
+
 def test_current_stream():
     """A call without a stream goes to the current one."""
     torch.cuda.init()
