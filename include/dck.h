@@ -168,7 +168,7 @@ dck_status dck_decode_attention(const dck_layer_desc* desc, const void* q,
  *   d_q_len      device int32 [B]: Q_b, 0 <= Q_b <= min(L_b, q_max); Q_b = 0
  *                writes nothing for sequence b
  *   q_max        the second dimension of q and out, 1 .. 2^24
- *   max_seq_len  an upper bound on every L_b, 1 .. 2^24 (sizes the launch)
+ *   max_seq_len  an upper bound on every L_b, 1 .. 2^24 (orders the work)
  *   kcache .. d_seq_len, rope_theta: as for dck_decode_attention
  *   out          [B, q_max, Hq, d]; rows i < Q_b of each sequence written (they
  *                hold the rotated queries until the results replace them); may
@@ -184,8 +184,7 @@ dck_status dck_decode_attention(const dck_layer_desc* desc, const void* q,
  * values.  A sequence with Q_b < 0, Q_b > L_b, Q_b > q_max, L_b > max_seq_len
  * or rows outside the cache is recorded as a device error (DCK_ERR_INVALID
  * from dck_last_device_error) and all q_max of its output rows are zero.
- * Two launches on `stream`: the reconstruction, then the attention; three
- * (values, keys, attention) where n_rows <= 2 B max_seq_len.
+ * Two launches on `stream`: the reconstruction, then the attention.
  */
 size_t dck_prefill_workspace_size(const dck_layer_desc* desc, int64_t n_rows);
 dck_status dck_prefill_attention(const dck_layer_desc* desc, const void* q, const int32_t* d_q_len,

@@ -64,6 +64,13 @@ constexpr int kMaxGroupsP = 16;
 // Then with deep loads for the queries, two epilogue warps per lane quadrant and
 // MMAs issued by a uniform warp, the launches alone (cold): MHA prompt 101 + 40 ->
 // 63 + 34 us, GQA prompt 81 + 21 -> 33 + 18 us.
+//
+// One launch for values and keys, whatever the size of the caller's cache: the row
+// tiles are those of the sequences.  A launch for each, the second starting early,
+// cost one set-up more and hid nothing: whole calls, us, two launches / one: one
+// token 34 / 31, MHA prompt of 1000 57 / 52, eight GQA prompts of 512 74 / 69, MHA
+// 2 x 4096 338 / 334, GQA 8192 451 / 442, 512 tokens after 32k 508 / 508 (GQA) and
+// 706 / 705 (MHA); only past 64k tokens are they level or 0.8% apart the other way.
 // ---------------------------------------------------------------------------
 
 constexpr int kREpiWarps = 8;    // two per TMEM lane quadrant
@@ -96,11 +103,11 @@ struct RArgs {
   const int32_t* q_len;
   int64_t n_rows;
   int B, Hq, Hkv, qmax, max_len;
-  int n_val, n_key;               // value and key column tiles of this launch (either may be 0)
+  int n_val, n_key;               // value and key column tiles of a row tile
   RCol col[kMaxColTiles];         // value tiles, then key tiles
   RopeFreqs rf;
   float qscale;                   // log2(e) / sqrt(d)
-  const __nv_bfloat16* q;         // null: this launch does not rotate the queries
+  const __nv_bfloat16* q;
   __nv_bfloat16* qr;              // rotated, scaled queries (the out buffer)
   __nv_bfloat16* kw;              // [n_rows][Hkv][d]
   __nv_bfloat16* vw;              // [n_rows][Hkv][d]
@@ -358,7 +365,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
       }
     }
     if (!ok && lane == 0) stop_peer();
-  } else if (ra.q) {
+  } else {
     // ---- queries: one warp per (sequence, new token); lane = (one of four heads
     // at a time, frequency pairs [8 c, 8 c + 8)).  Bound by the pass over q; the
     // loads of kQAhead rounds are issued before the first is used (with four
@@ -407,9 +414,6 @@ __global__ void __launch_bounds__(kRThreads, 1)
       }
     }
   }
-  // The keys' launch may start while the values' ends (it reads nothing of it); it
-  // is complete only after it, and so are both for the attention that follows.
-  griddep_wait();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
@@ -461,21 +465,19 @@ int recon_pairs_of_device() {
   return cache[dev];
 }
 
-cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, bool early, cudaStream_t s) {
+cudaError_t launch_recon(const RMaps& rm, const RArgs& ra, int pairs, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
   cfg.blockDim = dim3(kRThreads);
   cfg.dynamicSmemBytes = recon_smem(ra.B);
   cfg.stream = s;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = early ? 2 : 1;  // early: only after this call's own first launch
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, recon_kernel, rm, ra);
 }
 
@@ -1036,22 +1038,22 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   ra.Hkv = lt.Hkv;
   ra.qmax = qmax;
   ra.max_len = max_len;
-  RCol val[kMaxColTiles], key[kMaxColTiles];
-  int n_val = 0, n_key = 0;
   for (int h = 0; h < lt.Hkv; h += 2) {
     const int nh = std::min(2, lt.Hkv - h);
-    val[n_val++] = RCol{-1, (int16_t)(h * kPD), (int16_t)(nh * kPD), (int16_t)h, (int16_t)(h + 1), lt.rv};
+    ra.col[ra.n_val++] = RCol{-1, (int16_t)(h * kPD), (int16_t)(nh * kPD), (int16_t)h, (int16_t)(h + 1), lt.rv};
   }
   int head_at[kMaxGroupsP][kMaxKvHeads];
   for (int h = 0; h < lt.Hkv; ++h) head_at[lt.head_group[h]][lt.head_slot[h]] = h;
   for (int g = 0; g < lt.G; ++g)
     for (int sl = 0; sl < lt.grp_nh[g]; sl += 2) {
       const int nh = std::min(2, lt.grp_nh[g] - sl);
-      key[n_key++] = RCol{(int16_t)g, (int16_t)(sl * kPD), (int16_t)(nh * kPD), (int16_t)head_at[g][sl],
-                          (int16_t)(nh == 2 ? head_at[g][sl + 1] : 0), lt.grp_rank[g]};
+      ra.col[ra.n_val + ra.n_key++] = RCol{(int16_t)g, (int16_t)(sl * kPD), (int16_t)(nh * kPD),
+                                           (int16_t)head_at[g][sl],
+                                           (int16_t)(nh == 2 ? head_at[g][sl + 1] : 0), lt.grp_rank[g]};
     }
   ra.rf = rope_freqs_of(theta, kPD);
   ra.qscale = 1.4426950408889634f / std::sqrt((float)kPD);
+  ra.q = static_cast<const __nv_bfloat16*>(q);
   ra.kw = kw;
   ra.vw = vw;
   ra.qr = static_cast<__nv_bfloat16*>(out);
@@ -1063,19 +1065,8 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   if (pairs <= 0) return cudaErrorInvalidConfiguration;
   e = cudaFuncSetAttribute(prefill_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)asmem);
   if (e != cudaSuccess) return e;
-  // Where the caches hold little but these sequences' rows: the values (tensor
-  // bound, with the pass over q beside them), then the keys; in a pooled cache
-  // one launch for both.
-  const int n_launch = n_rows <= 2 * (int64_t)B * max_len ? 2 : 1;
-  for (int l = 0; l < n_launch; ++l) {
-    ra.n_val = l == 0 ? n_val : 0;
-    ra.n_key = l == n_launch - 1 ? n_key : 0;
-    ra.q = l == 0 ? static_cast<const __nv_bfloat16*>(q) : nullptr;
-    std::copy(val, val + ra.n_val, ra.col);
-    std::copy(key, key + ra.n_key, ra.col + ra.n_val);
-    if ((e = launch_recon(rm, ra, pairs, l > 0, s)) != cudaSuccess) return e;
-    if ((e = hook_launched(hook, s)) != cudaSuccess) return e;
-  }
+  if ((e = launch_recon(rm, ra, pairs, s)) != cudaSuccess) return e;
+  if ((e = hook_launched(hook, s)) != cudaSuccess) return e;
   AArgsP aa;
   std::memset(&aa, 0, sizeof(aa));
   aa.q_len = q_len;
@@ -1099,8 +1090,7 @@ cudaError_t launch_prefill_tc(const LayerTable& lt, const void* q, const int32_t
   cudaGetDevice(&dev);
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int64_t items = streams * aa.ntp;
-  // its set-up overlaps the reconstruction's end, as the keys' launch overlaps the
-  // values': eight short MHA prompts 58.3 -> 51.5 us, MHA prompt 2 x 4096 341 -> 336
+  // its set-up overlaps the reconstruction's end
   e = launch_pdl(prefill_attn_kernel, dim3((unsigned)std::min<int64_t>(items, sms)), dim3(kAThreadsP), asmem, s, am, aa);
   return e != cudaSuccess ? e : hook_launched(hook, s);
 }

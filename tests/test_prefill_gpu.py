@@ -3,8 +3,7 @@ fp64 oracle's prefill_attention: causal attention of each sequence's last Q_b
 cache rows over its prefix, keys and values rebuilt from the latents
 (Sec. III-A, III-C, III-D).
 
-Cases (the value reconstruction by the pair GEMM in all but the max_len case,
-where the reconstruction kernel rebuilds values too): Q = 1 (the decode call), Q = L (a whole prompt), ragged Q across the
+Cases: Q = 1 (the decode call), Q = L (a whole prompt), ragged Q across the
 batch, query and key tiles cut at and around the 128-row boundaries, MHA and
 both GQA layers, Q = 0 (nothing written), invalid sequences (recorded and
 zeroed), and a full 4096-token prompt sampled on two heads.  The tolerance is
@@ -44,9 +43,7 @@ def _run(spec, lens, q_lens, seed, q_max=None, q_std=1.0, max_len=None):
                                         buf.B_v, buf.seq_start, buf.seq_len, B, max_len, spec.rope_theta, out, ws,
                                         ws_bytes), "dck_prefill_attention")
     torch.cuda.synchronize()
-    # values rebuilt by the pair GEMM over all cache rows when the rows in use can be most of the
-    # cache (then three launches), else by the reconstruction kernel with the keys (two)
-    assert dck.dck_last_launch_count() == (3 if buf.n_rows <= 2 * B * max_len else 2)
+    assert dck.dck_last_launch_count() == 2  # the reconstruction, the attention
     return out.float().cpu().numpy().astype(np.float64), q, di
 
 

@@ -2,8 +2,8 @@
 counts and group sizes that leave a lone head in a tile, ranks at both ends of
 what the call takes (one 16-wide k-step, and past four 64-wide stages), value
 ranks that end inside a stage, sequences cut at the 256-row tiles, caches
-packed (values and keys in launches of their own) and pooled (one launch), a
-long context, and the output written over the queries.
+packed and pooled (the same launches for the same sequences), a long context,
+and the output written over the queries.
 
 The bound is the decode one, max|o - o_ref| / ||o_ref||_inf <= 2e-2: keys,
 values and probabilities are rounded to bf16 (2^-9 each) before products that
@@ -60,6 +60,7 @@ def test_prefill_tiles(name, shape, pool):
     dck.check(dck.dck_prefill_attention(buf.layer, qd, ql, q_max, buf.kcache, buf.vcache, buf.n_rows, buf.B_k,
                                         buf.B_v, buf.seq_start, sl, B, max(lens), spec.rope_theta, out, ws, n),
               "dck_prefill_attention")
+    assert dck.dck_last_launch_count() == 2  # by the sequences, not by the size of the caller's cache
     torch.cuda.synchronize()
     assert dck.dck_last_device_error() == dck.DCK_OK
     got = out.float().cpu().numpy().astype(np.float64)
