@@ -50,8 +50,8 @@ struct DecodeArgs {
   int64_t n_rows;
   int32_t B;
   int32_t n_items;
-  int32_t fine_below;  // tensor-core path: the pair-tile plan of tc_common.cuh (n_items = 2 x CTA pairs) with this
-                       // threshold of its fine split; 0: CUDA-core path
+  int32_t fine_below;  // tensor-core path: the pair-tile plan of tc_common.cuh (n_items = 2 x CTA pairs), its fine
+                       // split below this many tiles per pair (see main_tiles); 0: CUDA-core path
   float theta;
   float* part_u;   // [n_slots, Hq, rv]
   float* part_ml;  // [n_slots, Hq, 2]  (running max in log2 units, sum)
@@ -191,18 +191,28 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 
 // Tiles [0, main_tiles) are split in contiguous whole-tile ranges over the
-// n_items work items; with fewer than `fine_below` tiles per item, only n_items *
-// floor(NT / n_items) of them, the rest ("extra tiles") being shared out more
-// finely (see tc_common.cuh; 0 on the CUDA-core path).
+// n_items work items: all of them, or only n_items * floor(NT / n_items), the rest
+// ("extra tiles") being shared out more finely (see tc_common.cuh; fine_below 0, on
+// the CUDA-core path: never).  A whole tile more on some CTAs costs the call a tile's
+// time; an extra tile costs each of its CTAs a segment (a tile end, a partial), and
+// there are more of those the more tiles are left over.  So fewer than kFineAlways
+// tiles per item are always shared out, fewer than `fine_below` where no more than 3/8
+// of a tile per item are left over.  Calls of the 32-head MHA layer, us, shared out /
+// not, by tiles per CTA pair:
+//   8.1 224 / 236    8.5 240 / 236    8.9 257 / 242    8.1, 9.9 (32 ragged sequences) 246 / 258, 298 / 284
+//   16.1 401 / 410   16.5 415 / 413   16.9 433 / 417
+//   31.1 731 / 736   31.5 748 / 741   31.9 765 / 742   48.1 1100 / 1107
+// (from 32 tiles on a gain of 1% at most).  With several query heads per KV head a
+// segment also rotates its queries again: 8.1 140 / 142, 8.5 150 / 143, 12.1 183 / 185
+// and 16.1 228 / 229 on the 8-KV-head layer, so nothing is shared out from 8 tiles on.
+// (Below 8 the share matters as much, 4.1 93 / 96 and 4.9 115 / 99 there: not used.)
+constexpr int kFineAlways = 8;
 __host__ __device__ __forceinline__ int main_tiles(int NT, int n_items, int fine_below) {
-  return NT / n_items < fine_below ? NT / n_items * n_items : NT;
+  const int q = NT / n_items, whole = q * n_items;
+  const bool fine = q < fine_below && (q < kFineAlways || 8 * (NT - whole) <= 3 * n_items);
+  return fine ? whole : NT;
 }
-// An extra tile costs each of its CTAs a segment (a tile end, a partial); a whole
-// one more on some CTAs costs the call a tile's time.  32-head MHA layer, 32 ragged
-// sequences, 9.9 tiles per CTA pair: 300 us shared out, 311 not.  With several query
-// heads per KV head a segment also rotates its queries again: 8 x 32768 tokens,
-// 13.5 tiles per pair: 210 us shared out, 202 not.
-inline int fine_split_below(int qpg) { return qpg == 1 ? 32 : 8; }
+inline int fine_split_below(int qpg) { return qpg == 1 ? 32 : kFineAlways; }
 
 // The item whose tile range contains tile x (0 <= x < NT).
 __device__ __forceinline__ int item_of_tile(int x, int NT, int n_items) {

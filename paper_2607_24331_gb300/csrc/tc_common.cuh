@@ -61,9 +61,9 @@ __device__ __forceinline__ bool wait_slots(uint64_t* empty, int depth, int cnt, 
 // tokens, whose first 128 tokens belong to the pair's even CTA (half 0) and
 // the rest to its odd CTA (half 1).  The flattened pair-tile list (sequences in
 // order) is split over the pairs: pair p takes the contiguous range
-// [floor(p NPm / P), floor((p+1) NPm / P)) of the first NPm tiles; with fewer
-// than fine_split_below() tiles per pair the R = NP - NPm left over are shared
-// out by units (groups of heads) instead, pair p taking units
+// [floor(p NPm / P), floor((p+1) NPm / P)) of the first NPm = main_tiles() tiles;
+// the R = NP - NPm left over, where there are any, are shared out by units
+// (groups of heads) instead, pair p taking units
 // [floor(p R U / P), floor((p+1) R U / P)) of the flattened (extra tile, unit)
 // list.  The absorption kernel's CTA c = 2p + h follows half h of pair p's
 // tiles (its extra tiles it splits by r_v chunks instead).

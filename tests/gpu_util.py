@@ -43,15 +43,17 @@ def sm_count():
     return torch.cuda.get_device_properties(0).multi_processor_count
 
 
-def leftover_sequences(lens, sms):
+def leftover_sequences(lens, sms, spec):
     """Sequences with tiles in the finely split leftover range of the tensor-core
     path: sequences are cut into 256-token pair tiles, split over the CTA pairs
     (sms // 2 of them on a GPU whose TPCs all hold two SMs); with fewer than 8
-    pair tiles per pair, those from floor(NP / P) * P on are shared out by
-    groups of heads."""
+    pair tiles per pair, and with fewer than 32 on layers of one query head per
+    KV head where no more than 3/8 of a tile per pair are left over, those from
+    floor(NP / P) * P on are shared out by groups of heads."""
     nts = [(int(L) + 255) // 256 for L in lens]
     NP, P = sum(nts), sms // 2
-    NPm = NP // P * P if NP // P < 8 else NP
+    fine = NP // P < 8 or (spec.n_q_heads == spec.n_kv_heads and NP // P < 32 and 8 * (NP % P) <= 3 * P)
+    NPm = NP // P * P if fine else NP
     out, pre = [], 0
     for b, n in enumerate(nts):
         if n and pre + n > NPm:

@@ -47,7 +47,7 @@ def test_full_size_every_head_of_two_sequences(cfg):
     di = S.make_decode_inputs(spec, w.seq_lens, seed=w.seed)
     got, _ = gpu_decode(spec, w.seq_lens, di=di)
     assert np.isfinite(got).all()
-    left = leftover_sequences(w.seq_lens, sm_count())
+    left = leftover_sequences(w.seq_lens, sm_count(), spec)
     bs = sorted({0, left[-1] if left else w.batch - 1})
     for b in bs:
         ref = oracle_decode(di, batch_ids=[b])
@@ -63,7 +63,7 @@ def test_needles_at_a_tile_boundary_and_in_a_leftover_tile(cfg):
     lens = (64 * 128, (nt - 64 - 1) * 128 + 77)
     spec = S.workload(cfg).layer
     di = S.make_decode_inputs(spec, lens, seed=31 + cfg)
-    left = leftover_sequences(lens, sms)
+    left = leftover_sequences(lens, sms, spec)
     assert 1 in left
     k_left = nt - 64 - 2                          # second-last tile of sequence 1: a leftover tile
     # a pair-tile boundary (2560: the first token of pair tile 10, 2559: the last of

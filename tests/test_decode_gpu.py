@@ -161,6 +161,47 @@ def test_leftover_tiles_split_finely(cfg, extra):
     assert np.isfinite(got).all()
 
 
+@pytest.mark.parametrize("qpg,per_pair,left", [(1, 7, "most"), (1, 8, "3/8"), (1, 8, "more"), (1, 31, "3/8"),
+                                               (1, 31, "more"), (1, 32, "3/8"), (2, 7, "most"), (2, 8, "3/8")])
+def test_leftover_tiles_at_the_lines_of_their_split(qpg, per_pair, left):
+    """Either side of what decides whether leftover pair tiles are shared out: 8 tiles per CTA pair, and with one
+    query head per KV head up to 32 where no more than 3/8 of a tile per pair are left over."""
+    P = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    tiles = per_pair * P + {"most": P - 1, "3/8": 3 * P // 8, "more": 3 * P // 8 + 1}[left]
+    lens = ((tiles - 2) * 256 - 100, 256, 40)
+    spec = S.LayerSpec(256, 4 * qpg, 4, 128, ((2, 0), (1, 3)), (16, 48), 128, "bf16", 1e4)
+    buf = device.DecodeBuffers(spec, lens).synth(seed=per_pair, q_std=2.0)
+    dck.check(buf.run(), "decode")
+    torch.cuda.synchronize()
+    assert dck.dck_last_device_error() == dck.DCK_OK
+    got = buf.out.float().cpu().numpy().astype(np.float64)
+    di = S.DecodeInputs(spec, *(t.float().cpu().numpy() for t in (buf.q, buf.kcache, buf.vcache, buf.B_k, buf.B_v)),
+                        S.seq_starts(np.asarray(lens)), np.asarray(lens))
+    for b, j in ((0, 0), (0, 4 * qpg - 1), (1, 1), (2, 2)):
+        ref = oracle_decode(di, heads=[j], batch_ids=[b])
+        assert_parity(got[b:b + 1, j:j + 1], ref[b:b + 1, j:j + 1], "bf16", f"{per_pair} {left} b{b} j{j}")
+
+
+@pytest.mark.parametrize("per_pair", [8, 12])
+def test_fewer_tokens_take_no_longer(per_pair):
+    """One query head per KV head: 9 tiles on every CTA pair against 8.9 (13 against 12.9).  With those left over
+    shared out, the fewer tokens took 5 to 7% longer."""
+    spec, P = S.workload(5).layer, torch.cuda.get_device_properties(0).multi_processor_count // 2
+    us = []
+    for tiles in (per_pair * P + int(0.9 * P), (per_pair + 1) * P):
+        buf = device.DecodeBuffers(spec, (tiles // 2 * 256, (tiles - tiles // 2) * 256)).synth(seed=1)
+        times = []
+        for _ in range(25):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            dck.check(buf.run(), "decode")
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1))
+        us.append(sorted(times)[12])
+    assert us[0] <= 1.025 * us[1], us
+
+
 @pytest.mark.parametrize("batch", [1, 8, 32, 64])
 def test_32_layer_ragged_sampled(batch):
     """32-layer ragged workload: device-generated inputs (checked bit-exact against the host
