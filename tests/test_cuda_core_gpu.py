@@ -59,6 +59,16 @@ def test_step_fp32(lens):
     _step(S.workload(0).layer, lens, seed=6)
 
 
+@pytest.mark.parametrize("hidden,rv,n", [(200, 32, 5), (130, 32, 5), (256, 64, 300), (256, 32, 300), (36, 2048, 40)],
+                         ids=["cluster", "few", "pairs", "tiles", "core-tiles"])
+@pytest.mark.parametrize("qpg", [1, 2])
+def test_step_bf16_behind_each_append(hidden, rv, n, qpg):
+    """The decode kernel starts early behind the step's own append: bf16 layers of head dim 64 behind each kernel that
+    appends for them, the last tokens (all of a one-token sequence) being this step's own."""
+    lens = (1, 31, 33, 400, 1) if n == 5 else tuple(1 + (13 * i) % 40 for i in range(n))
+    _step(S.LayerSpec(hidden, 2 * qpg, 2, 64, ((1,), (0,)), (16, 48), rv, "bf16", 1e4), lens, seed=hidden + rv)
+
+
 @pytest.mark.parametrize("hidden", [1, 8, 127, 128, 130, 200, 512, 1100])
 @pytest.mark.parametrize("n_tok", [1, 8, 9, 129, 256, 512, 513])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
