@@ -38,13 +38,6 @@
 #include "tc_host.h"
 #include "tmap.h"
 
-#ifndef DCK_AB_TRACE
-#define DCK_AB_TRACE(code) ((void)0)
-#endif
-#ifndef DCK_AB_TRACE_FLUSH
-#define DCK_AB_TRACE_FLUSH() ((void)0)
-#endif
-
 namespace dck {
 namespace {
 
@@ -155,7 +148,6 @@ __global__ void __launch_bounds__(kAThreads, 1)
   volatile int* abort_flag = &sm.abort_flag;
   const int Hq = lt.Hq, hq_pad = aa.hq_pad, n_chunks = aa.n_chunks;
   const uint32_t pbytes = (uint32_t)hq_pad * 256;
-  DCK_AB_TRACE(99);
   griddep_launch();  // the combine kernel may stage its factors as CTAs finish
 
   if (warp == 0) {  // a barrier per lane
@@ -191,10 +183,8 @@ __global__ void __launch_bounds__(kAThreads, 1)
   pl.pr = blockIdx.x >> 1;
   pl.hh = blockIdx.x & 1;
   pl.nc = n_chunks;
-  DCK_AB_TRACE(3);
   const PairScan scan = pair_scan(a, sm.sc);
   const int NP = scan.total256;
-  DCK_AB_TRACE(4);
   const PSplit sp(NP, pl.P, a.fine_below);
   pl.NPm = sp.NPm;
   const bool fits = scan.total128 <= aa.max_tiles;  // else the scores kernel has reported the input
@@ -222,7 +212,6 @@ __global__ void __launch_bounds__(kAThreads, 1)
   const uint32_t ucols = (uint32_t)(n_chunks * hq_pad);
   const int nub = 2 * ucols <= kTmemCols ? 2 : 1;
   ASeg seg;
-  DCK_AB_TRACE(0);
 
   if (warp == 0) {
     // ---- producer ------------------------------------------------------------
@@ -309,14 +298,12 @@ __global__ void __launch_bounds__(kAThreads, 1)
             m_prev = m_now;
           }
           __syncwarp();
-          DCK_AB_TRACE(1);
           ++p_cnt;
           for (; done < nch && ok; ++done) {
             int c, r;
             chunk_at(done, c, r);
             if (!(ok = wait_slots(sm.v_empty + r * kNVr, kNVr, v_cnt[r], 1, lane, abort_flag))) break;
             issue_chunk(c, r);
-            DCK_AB_TRACE(2);
           }
         }
       }
@@ -448,7 +435,6 @@ __global__ void __launch_bounds__(kAThreads, 1)
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&sm.tile_ok);
-          DCK_AB_TRACE(20);
           ++rc;
         }
       }
@@ -456,7 +442,6 @@ __global__ void __launch_bounds__(kAThreads, 1)
       // segment end: U -> the segment's partial slot
       if (!(ok = wwait(&sm.u_ready[sgc % nub], (sgc / nub) & 1, abort_flag))) break;
       tc_fence_after();
-      DCK_AB_TRACE(22);
       float* dst = a.part_u + seg.slot * Hq * lt.rv + tau;
       const int ca = seg.ca, cb = seg.cb;
       for (int c = ca; c < cb; ++c) {
@@ -474,17 +459,13 @@ __global__ void __launch_bounds__(kAThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.u_free[sgc % nub]);
-      DCK_AB_TRACE(23);
       ++sgc;
     }
   }
   tc_fence_before();
   __syncthreads();
-  DCK_AB_TRACE_FLUSH();
   if (sm.abort_flag) {
-    const long long c0 = clock64();
-    while (clock64() - c0 < 4000000ll) {
-    }
+    drain_in_flight();
     if (tid == 0) atomicOr(a.err, kErrTimeout);
   }
   __syncthreads();

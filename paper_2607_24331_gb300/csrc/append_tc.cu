@@ -32,7 +32,7 @@ constexpr int kSplitMaxTok = 256;
 constexpr int kMaxSplit = 32;  // slices of a small batch that the workspace query has always allowed for
 
 struct AppendParams {
-  int n_tok, D, Rk, rv;
+  int n_tok, Rk, rv;
   int nt_k;      // N tiles over the key output
   int kblocks;   // ceil(D / 64)
   const int64_t* rows;  // cache row of each token
@@ -57,8 +57,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      const __grid_constant__ CUtensorMap tm_av, const AppendParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = align_1024(smem_raw);
-  constexpr int nst = kStages;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + nst * kStageBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
   uint64_t* empty = full + kStages;
   uint64_t* acc_bar = empty + kStages;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_bar + 1);
@@ -69,11 +68,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   int n0, nt;
   tile_of(p, blockIdx.x, is_k, n0, nt);
   const int m0 = blockIdx.y * kBM;
-  const int kb0 = 0, kb1 = p.kblocks;
   const int nboxes = (nt + 63) / 64;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < nst; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -98,9 +96,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tm_x);
     tma_prefetch_desc(tmb);
-    for (int kb = kb0; kb < kb1 - (kWithhold ? 1 : 0); ++kb) {
-      const int i = kb - kb0, s = i % nst;
-      if (i >= nst && !mbar_wait(&empty[s], ((i / nst) - 1) & 1, abort_flag)) break;
+    for (int kb = 0; kb < p.kblocks - (kWithhold ? 1 : 0); ++kb) {
+      const int s = kb % kStages;
+      if (kb >= kStages && !mbar_wait(&empty[s], ((kb / kStages) - 1) & 1, abort_flag)) break;
       uint8_t* a = smem + s * kStageBytes;
       uint8_t* b = a + kABytes;
       mbar_expect_tx(&full[s], kABytes + nboxes * (kBK * 64 * 2));
@@ -110,9 +108,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1 && lane == 0) {
     const uint32_t idesc = idesc_bf16(kBM, nt, false, true);
     bool ok = true;
-    for (int kb = kb0; kb < kb1; ++kb) {
-      const int i = kb - kb0, s = i % nst;
-      if (!(ok = mbar_wait(&full[s], (i / nst) & 1, abort_flag, kWithhold ? p.limit : kWaitCycles))) break;
+    for (int kb = 0; kb < p.kblocks; ++kb) {
+      const int s = kb % kStages;
+      if (!(ok = mbar_wait(&full[s], (kb / kStages) & 1, abort_flag, kWithhold ? p.limit : kWaitCycles))) break;
       tc_fence_after();
       const uint32_t a = smem_u32(smem + s * kStageBytes);
       const uint32_t b = a + kABytes;
@@ -120,7 +118,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int k = 0; k < kBK / 16; ++k) {
         const uint64_t ad = sdesc(a + k * 32, 16, 1024, kSw128);
         const uint64_t bd = sdesc(b + k * 2048, kBK * 64 * 2, 1024, kSw128);
-        umma_f16(tmem, ad, bd, idesc, (i > 0 || k > 0) ? 1u : 0u);
+        umma_f16(tmem, ad, bd, idesc, (kb > 0 || k > 0) ? 1u : 0u);
       }
       umma_commit(&empty[s]);
     }
@@ -574,10 +572,7 @@ __global__ void __launch_bounds__(kPThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
-    // let copies and MMAs already in flight land before the memory is released
-    const long long c0 = clock64();
-    while (clock64() - c0 < 4000000ll) {
-    }
+    drain_in_flight();
     if (threadIdx.x == 0) atomicOr(p.err, kErrTimeout);
   }
   cluster_sync();  // the peer no longer reads this CTA's operands or arrives on its barriers
@@ -633,7 +628,6 @@ cudaError_t launch_append_tc(const void* x, int n_tok, int D, const void* A_k, c
   const bool withhold = withhold_limit > 0;
   AppendParams p;
   p.n_tok = n_tok;
-  p.D = D;
   p.Rk = Rk;
   p.rv = rv;
   p.nt_k = (Rk + kMaxBN - 1) / kMaxBN;

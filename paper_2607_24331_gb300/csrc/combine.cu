@@ -34,10 +34,6 @@
 
 namespace cg = cooperative_groups;
 
-#ifndef DCK_CB_TRACE
-#define DCK_CB_TRACE(code) ((void)0)
-#endif
-
 namespace dck {
 namespace {
 
@@ -45,14 +41,6 @@ constexpr int kThreads = 256;
 constexpr int kMaxSplit = 8;    // CTAs per cluster (r_v split), portable cluster size
 constexpr int kMaxRows = 16;    // (sequence, query head) rows per cluster
 constexpr int kMergeBatch = 16; // partial loads of a row in flight together
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t f32_to_tf32(float x) {
   uint32_t r;
@@ -96,7 +84,6 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   const int nrow = nb * qpg;
   const int rr = rv >> lsplit;            // rows of u / B_v owned by this CTA (a multiple of 4)
   const int r0 = rank * rr;
-  DCK_CB_TRACE(99);
 
   // shared layout: B_v rows [rr][ldb] T | u rows [kMaxRows][rr + 4] | received partial o [split][kMaxRows * D / split]
   // | 1/l | per row: partial weights [kMaxRows][cap] f32, sums [kMaxRows][cap] f32, slots [kMaxRows][cap] i32,
@@ -173,12 +160,10 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
   }
   __syncthreads();
 
-  DCK_CB_TRACE(1);
   // Launched under programmatic dependent launch: everything above reads only the
   // call's inputs; the partials come from the kernels before, complete once the
   // preceding grid is.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  DCK_CB_TRACE(2);
 
   // (1) sixteen lanes per row, all rows at once: each live partial's slot, reference max m (log2
   // units) and sum l, their loads all in flight together (a lane per
@@ -241,7 +226,6 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
     }
   }
   __syncthreads();
-  DCK_CB_TRACE(3);
   const int rr4 = rr / 4;
   for (int idx = threadIdx.x; idx < nrow * rr4; idx += kThreads) {
     const int i = idx / rr4, r4 = idx % rr4;
@@ -274,10 +258,8 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
     reinterpret_cast<float4*>(su + (size_t)i * ldu)[r4] =
         make_float4(acc0.x + acc1.x, acc0.y + acc1.y, acc0.z + acc1.z, acc0.w + acc1.w);
   }
-  DCK_CB_TRACE(4);
-  cp_async_wait_all();
+  cp_async_wait<0>();
   __syncthreads();
-  DCK_CB_TRACE(5);
   const int share = kMaxRows * D >> lsplit;
   if constexpr (std::is_same<T, __nv_bfloat16>::value && D == 128) {
     // partial o over this CTA's rows of B_v on the tensor cores: o[16 x 128] =
@@ -356,9 +338,7 @@ __global__ void __launch_bounds__(kThreads, 2) combine_kernel(const LayerTable l
       }
   }
   }
-  DCK_CB_TRACE(6);
   cluster.sync();
-  DCK_CB_TRACE(7);
   T* out = static_cast<T*>(a.out);
   for (int pos = threadIdx.x; pos * split < nrow * D; pos += kThreads) {
     const int e = pos * split + rank;

@@ -167,6 +167,20 @@ __host__ __device__ __forceinline__ int item_begin(int c, int NT, int n_items) {
   return (int)(((int64_t)c * NT) / n_items);
 }
 
+// 16-byte global -> shared copies tracked per thread (cp.async groups).
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  cp_async16((uint32_t)__cvta_generic_to_shared(dst), src);
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the last N groups of this thread have landed
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Programmatic dependent launch: a kernel launched with launch_pdl may start
 // while the previous kernel on the stream finishes; pdl_wait() returns once
 // that kernel is complete and its memory visible (a no-op without PDL), and

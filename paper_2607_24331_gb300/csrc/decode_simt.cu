@@ -42,13 +42,6 @@ constexpr int kMaxRankK = 256;  // per-group rank handled by this kernel
 constexpr int kBlocksPerSm = 2;
 constexpr float kLog2e = 1.4426950408889634f;
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
 __device__ __forceinline__ float2 pair_of(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ float2 pair_of(const __nv_bfloat16* p) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
@@ -180,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, QP == 1 ? kBlocksPerSm : 1)
 
     for (int t0 = t_begin; t0 < t_end; t0 += kTok) {
       const int nt = min(kTok, t_end - t0);
-      cp_async_wait_all();
+      cp_async_wait<0>();
       __syncthreads();  // the tile (and the factor slice, the queries) are there; the other buffer is free
       const T* cb = sC + (size_t)buf * kTok * ldc_of<T>(rmax);
       buf ^= 1;

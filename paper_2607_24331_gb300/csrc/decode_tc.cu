@@ -147,23 +147,20 @@ struct Maps {
 
 // Per-group facts the hot loops need; copied to shared memory at kernel start
 // (indexing kernel-parameter tables at run time goes through the small constant
-// cache, which several warps would share).
-struct GroupSm {
+// cache, which several warps would share).  32 bytes each: at 24 the 32-head layer's
+// steps took 2% longer (16 x 4096 tokens 128.7 -> 130.9 us).
+struct alignas(32) GroupSm {
   int32_t roff;          // first key-cache column of the group
   int8_t np;             // latent pieces
-  int8_t h0, nh;         // MMA position of the group's first head, heads
+  int8_t nh;             // heads
   int8_t nu;             // units (pairs of heads, the last one single when nh is odd)
   int8_t w[kMaxPieces];  // piece widths (ranks)
-  int8_t pad;
   int16_t u0;            // the group's first unit in the tile's unit order
   int16_t k[kMaxPieces]; // first rank of each piece
-  int16_t i0;            // the group's first factor item in the tile's item order
-  int16_t rank;          // r_g
 };
 
 struct TcArgs {
   int hq_pad;
-  int n_items;                   // factor items per tile
   int n_pairs;                   // P
   int64_t fimg_seq_bytes;        // factor image bytes per sequence (query-folded mode)
   uint8_t* pglob;                // per-tile P images (workspace)
@@ -227,8 +224,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
                      const __grid_constant__ TcArgs ta) {
   constexpr int kMma = Ring<kFold>::kMma, NW = Ring<kFold>::NW, kNA = Ring<kFold>::NA;
   extern __shared__ uint8_t smem_raw[];
-  Smem<kFold>& sm =
-      *reinterpret_cast<Smem<kFold>*>(align_1024(smem_raw));
+  Smem<kFold>& sm = *reinterpret_cast<Smem<kFold>*>(align_1024(smem_raw));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   volatile int* abort_flag = &sm.abort_flag;
   const int hq_pad = ta.hq_pad;
@@ -718,10 +714,7 @@ __global__ void __launch_bounds__(kThreadsTc, 1)
   tc_fence_before();
   __syncthreads();
   if (sm.abort_flag) {
-    // let copies and MMAs already in flight land before the memory is released
-    const long long c0 = clock64();
-    while (clock64() - c0 < 4000000ll) {
-    }
+    drain_in_flight();
     if (tid == 0) atomicOr(a.err, kErrTimeout);
   }
   cluster_sync();  // the peer no longer reads this CTA's operands or arrives on its barriers
@@ -771,30 +764,11 @@ constexpr int kAppCols = 16;     // output columns of one GEMV block
 constexpr int kAppMaxTok = 64;   // tokens of a fused append
 constexpr int kAppWarps = 8;     // warps of a GEMV block, each a K range of D / 8
 
-// d += a b for one 16 x 8 x 16 tile, bf16 inputs, fp32 accumulators (row.col).
-__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                          uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // Four 8x8 b16 matrices from shared memory, transposed.
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
-}
-
-// 16-byte global -> shared copies tracked per thread (cp.async groups).
-__device__ __forceinline__ void cp_async16_cg(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // Four 8x8 b16 matrices from shared memory.
@@ -867,10 +841,10 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
     if (left <= 0) return;
     --left;
     const uint32_t st = rbase + (uint32_t)(slot * sb) + so;
-    cp_async16_cg(st, pa);
+    cp_async16(st, pa);
 #pragma unroll
     for (int m = 0; m < kAppMaxTok / 16; ++m)
-      if (m < mt && 16 * m + tr < B) cp_async16_cg(st + 512 + 512 * m, px + (int64_t)(16 * m) * D);
+      if (m < mt && 16 * m + tr < B) cp_async16(st + 512 + 512 * m, px + (int64_t)(16 * m) * D);
     pa += astep;
     px += 16;
   };
@@ -879,7 +853,7 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
   for (int q = 0; q < kPairs - 1; ++q) {
     issue(2 * q);
     issue(2 * q + 1);
-    cp_async_commit_group();
+    cp_async_commit();
   }
   int rd = 0, wr = kPairs - 1;  // slots read and refilled next
   const int m8 = lane >> 3, r8 = lane & 7;
@@ -887,9 +861,9 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
   for (int kk = 0; kk < nks; kk += 2) {
     issue(2 * wr);
     issue(2 * wr + 1);
-    cp_async_commit_group();
+    cp_async_commit();
     wr = wr + 1 == kPairs ? 0 : wr + 1;
-    cp_async_wait_group<kPairs - 1>();  // this slot has landed (this thread's copies)
+    cp_async_wait<kPairs - 1>();  // this slot has landed (this thread's copies)
     __syncwarp();
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -904,14 +878,14 @@ __device__ __forceinline__ void step_append_block(const LayerTable& lt, const De
         // A fragments (tokens 16 m .., k 0..15): matrix q = lane / 8 covers rows 8 (q & 1) .., k 8 (q >> 1) ..
         uint32_t af[4];
         ldmatrix_x4_plain(af, st + 512 + 512 * m);
-        mma_16816(acc[m][0], af[0], af[1], af[2], af[3], bf[0], bf[1]);
-        mma_16816(acc[m][1], af[0], af[1], af[2], af[3], bf[2], bf[3]);
+        mma_bf16_16816(acc[m][0], af, bf[0], bf[1]);
+        mma_bf16_16816(acc[m][1], af, bf[2], bf[3]);
       }
     }
     rd = rd + 1 == kPairs ? 0 : rd + 1;
     __syncwarp();  // every lane is done with the slot before it is refilled
   }
-  cp_async_wait_group<0>();
+  cp_async_wait<0>();
   __syncthreads();  // every warp is done with its ring
   // partial sums -> shared memory: token 16 m + gid (+8), column 8 n + 2 tig (+1)
 #pragma unroll
@@ -1211,16 +1185,14 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
     const int g = gorder[gi];
     GroupSm& gs = ta.grp[gi];
     gs.roff = lt.grp_roff[g];
-    gs.rank = (int16_t)lt.grp_rank[g];
     int16_t kk[kMaxPieces];
     gs.np = (int8_t)make_pieces(lt.grp_rank[g], gs.w, kk);
     if (gs.np > kMaxPieces || gs.np > std::min(Ring<true>::NA, Ring<false>::NA)) return false;
     for (int p = 0; p < gs.np; ++p) gs.k[p] = kk[p];
-    gs.h0 = (int8_t)pos;
+    const int h0 = pos;  // MMA position of the group's first head
     gs.nh = (int8_t)lt.grp_nh[g];
     gs.nu = (int8_t)((lt.grp_nh[g] + 1) / 2);
     gs.u0 = (int16_t)unit;
-    gs.i0 = (int16_t)item;
     for (int sl = 0; sl < lt.grp_nh[g]; ++sl)
       for (int h = 0; h < lt.Hkv; ++h)
         if (lt.head_group[h] == g && lt.head_slot[h] == sl) {
@@ -1232,7 +1204,7 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
       const int nh = std::min(2, lt.grp_nh[g] - s0);
       if (unit >= kMaxUnits) return false;
       ta.uitem[unit] = (int16_t)item;
-      ta.uinfo[unit++] = (uint32_t)(order[gs.h0 + s0] | (nh == 2 ? order[gs.h0 + s0 + 1] << 8 : 0) | nh << 16);
+      ta.uinfo[unit++] = (uint32_t)(order[h0 + s0] | (nh == 2 ? order[h0 + s0 + 1] << 8 : 0) | nh << 16);
       for (int p = 0; p < gs.np; ++p) {
         if (item >= kMaxItems) return false;
         const int w = gs.w[p], bytes = nh * w * 256;
@@ -1254,7 +1226,6 @@ bool build_tables(const LayerTable& lt, TcArgs& ta, PrepArgs& pa) {
   }
   ta.n_units = unit;
   ta.uitem[unit] = (int16_t)item;
-  ta.n_items = item;
   pa.n_units = off / kUnitBytes;
   pa.seq_bytes = off;
   ta.fimg_seq_bytes = off;

@@ -417,10 +417,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (*abort_flag) {
-    // let copies and MMAs already in flight land before the memory is released
-    const long long c0 = clock64();
-    while (clock64() - c0 < 4000000ll) {
-    }
+    drain_in_flight();
     if (tid == 0) atomicOr(ra.err, kErrTimeout);
   }
   cluster_sync();  // the peer no longer reads this CTA's operands or arrives on its barriers
@@ -964,9 +961,7 @@ __global__ void __launch_bounds__(kAThreadsP, 1)
   tc_fence_before();
   __syncthreads();
   if (sm.abort_flag) {
-    const long long c0 = clock64();
-    while (clock64() - c0 < 4000000ll) {
-    }
+    drain_in_flight();
     if (tid == 0) atomicOr(aa.err, kErrTimeout);
   }
   __syncthreads();
