@@ -28,8 +28,16 @@ constexpr int kABytes = kBM * kBK * 2;          // 16 KB
 constexpr int kBBytes = kBK * kMaxBN * 2;       // 32 KB
 constexpr int kStageBytes = kABytes + kBBytes;
 constexpr int kThreads = 192;
+// Up to this many tokens K is split over clusters (append_few_kernel): the line of the
+// split it replaced, at which its gain is largest, and not where the two kernels meet.
+// Clusters / pairs, us, 32-head layer, 8-KV-head layer, 8-KV-head long-context layer:
+// 256 tokens 16.8, 15.9, 8.9 / 23.6, 23.4, 23.4 (at 257); 300 22.4, 15.9, 14.4 / 24.0,
+// 23.5, 23.4; 512 32.7, 24.2, 17.0 / 24.0, 23.7, 23.7; 1024 62.8, 40.4, 32.9 / 24.2,
+// 24.3, 23.7 (the clusters' CTAs take two waves where they are level).
 constexpr int kSplitMaxTok = 256;
-constexpr int kMaxSplit = 32;  // slices of a small batch that the workspace query has always allowed for
+// fp32 slices of a small batch's output that the workspace query asks for: no kernel
+// uses them now, but a call without that space has always been refused.
+constexpr int kMaxSplit = 32;
 
 struct AppendParams {
   int n_tok, Rk, rv;

@@ -3,7 +3,8 @@ counts and group sizes that leave a lone head in a tile, ranks at both ends of
 what the call takes (one 16-wide k-step, and past four 64-wide stages), value
 ranks that end inside a stage, sequences cut at the 256-row tiles, caches
 packed and pooled (the same launches for the same sequences), a long context,
-and the output written over the queries.
+one sequence with nearly all of the batch's new tokens, and the output written
+over the queries.
 
 The bound is the decode one, max|o - o_ref| / ||o_ref||_inf <= 2e-2: keys,
 values and probabilities are rounded to bf16 (2^-9 each) before products that
@@ -37,11 +38,12 @@ SHAPES = [
     ((1, 255, 256, 257), (1, 255, 10, 257)),
     ((600, 0, 513), (599, 0, 1)),
     ((20000,), (3,)),
+    ((40, 1100, 300, 1, 700), (1, 1100, 2, 1, 0)),
 ]
 
 
 @pytest.mark.parametrize("pool", [1, 5])
-@pytest.mark.parametrize("shape", SHAPES, ids=["edges", "chunk", "long"])
+@pytest.mark.parametrize("shape", SHAPES, ids=["edges", "chunk", "long", "one-long"])
 @pytest.mark.parametrize("name", list(LAYERS))
 def test_prefill_tiles(name, shape, pool):
     spec = LAYERS[name]
